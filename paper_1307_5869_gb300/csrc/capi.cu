@@ -7,6 +7,7 @@
 #include <mutex>
 #include <new>
 
+#include "gm_tc_table.h"
 #include "prand_internal.h"
 
 namespace prand {
@@ -141,6 +142,16 @@ prand_status_t get_tables(int gen, DevTables **out)
         if (!dev_alloc(&T.lfsr, lfsr_b)) return PRAND_ERR_NOMEM;
         for (int g = 0; g < 8; ++g)
             if (!dev_alloc(&T.gm[g], gm_b)) return PRAND_ERR_NOMEM;
+        if (!host_alloc((uint32_t **)&T.wait_failed, 64, cudaHostAllocMapped)) return PRAND_ERR_NOMEM;
+        *T.wait_failed = 0;
+        for (int g = 0; g < 8; ++g) {
+            const GmParams &G = gm_params(PRAND_GM19 + g);
+            if (G.s != 32 && G.s != 8) continue;
+            static GmTcTable host;  // under g_tables_mu
+            if (!gm_tc_build(PRAND_GM19 + g, &host)) return PRAND_ERR_STATE;
+            if (!dev_alloc(&T.gm_tc[g], sizeof host)) return PRAND_ERR_NOMEM;
+            if (cudaMemcpy(T.gm_tc[g], &host, sizeof host, cudaMemcpyHostToDevice) != cudaSuccess) return PRAND_ERR_CUDA;
+        }
         prand_status_t s = mrg_build_table(T.mrg, 0);
         if (s == PRAND_OK) s = lfsr_build_table(T.lfsr, 0);
         for (int g = 0; g < 8 && s == PRAND_OK; ++g) s = gm_build_table(PRAND_GM19 + g, T.gm[g], 0);
@@ -224,7 +235,7 @@ bool mul_overflows(uint64_t a, uint64_t b, uint64_t *r)
     return __builtin_mul_overflow(a, b, r);
 }
 
-prand_status_t generate_any(prand_handle_t h, void *out, int dtype, uint64_t nper, prand_stream_t stream)
+prand_status_t generate_any(prand_handle_t h, void *out, int dtype, uint64_t nper, prand_stream_t stream, bool host = false)
 {
     if (!h || !out) return PRAND_ERR_ARG;
     size_t esz = dtype == PRAND_DTYPE_F64 ? 8 : 4;
@@ -238,6 +249,7 @@ prand_status_t generate_any(prand_handle_t h, void *out, int dtype, uint64_t npe
     cudaStream_t st = (cudaStream_t)stream;
     StreamRange R;
     R.stride = R.count = h->n;
+    R.host = host;
     if (h->gen == PRAND_MT19937) s = mt_gen(h->d_state, h->n, &h->mt_idx, out, dtype, nper, st);
     else if (is_gm(h->gen)) s = gm_gen(h->gen, h->T, h->d_state, h->d_spare, R, out, dtype, nper, st);
     else s = mrg_lfsr_gen(h->gen, h->T, h->d_state, h->d_spare, R, out, dtype, nper, st);
@@ -322,7 +334,7 @@ prand_status_t generate_host(prand_handle_t h, void *host_out, int dtype, uint64
     if (mul_overflows(h->n, nper, &total) || mul_overflows(total, esz, &bytes)) return PRAND_ERR_ARG;
     if (nper == 0) return PRAND_OK;
     if (void *mapped = mapped_host_address(host_out)) {
-        s = generate_any(h, mapped, dtype, nper, stream);
+        s = generate_any(h, mapped, dtype, nper, stream, true);
         if (s == PRAND_OK && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) s = PRAND_ERR_CUDA;
         return s;
     }

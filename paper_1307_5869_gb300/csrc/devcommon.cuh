@@ -180,6 +180,14 @@ struct Cvt<double, false> { __device__ __forceinline__ static double f(uint32_t 
 template <>
 struct Cvt<double, true> { __device__ __forceinline__ static double f(uint32_t u) { return mrg_to_f64(u); } };
 
+// Store two consecutive elements at p (aligned to both).
+template <typename OutT>
+__device__ __forceinline__ void store2(OutT *p, OutT a, OutT b)
+{
+    struct alignas(2 * sizeof(OutT)) Two { OutT a, b; };
+    *reinterpret_cast<Two *>(p) = Two{ a, b };
+}
+
 // Store four consecutive elements at p (16-byte aligned for 4-byte types,
 // 32-byte aligned for doubles when vec is true).
 template <typename OutT>

@@ -1,5 +1,5 @@
-// GM55 instantiation of the torus-map ensemble kernels (see gm_impl.cuh).
-#include "gm_impl.cuh"
+// GM55 instantiation of the torus-map ensemble kernels (see gm_host.cuh).
+#include "gm_host.cuh"
 
 namespace prand {
 PRAND_GM_INSTANTIATE(PRAND_GM55, gm55)

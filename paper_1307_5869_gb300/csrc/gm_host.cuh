@@ -1,0 +1,161 @@
+// Host side of the GM/GQ ensembles: launches of the kernels of gm_impl.cuh and
+// gm_tc.cuh, instantiated one translation unit per generator.
+#pragma once
+#include "gm_tc.cuh"
+
+namespace prand {
+
+template <int GEN>
+inline prand_status_t gm_build_table_t(uint64_t *tab, cudaStream_t st)
+{
+    gm_table_kernel<GEN><<<1, 32, 0, st>>>(tab);
+    return launch_check();
+}
+
+inline unsigned gm_grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1) / block); }
+
+template <int GEN>
+struct GmHost {
+    static prand_status_t seed(const uint64_t *tab, uint64_t *base, uint64_t seed, const Variant &V, cudaStream_t st)
+    {
+        gm_seed_kernel<GEN><<<1, 32, 0, st>>>(tab, base, seed, V.D[0], V.D[1]);
+        return launch_check();
+    }
+    static prand_status_t init(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first, uint64_t n,
+                               const Variant &V, cudaStream_t st)
+    {
+        const unsigned B = 128;
+        gm_init_kernel<GEN><<<gm_grid_for(n * GmT<GEN>::s, B), B, 0, st>>>(tab, base, state, first, n, V.L[0], V.L[1]);
+        return launch_check();
+    }
+    static prand_status_t skip(const uint64_t *tab, uint64_t *state, uint64_t n, const U256 &off, cudaStream_t st)
+    {
+        const unsigned B = 128;
+        gm_skip_kernel<GEN><<<gm_grid_for(n * GmT<GEN>::s, B), B, 0, st>>>(tab, state, n, off);
+        return launch_check();
+    }
+    // Sections per stream: whole waves of the kernel's resident sections (warps, threads
+    // or groups of lanes: cap), of at least min_len outputs, on multiples of `align`;
+    // a section's fixed work is worth `fixed` outputs.
+    static void pick(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t align, uint64_t min_len, uint64_t fixed,
+                     uint32_t *nsec, uint64_t *seclen)
+    {
+        const uint32_t s = pick_nsec(nstreams, cap, nper / min_len, nper, fixed);
+        uint64_t len = (nper + s - 1) / s;
+        len = (len + align - 1) / align * align;
+        if (len == 0) len = align;
+        *seclen = len;
+        *nsec = (uint32_t)((nper + len - 1) / len);
+        if (*nsec == 0) *nsec = 1;
+    }
+    // Whether a fill goes to the tensor-core kernel (cap: its resident sections) or to
+    // this file's other one.  With streams for more than one wave, by the work of a
+    // row: the tensor-core kernel makes whole blocks of 64 outputs and spends 0.9
+    // block's time per row besides, the other one 14 outputs' time, and an output
+    // takes kRatio / 100 times as long there (2^20 streams, u32, ns per output of a
+    // stream, other / this: GM31 11.6 / 7.1, GM61 20.3 / 8.2, GM55 7.1 / 2.7, GQ58.4
+    // 3.8 / 2.3, GM29 8.0 / 7.0).  With fewer the launch and the chain of steps count:
+    // 7 us whatever the row up to 200 outputs here, 16 (GM31) to 300 ns (GM55) a step
+    // there (64 streams x 100: GM31 6.6 / 7.0, GM61 7.6 / 7.0, GQ58.4 16.4 / 6.9 us).
+    // A fill of more than a wave into host memory is bound by the link, which takes the
+    // lane-per-point kernel's rows (9728 at once, out of step) 1 to 2 % faster than this
+    // one's 2432 (65536 x 1024 f32: GM61 1439 / 1459 us, GM31 1413 / 1442; stores of 4, 8
+    // or 16 bytes per lane alike).
+    static bool use_tc(uint64_t nstreams, uint64_t nper, uint64_t cap, bool host)
+    {
+        constexpr uint64_t ratio = GEN == PRAND_GM61 ? 249 : GEN == PRAND_GM55 ? 260 : GEN == PRAND_GQ58_4 ? 167
+                                 : GEN == PRAND_GM31 || GEN == PRAND_GQ58_1 ? 164 : 114;
+        constexpr uint64_t one_wave = GEN == PRAND_GM61 ? 80 : GmT<GEN>::v == 4 ? 24
+                                    : GEN == PRAND_GM31 || GEN == PRAND_GQ58_1 ? 128 : UINT64_MAX;
+        if (nstreams <= cap) return nper >= one_wave;
+        if (host && GmT<GEN>::v == 1) return false;
+        if (nper > 65536) return true;
+        return 100 * ((nper + kTcSteps - 1) / kTcSteps * kTcSteps + 56) < ratio * (nper + 14);
+    }
+    template <typename OutT>
+    static prand_status_t gen(const uint64_t *tab, const GmTcTable *tc, volatile uint32_t *failed, uint64_t *state,
+                              uint64_t *spare, StreamRange &R, OutT *out, uint64_t nper, cudaStream_t st)
+    {
+        using P = GmT<GEN>;
+        const unsigned B = 256;
+        const uint64_t off = R.j0 * P::s;
+        const uint64_t *sin = state + off;
+        if constexpr (GmTc<GEN>::kUse) {
+            const uint64_t ctas = (uint64_t)device_sm_count() * kTcCtas;
+            if (use_tc(R.count, nper, ctas * GmTc<GEN>::kStreams, R.host)) {
+                if (*failed) return PRAND_ERR_TIMEOUT;
+                if (R.nsec == 0) pick(R.count, nper, ctas * GmTc<GEN>::kStreams, kTcSteps, 256, 256, &R.nsec, &R.seclen);
+                const uint32_t nsec = R.nsec;
+                const uint64_t seclen = R.seclen, units = R.count * nsec;
+                if (units <= UINT32_MAX && seclen <= UINT32_MAX) {
+                    uint64_t *sout = (nsec > 1 ? spare : state) + off;
+                    // stores of two (v = 1) or four elements (sections start on multiples of 64)
+                    constexpr uint64_t V = GmT<GEN>::v == 1 ? 2 : 4;
+                    const bool vec = (uintptr_t)out % (sizeof(OutT) * V) == 0 && nper % V == 0;
+                    const uint64_t tiles = (units + GmTc<GEN>::kStreams - 1) / GmTc<GEN>::kStreams;
+                    const unsigned grid = (unsigned)(tiles < ctas ? tiles : ctas);
+                    const auto k = vec ? gm_tc_kernel<GEN, OutT, true> : gm_tc_kernel<GEN, OutT, false>;
+                    k<<<grid, kTcThreads, kTcSmem, st>>>(tc, tab, sin, sout, (uint32_t)R.count, R.stride, nper, (uint32_t)units,
+                                                         seclen, out, failed);
+                    return launch_check();
+                }
+            }
+        }
+        if constexpr (P::lanes == 32) {
+            if (R.nsec == 0) pick(R.count, nper, resident_threads<GEN>(gm_gen_kernel<GEN, OutT, true>) / 32, 128, 512, 128, &R.nsec, &R.seclen);
+            const uint32_t nsec = R.nsec;
+            const uint64_t seclen = R.seclen, nstreams = R.count;
+            uint64_t *sout = (nsec > 1 ? spare : state) + off;
+            // section starts are multiples of 128, so rows start 16-byte aligned
+            // when the output is aligned and n_per_stream is a multiple of 4
+            const bool vec = ((uintptr_t)out % (sizeof(OutT) == 8 ? 32 : 16)) == 0 && nper % 4 == 0;
+            const unsigned grid = gm_grid_for(nstreams * nsec * 32, B);
+            if (vec) gm_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+            else gm_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+        } else {
+            if (R.nsec == 0) pick(R.count, nper, resident_threads<200 + GEN>(gmt_gen_kernel<GEN, OutT, true>), 32, 256, 128, &R.nsec, &R.seclen);
+            const uint32_t nsec = R.nsec;
+            const uint64_t seclen = R.seclen, nstreams = R.count;
+            uint64_t *sout = (nsec > 1 ? spare : state) + off;
+            constexpr uint64_t E = RowFill<OutT>::E;
+            const bool rows = ((uintptr_t)out % 16) == 0 && nper % E == 0 && seclen % E == 0;
+            const unsigned grid = gm_grid_for(nstreams * nsec, B);
+            if (rows) gmt_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+            else gmt_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+        }
+        return launch_check();
+    }
+};
+
+
+// Per-generator entry points, instantiated one translation unit per generator.
+#define PRAND_GM_INSTANTIATE(GEN, NAME)                                                                          \
+    prand_status_t NAME##_table(uint64_t *tab, cudaStream_t st) { return gm_build_table_t<GEN>(tab, st); }      \
+    prand_status_t NAME##_seed(const uint64_t *tab, uint64_t *base, uint64_t seed, const Variant &V,           \
+                               cudaStream_t st)                                                               \
+    {                                                                                                         \
+        return GmHost<GEN>::seed(tab, base, seed, V, st);                                                     \
+    }                                                                                                         \
+    prand_status_t NAME##_init(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first,     \
+                               uint64_t n, const Variant &V, cudaStream_t st)                                 \
+    {                                                                                                         \
+        return GmHost<GEN>::init(tab, base, state, first, n, V, st);                                          \
+    }                                                                                                         \
+    prand_status_t NAME##_skip(const uint64_t *tab, uint64_t *state, uint64_t n, const U256 &off,             \
+                               cudaStream_t st)                                                               \
+    {                                                                                                         \
+        return GmHost<GEN>::skip(tab, state, n, off, st);                                                     \
+    }                                                                                                         \
+    prand_status_t NAME##_gen(const DevTables *T, uint64_t *state, uint64_t *spare, StreamRange &R,            \
+                              void *out, int dtype, uint64_t nper, cudaStream_t st)                            \
+    {                                                                                                         \
+        const uint64_t *tab = T->gm[GEN - PRAND_GM19];                                                        \
+        const GmTcTable *tc = T->gm_tc[GEN - PRAND_GM19];                                                     \
+        if (dtype == PRAND_DTYPE_U32)                                                                         \
+            return GmHost<GEN>::template gen<uint32_t>(tab, tc, T->wait_failed, state, spare, R, (uint32_t *)out, nper, st); \
+        if (dtype == PRAND_DTYPE_F32)                                                                         \
+            return GmHost<GEN>::template gen<float>(tab, tc, T->wait_failed, state, spare, R, (float *)out, nper, st);  \
+        return GmHost<GEN>::template gen<double>(tab, tc, T->wait_failed, state, spare, R, (double *)out, nper, st);    \
+    }
+
+}  // namespace prand

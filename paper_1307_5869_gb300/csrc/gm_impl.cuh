@@ -14,6 +14,8 @@
 //    word by one logic operation, so no lane waits on another.  Rows leave
 //    through the staged 128-byte row stores of the thread-per-stream
 //    generators.
+// Long rows of all but GQ58.3 go through the tensor cores instead (gm_tc.cuh; the
+// rule is in gm_host.cuh).
 //
 // Arithmetic is exact on z = x / 2^t modulo the prime p (g = 2^t p; for GM55
 // and GQ58.x, k and q are even, so states kept on multiples of 2^t stay there
@@ -632,112 +634,5 @@ __global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict
     }
     if (len && start + len == nper) gmt_store<GEN>(zc, zp, state_out + j * P::s, state_out + (stride + j) * P::s);
 }
-
-// ----------------------------------------------------------------- host side
-template <int GEN>
-inline prand_status_t gm_build_table_t(uint64_t *tab, cudaStream_t st)
-{
-    gm_table_kernel<GEN><<<1, 32, 0, st>>>(tab);
-    return launch_check();
-}
-
-inline unsigned gm_grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1) / block); }
-
-template <int GEN>
-struct GmHost {
-    static prand_status_t seed(const uint64_t *tab, uint64_t *base, uint64_t seed, const Variant &V, cudaStream_t st)
-    {
-        gm_seed_kernel<GEN><<<1, 32, 0, st>>>(tab, base, seed, V.D[0], V.D[1]);
-        return launch_check();
-    }
-    static prand_status_t init(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first, uint64_t n,
-                               const Variant &V, cudaStream_t st)
-    {
-        const unsigned B = 128;
-        gm_init_kernel<GEN><<<gm_grid_for(n * GmT<GEN>::s, B), B, 0, st>>>(tab, base, state, first, n, V.L[0], V.L[1]);
-        return launch_check();
-    }
-    static prand_status_t skip(const uint64_t *tab, uint64_t *state, uint64_t n, const U256 &off, cudaStream_t st)
-    {
-        const unsigned B = 128;
-        gm_skip_kernel<GEN><<<gm_grid_for(n * GmT<GEN>::s, B), B, 0, st>>>(tab, state, n, off);
-        return launch_check();
-    }
-    // Sections per stream: whole waves of the kernel's resident warps (lane
-    // per point) or threads (thread per stream), cap; sections start on
-    // multiples of 128 outputs (a warp's round) or 32 outputs (a 128-byte row).
-    static void pick(uint64_t nstreams, uint64_t nper, uint64_t cap, uint32_t *nsec, uint64_t *seclen)
-    {
-        constexpr uint64_t A = GmT<GEN>::lanes == 32 ? 128 : 32;
-        const uint32_t s = pick_nsec(nstreams, cap, GmT<GEN>::lanes == 32 ? nper / 512 : nper / 256, nper);
-        uint64_t len = (nper + s - 1) / s;
-        len = (len + A - 1) / A * A;
-        if (len == 0) len = A;
-        *seclen = len;
-        *nsec = (uint32_t)((nper + len - 1) / len);
-        if (*nsec == 0) *nsec = 1;
-    }
-    template <typename OutT>
-    static prand_status_t gen(const uint64_t *tab, uint64_t *state, uint64_t *spare, StreamRange &R, OutT *out,
-                              uint64_t nper, cudaStream_t st)
-    {
-        using P = GmT<GEN>;
-        const unsigned B = 256;
-        const uint64_t off = R.j0 * P::s;
-        const uint64_t *sin = state + off;
-        if constexpr (P::lanes == 32) {
-            if (R.nsec == 0) pick(R.count, nper, resident_threads<GEN>(gm_gen_kernel<GEN, OutT, true>) / 32, &R.nsec, &R.seclen);
-            const uint32_t nsec = R.nsec;
-            const uint64_t seclen = R.seclen, nstreams = R.count;
-            uint64_t *sout = (nsec > 1 ? spare : state) + off;
-            // section starts are multiples of 128, so rows start 16-byte aligned
-            // when the output is aligned and n_per_stream is a multiple of 4
-            const bool vec = ((uintptr_t)out % (sizeof(OutT) == 8 ? 32 : 16)) == 0 && nper % 4 == 0;
-            const unsigned grid = gm_grid_for(nstreams * nsec * 32, B);
-            if (vec) gm_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-            else gm_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-        } else {
-            if (R.nsec == 0) pick(R.count, nper, resident_threads<200 + GEN>(gmt_gen_kernel<GEN, OutT, true>), &R.nsec, &R.seclen);
-            const uint32_t nsec = R.nsec;
-            const uint64_t seclen = R.seclen, nstreams = R.count;
-            uint64_t *sout = (nsec > 1 ? spare : state) + off;
-            constexpr uint64_t E = RowFill<OutT>::E;
-            const bool rows = ((uintptr_t)out % 16) == 0 && nper % E == 0 && seclen % E == 0;
-            const unsigned grid = gm_grid_for(nstreams * nsec, B);
-            if (rows) gmt_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-            else gmt_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-        }
-        return launch_check();
-    }
-};
-
-
-// Per-generator entry points, instantiated one translation unit per generator.
-#define PRAND_GM_INSTANTIATE(GEN, NAME)                                                                          \
-    prand_status_t NAME##_table(uint64_t *tab, cudaStream_t st) { return gm_build_table_t<GEN>(tab, st); }      \
-    prand_status_t NAME##_seed(const uint64_t *tab, uint64_t *base, uint64_t seed, const Variant &V,           \
-                               cudaStream_t st)                                                               \
-    {                                                                                                         \
-        return GmHost<GEN>::seed(tab, base, seed, V, st);                                                     \
-    }                                                                                                         \
-    prand_status_t NAME##_init(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first,     \
-                               uint64_t n, const Variant &V, cudaStream_t st)                                 \
-    {                                                                                                         \
-        return GmHost<GEN>::init(tab, base, state, first, n, V, st);                                          \
-    }                                                                                                         \
-    prand_status_t NAME##_skip(const uint64_t *tab, uint64_t *state, uint64_t n, const U256 &off,             \
-                               cudaStream_t st)                                                               \
-    {                                                                                                         \
-        return GmHost<GEN>::skip(tab, state, n, off, st);                                                     \
-    }                                                                                                         \
-    prand_status_t NAME##_gen(const uint64_t *tab, uint64_t *state, uint64_t *spare, StreamRange &R,          \
-                              void *out, int dtype, uint64_t nper, cudaStream_t st)                            \
-    {                                                                                                         \
-        if (dtype == PRAND_DTYPE_U32)                                                                         \
-            return GmHost<GEN>::template gen<uint32_t>(tab, state, spare, R, (uint32_t *)out, nper, st); \
-        if (dtype == PRAND_DTYPE_F32)                                                                         \
-            return GmHost<GEN>::template gen<float>(tab, state, spare, R, (float *)out, nper, st);  \
-        return GmHost<GEN>::template gen<double>(tab, state, spare, R, (double *)out, nper, st);    \
-    }
 
 }  // namespace prand

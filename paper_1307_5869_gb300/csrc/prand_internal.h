@@ -117,6 +117,8 @@ struct DevTables {
     uint32_t *mrg = nullptr;      // [kJumpBits][18]: A^(2^b) mod m1 (9 words), B^(2^b) mod m2 (9 words)
     uint32_t *lfsr = nullptr;     // [4][kJumpBits][32]: column images of T_c^(2^b)
     uint64_t *gm[8] = {};         // per GM/GQ generator: [kJumpBits][4] = M^(2^b) mod p
+    struct GmTcTable *gm_tc[8] = {};      // the tensor-core generation's constants (null: not used by the generator)
+    volatile uint32_t *wait_failed = nullptr;  // mapped host memory: set by a kernel whose bounded wait ran out
     uint32_t *mt = nullptr;       // [kMtPolyCount][kMtPolyWords]: x^(2^b) mod phi
     uint32_t *mt_win = nullptr;   // [kMtWinPositions][kMtWinDigits][kMtPolyWords]: x^(d 2^(432 + 8 i)) mod phi
     bool ready_basic = false;
@@ -157,25 +159,27 @@ struct U256 { uint64_t w[4]; };
 // (nsec and seclen are written back); otherwise the given pair is used, so the
 // fills of several ranges in one call split their streams alike and keep their
 // next states in the same buffer (in place when nsec == 1, the spare otherwise).
+// host: the outputs go over the host link (page-locked host memory).
 struct StreamRange {
     uint64_t stride = 0, j0 = 0, count = 0;
     uint32_t nsec = 0;
     uint64_t seclen = 0;
+    bool host = false;
 };
 
 // Sections per stream for a launch of `units` work items (threads or lane
 // groups, one per stream) with nper outputs each, when `cap` items are
 // resident at once: the count in [1, max_s] whose grid best fills whole waves,
 // discounted for the fixed work each section starts with (its jump, state
-// load and store: about 128 outputs' worth).  Candidates: 1..64, multiples of one wave's worth, max_s.
-inline uint32_t pick_nsec(uint64_t units, uint64_t cap, uint64_t max_s, uint64_t nper)
+// load and store: `fixed` outputs' worth).  Candidates: 1..64, multiples of one wave's worth, max_s.
+inline uint32_t pick_nsec(uint64_t units, uint64_t cap, uint64_t max_s, uint64_t nper, uint64_t fixed = 128)
 {
     if (cap == 0 || units == 0 || nper == 0) return 1;
     if (max_s < 1) max_s = 1;
     if (max_s > 65535) max_s = 65535;
     auto score = [&](uint64_t s) {
         const uint64_t n = units * s, waves = (n + cap - 1) / cap;
-        return ((double)n / (double)(waves * cap)) / (1.0 + 128.0 * (double)s / (double)nper);
+        return ((double)n / (double)(waves * cap)) / (1.0 + (double)fixed * (double)s / (double)nper);
     };
     uint64_t best = 1;
     double best_score = score(1);
