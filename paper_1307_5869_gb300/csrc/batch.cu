@@ -5,8 +5,9 @@
 //
 // Work unit: a tile, run by one warp.  MRG32K3A / LFSR113 tiles are up to 32
 // sections of one request (one lane each, rows written through the staged
-// 128-byte row stores); GM/GQ tiles are up to 32 / lanes sections (one lane
-// group each); MT19937 tiles are one whole request (the jump is a chain of
+// 128-byte row stores); GQ58.3 tiles likewise; the other GM/GQ requests go to the
+// tensor-core kernels in tiles of 4 or 16 sections (in the server, whose tiles start
+// from state slots, to tiles of up to 32 / lanes sections); MT19937 tiles are one whole request (the jump is a chain of
 // polynomial applications by the warp, Sec. 5.4).  Warps claim tiles from an
 // atomic counter, so short and long tiles balance across the GPU; tiles are
 // ordered longest first.
@@ -219,13 +220,41 @@ uint64_t plan_tile_count(const prand_request_t &r, const BatchParams &P, uint32_
     return (r.length + per_tile - 1) / per_tile;
 }
 
+// Tensor-core tiles: the 4 (v = 1) or 16 (v = 4) sections of a tile are made in step by
+// one block, each from its own jump, so a tile's sections are of one length, whole
+// blocks of 64 outputs, at most kTcSection: long enough that a jump is a small part of
+// a section, short enough that the longest requests still spread over tens of blocks
+// (10^4 mixed requests, the part's five larger generators alone: 6.1 ms at 512, 4.0 at
+// 1024, 3.0 at 2048, 2.5 at 4096, 2.3 at 8192; 100 requests without MT19937: 0.58,
+// 0.57, 0.57, 0.57, 0.62 ms).
+constexpr uint64_t kTcSection = 4096;
+
+bool tc_tile_gen(int gen) { return is_gm(gen) && gen != PRAND_GQ58_3; }
+
+static void plan_tc(const prand_request_t &r, std::vector<BatchTile> &out)
+{
+    const GmParams &G = gm_params(r.gen);
+    const uint64_t n = G.s == 32 ? 4 : 16, es = esize(r.dtype);
+    const uint64_t tiles = (r.length + n * kTcSection - 1) / (n * kTcSection);
+    const uint64_t sec = ((r.length + n * tiles - 1) / (n * tiles) + 63) & ~63ull, per_tile = sec * n;
+    for (uint64_t off = 0; off < r.length; off += per_tile) {
+        BatchTile t = {};
+        t.stream = r.stream; t.start = off; t.len = std::min(per_tile, r.length - off);
+        t.out = (uintptr_t)r.dev_out + off * es;
+        t.seclen = (uint32_t)sec; t.gen = (uint8_t)r.gen; t.dtype = (uint8_t)r.dtype; t.slot = t.wslot = -1;
+        t.flags = (uint16_t)(kTileTc | ((uintptr_t)r.dev_out % (es * (G.v == 1 ? 2 : 4)) == 0 ? kTileVec : 0u));
+        out.push_back(t);
+    }
+}
+
 void plan_request(const prand_request_t &r, int32_t slot, int32_t wslot, bool from_slot, const BatchParams &P,
-                  std::vector<BatchTile> &out, uint32_t max_tiles)
+                  std::vector<BatchTile> &out, uint32_t max_tiles, bool tc)
 {
     if (r.length == 0) return;
     const int gen = r.gen;
     const size_t es = esize(r.dtype);
     const uintptr_t base = (uintptr_t)r.dev_out;
+    if (tc && tc_tile_gen(gen)) return plan_tc(r, out);
     auto vec_ok = [&](uint64_t seclen) { return base % 16 == 0 && (seclen * es) % 16 == 0 && seclen % 4 == 0; };
     const uint16_t fs = from_slot ? (uint16_t)kTileFromSlot : (uint16_t)0;
     if (gen == PRAND_MT19937) {
@@ -258,13 +287,14 @@ size_t slot_words(int gen)
 
 bool wide_tile_gen(int gen) { return is_gm(gen) && gm_params(gen).lanes == 1; }
 
-// MT19937 tiles first, then the thread-per-stream GM/GQ tiles, then the rest;
-// longest first within each part (MT19937 jump chains are the longest).
+// The parts of BatchParts in order; longest first within each part (MT19937 jump
+// chains are the longest).
 static uint64_t tile_cost(const BatchTile &t)
 {
-    if (t.gen == PRAND_MT19937) return (1ull << 41) + t.len;
-    if (wide_tile_gen(t.gen)) return (1ull << 40) + t.len;
-    return t.len / (t.gen == PRAND_MRG32K3A || t.gen == PRAND_LFSR113 ? 32 : 1);
+    if (t.gen == PRAND_MT19937) return (3ull << 60) + t.len;
+    if (t.flags & kTileTc) return ((uint64_t)(PRAND_NUM_GENERATORS - t.gen) << 44) + std::min<uint64_t>(t.len, 1ull << 40);
+    if (wide_tile_gen(t.gen)) return (2ull << 60) + t.len;
+    return (1ull << 60) + t.len / (t.gen == PRAND_MRG32K3A || t.gen == PRAND_LFSR113 ? 32 : 1);
 }
 
 void order_tiles(std::vector<BatchTile> &tiles)
@@ -298,27 +328,21 @@ static unsigned batch_grid(uint32_t ntiles, uint32_t block, int blocks_per_sm)
     return (unsigned)std::max<uint64_t>(g, 1);
 }
 
-uint32_t count_mt_tiles(const std::vector<BatchTile> &tiles)
+BatchParts batch_parts(const std::vector<BatchTile> &tiles)
 {
-    uint32_t n = 0;
-    while (n < tiles.size() && tiles[n].gen == PRAND_MT19937) ++n;
-    return n;
+    BatchParts p;
+    for (const BatchTile &t : tiles) {
+        if (t.gen == PRAND_MT19937) ++p.mt;
+        else if (t.flags & kTileTc) ++p.tc[t.gen - PRAND_GM19];
+        else if (wide_tile_gen(t.gen)) ++p.wide;
+        else ++p.rest;
+    }
+    return p;
 }
 
-uint32_t count_wide_tiles(const std::vector<BatchTile> &tiles, uint32_t nmt)
-{
-    uint32_t n = 0;
-    while (nmt + n < tiles.size() && wide_tile_gen(tiles[nmt + n].gen)) ++n;
-    return n;
-}
-
-// Tiles [0, nmt): MT19937 (counter[0]); [nmt, nmt + nwide): thread-per-stream
-// GM/GQ (counter[2]); the rest (counter[1]).  With MT19937 tiles beside others
-// with side branches the MT19937 part runs on br->st[0] and the
-// thread-per-stream part on br->st[1], each forked from and joined back into `st`.
 prand_status_t Branches::create()
 {
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < kBranches; ++b)
         if (cudaStreamCreateWithFlags(&st[b], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&fork[b], cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&join[b], cudaEventDisableTiming) != cudaSuccess)
@@ -328,7 +352,7 @@ prand_status_t Branches::create()
 
 void Branches::destroy()
 {
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < kBranches; ++b) {
         if (st[b]) cudaStreamDestroy(st[b]);
         if (fork[b]) cudaEventDestroy(fork[b]);
         if (join[b]) cudaEventDestroy(join[b]);
@@ -337,16 +361,17 @@ void Branches::destroy()
     }
 }
 
-prand_status_t launch_batch(const BatchTile *d_tiles, uint32_t ntiles, uint32_t nmt, uint32_t nwide,
-                            uint32_t *d_counter, const BatchCtx &ctx, cudaStream_t st, const Branches *br)
+// d_counter: [0] MT19937, [1] the rest, [2] thread-per-stream tiles.
+prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter, const BatchCtx &ctx,
+                            cudaStream_t st, const Branches *br)
 {
     if (cudaMemsetAsync(d_counter, 0, 3 * sizeof(uint32_t), st) != cudaSuccess) return PRAND_ERR_CUDA;
-    if (!ntiles) return PRAND_OK;
-    const uint32_t nrest = ntiles - nmt - nwide;
-    // a part goes to its branch when another part runs beside it
-    const bool on_branch[2] = { br && nmt && (nwide || nrest), br && nwide && nrest };
+    if (!parts.all()) return PRAND_OK;
+    const uint32_t nmt = parts.mt, nwide = parts.wide, nrest = parts.rest, ntc = parts.tc_all();
+    // a part goes to its branch when a later part runs beside it
+    const bool on_branch[kBranches] = { br && nmt && (nwide || nrest || ntc), br && nwide && (nrest || ntc), br && ntc && nrest };
     prand_status_t s = PRAND_OK;
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < kBranches; ++b)
         if (on_branch[b] && (cudaEventRecord(br->fork[b], st) != cudaSuccess ||
                              cudaStreamWaitEvent(br->st[b], br->fork[b], 0) != cudaSuccess))
             return PRAND_ERR_CUDA;
@@ -364,13 +389,20 @@ prand_status_t launch_batch(const BatchTile *d_tiles, uint32_t ntiles, uint32_t 
             d_tiles + nmt, nwide, d_counter + 2, ctx);
         if ((s = launch_check()) != PRAND_OK) return s;
     }
+    const BatchTile *tc_tiles = d_tiles + nmt + nwide + nrest;
+    for (int g = 0; g < 8; ++g) {
+        if (!parts.tc[g]) continue;
+        s = gm_batch(PRAND_GM19 + g, E->T, tc_tiles, parts.tc[g], ctx.base[PRAND_GM19 + g], on_branch[2] ? br->st[2] : st);
+        if (s != PRAND_OK) return s;
+        tc_tiles += parts.tc[g];
+    }
     if (nrest) {
         const int v = rest_variant(E->params.block, E->params.row_bytes);
         rest_launch(v, batch_grid(nrest, rest_block(v), E->rest_bps[v]), st, d_tiles + nmt + nwide, nrest,
                     d_counter + 1, ctx);
         if ((s = launch_check()) != PRAND_OK) return s;
     }
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < kBranches; ++b)
         if (on_branch[b] && (cudaEventRecord(br->join[b], br->st[b]) != cudaSuccess ||
                              cudaStreamWaitEvent(st, br->join[b], 0) != cudaSuccess))
             return PRAND_ERR_CUDA;
@@ -414,7 +446,7 @@ using namespace prand;
 struct prand_batch_plan_s {
     int device = -1;
     BatchTile *d_tiles = nullptr;
-    uint32_t ntiles = 0, nmt = 0, nwide = 0;
+    BatchParts parts;
     Branches br;  // the side branches while capturing
     uint32_t *d_counter = nullptr;
     BatchCtx ctx;
@@ -434,7 +466,7 @@ prand_status_t prand_batch_run(const prand_request_t *reqs, size_t n, uint64_t s
     const BatchParams P = batch_params();
     std::vector<BatchTile> tiles;
     tiles.reserve(n * 2);
-    for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles);
+    for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles, 0, true);
     order_tiles(tiles);
     if (tiles.size() > 0xFFFFFFFFull) return PRAND_ERR_ARG;
     BatchTile *d_tiles;
@@ -443,8 +475,7 @@ prand_status_t prand_batch_run(const prand_request_t *reqs, size_t n, uint64_t s
     Engine *E;
     if ((s = engine_get(&E)) != PRAND_OK) return s;
     std::lock_guard<std::mutex> lk(E->aux_mu);  // one user of the branches at a time
-    const uint32_t nmt = count_mt_tiles(tiles);
-    return launch_batch(d_tiles, (uint32_t)tiles.size(), nmt, count_wide_tiles(tiles, nmt), counter, ctx, st, &E->br);
+    return launch_batch(d_tiles, batch_parts(tiles), counter, ctx, st, &E->br);
 }
 
 prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_request_t *reqs, size_t n, uint64_t seed)
@@ -470,15 +501,13 @@ prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_requ
     if ((s = batch_ctx(seed, 0, &p->ctx, nullptr)) != PRAND_OK) return fail(s);
     const BatchParams P = batch_params();
     std::vector<BatchTile> tiles;
-    for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles);
+    for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles, 0, true);
     order_tiles(tiles);
     if (tiles.size() > 0xFFFFFFFFull) return fail(PRAND_ERR_ARG);
-    p->ntiles = (uint32_t)tiles.size();
-    p->nmt = count_mt_tiles(tiles);
-    p->nwide = count_wide_tiles(tiles, p->nmt);
+    p->parts = batch_parts(tiles);
     if (!dev_alloc(&p->d_counter, 64)) return fail(PRAND_ERR_NOMEM);
     if (p->br.create() != PRAND_OK) return fail(PRAND_ERR_CUDA);
-    if (p->ntiles) {
+    if (!tiles.empty()) {
         if (!dev_alloc(&p->d_tiles, tiles.size() * sizeof(BatchTile))) return fail(PRAND_ERR_NOMEM);
         if (cudaMemcpy(p->d_tiles, tiles.data(), tiles.size() * sizeof(BatchTile), cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(PRAND_ERR_CUDA);
@@ -488,7 +517,7 @@ prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_requ
     // thread-per-stream parts forked onto the plan's branch streams and joined back)
     if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return fail(PRAND_ERR_CUDA);
     if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return fail(PRAND_ERR_CUDA);
-    prand_status_t ls = launch_batch(p->d_tiles, p->ntiles, p->nmt, p->nwide, p->d_counter, p->ctx, cap, &p->br);
+    prand_status_t ls = launch_batch(p->d_tiles, p->parts, p->d_counter, p->ctx, cap, &p->br);
     cudaGraph_t g = nullptr;
     cudaError_t ce = cudaStreamEndCapture(cap, &g);
     p->graph = g;
@@ -505,7 +534,7 @@ prand_status_t prand_batch_plan_launch(prand_batch_plan_t p, prand_stream_t stre
     if (!p || !p->exec) return PRAND_ERR_ARG;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) return PRAND_ERR_STATE;
-    g_launches.fetch_add(p->ntiles ? 1 : 0, std::memory_order_relaxed);
+    g_launches.fetch_add(p->parts.all() ? 1 : 0, std::memory_order_relaxed);
     return cudaGraphLaunch(p->exec, (cudaStream_t)stream) == cudaSuccess ? PRAND_OK : PRAND_ERR_CUDA;
 }
 

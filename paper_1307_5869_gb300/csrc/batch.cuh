@@ -11,6 +11,7 @@ namespace prand {
 constexpr uint32_t kTileLast = 1u;      // the tile holds the request's last output: write the next state to wslot
 constexpr uint32_t kTileVec = 2u;       // every row start is 16-byte aligned: vector / staged-row stores
 constexpr uint32_t kTileFromSlot = 4u;  // start from the state in slot (else from the seeded base + stream * L)
+constexpr uint32_t kTileTc = 8u;        // a tile of the tensor-core kernels (gm_tc.cuh): seclen outputs per section
 
 // One unit of work for one warp (64 bytes).
 struct BatchTile {
@@ -40,7 +41,9 @@ struct BatchCtx {
 };
 
 struct BatchParams {
-    uint32_t seclen_mrg_lfsr = 8192;  // outputs per lane section (thread-per-section tiles), chosen by the tuner
+    // outputs per lane section (thread-per-section tiles), chosen by the tuner; before it
+    // has run, its choice for 10^4 mixed requests (11.3 ms at 8192, 10.1 at 2048)
+    uint32_t seclen_mrg_lfsr = 2048;
     uint32_t seclen_gm = 8192;        // outputs per warp section (lane-per-point GM/GQ tiles)
     uint32_t block = 64;              // threads per block of the rest-of-generators build (64 or 128)
     uint32_t row_bytes = 128;         // its staged row size (128 or 256 bytes: 32 or 64 u32 outputs per row store)
@@ -48,32 +51,43 @@ struct BatchParams {
 
 prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, DevTables **T);
 BatchParams batch_params();
+// tc: GM/GQ requests may go to the tensor-core kernels (from the seeded base only).
 void plan_request(const prand_request_t &r, int32_t slot, int32_t wslot, bool from_slot, const BatchParams &P,
-                  std::vector<BatchTile> &out, uint32_t max_tiles = 0);
+                  std::vector<BatchTile> &out, uint32_t max_tiles = 0, bool tc = false);
 // Number of tiles plan_request() makes for r (without planning it).
 uint64_t plan_tile_count(const prand_request_t &r, const BatchParams &P, uint32_t max_tiles = 0);
 size_t slot_words(int gen);  // 32-bit words per state slot
 prand_status_t upload_tiles(const std::vector<BatchTile> &tiles, cudaStream_t st, BatchTile **d_out, uint32_t **counter);
 void order_tiles(std::vector<BatchTile> &tiles);
 prand_status_t validate_requests(const prand_request_t *reqs, size_t n);
-// A tile list runs in three parts, each a persistent launch of its own kernel
-// build: [0, nmt) MT19937 tiles (many registers, shared memory), [nmt, nmt +
-// nwide) the thread-per-stream GM/GQ tiles (GM55, GQ58.3, GQ58.4: their points
-// need more registers than the last build allows), then every other generator
-// (few registers, many resident warps).  order_tiles puts them in that order.
-// With side branches (Branches), the MT19937 part and the thread-per-stream
-// part each run on a branch stream of their own, forked from and joined back
-// into `st`, so all three builds share the GPU at once; without them (the
-// server's flights, one stream each) the parts run one after the other.
+// A tile list runs in parts, each a persistent launch of its own kernel build, in
+// this order (order_tiles): MT19937 tiles (many registers, shared memory), the
+// thread-per-stream GM/GQ tiles (GM55, GQ58.3, GQ58.4: their points need more
+// registers than the next build allows), every other generator's (few registers,
+// many resident warps), and the tensor-core tiles, generator by generator.
+// With side branches (Branches), the MT19937, thread-per-stream and tensor-core
+// parts each run on a branch stream of their own, forked from and joined back
+// into `st`, so all share the GPU at once; without them (the server's flights, one
+// stream each) the parts run one after the other.
+struct BatchParts {
+    uint32_t mt = 0, wide = 0, rest = 0, tc[8] = {};  // tc: by generator, PRAND_GM19 first
+    uint32_t tc_all() const
+    {
+        uint32_t n = 0;
+        for (uint32_t t : tc) n += t;
+        return n;
+    }
+    uint32_t all() const { return mt + wide + rest + tc_all(); }
+};
+BatchParts batch_parts(const std::vector<BatchTile> &tiles);  // of an ordered list
+constexpr int kBranches = 3;
 struct Branches {
-    cudaStream_t st[2] = {};  // [0] MT19937 tiles, [1] thread-per-stream GM/GQ tiles
-    cudaEvent_t fork[2] = {}, join[2] = {};
+    cudaStream_t st[kBranches] = {};  // MT19937, thread-per-stream GM/GQ and tensor-core tiles
+    cudaEvent_t fork[kBranches] = {}, join[kBranches] = {};
     prand_status_t create();
     void destroy();
 };
 bool wide_tile_gen(int gen);
-uint32_t count_mt_tiles(const std::vector<BatchTile> &tiles);
-uint32_t count_wide_tiles(const std::vector<BatchTile> &tiles, uint32_t nmt);
 // Warps per MT19937 tile: the team applies each jump polynomial together
 // (each warp takes a quarter of its coefficients) and then twists each output
 // block together (five rounds of four 32-word chunks), for batches and the
@@ -81,7 +95,10 @@ uint32_t count_wide_tiles(const std::vector<BatchTile> &tiles, uint32_t nmt);
 // one warp per tile).
 constexpr int kMtTeam = 4;
 
-prand_status_t launch_batch(const BatchTile *d_tiles, uint32_t ntiles, uint32_t nmt, uint32_t nwide,
-                            uint32_t *d_counter, const BatchCtx &ctx, cudaStream_t st, const Branches *br = nullptr);
+prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter, const BatchCtx &ctx,
+                            cudaStream_t st, const Branches *br = nullptr);
+
+// The tensor-core tiles of one generator (gm_tc.cuh), from its seeded base.
+prand_status_t gm_batch(int gen, const DevTables *T, const BatchTile *tiles, uint32_t n, const void *base, cudaStream_t st);
 
 }  // namespace prand

@@ -1,6 +1,6 @@
 // Dispatch of the GM/GQ entry points to the per-generator translation units,
 // and the host copy of the Table 2 / Table 4 parameters.
-#include "prand_internal.h"
+#include "batch.cuh"
 
 namespace prand {
 
@@ -9,31 +9,37 @@ prand_status_t gm19_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &
 prand_status_t gm19_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm19_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gm19_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gm19_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gm29_table(uint64_t *, cudaStream_t);
 prand_status_t gm29_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm29_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm29_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gm29_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gm29_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gm31_table(uint64_t *, cudaStream_t);
 prand_status_t gm31_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm31_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm31_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gm31_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gm31_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gm55_table(uint64_t *, cudaStream_t);
 prand_status_t gm55_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm55_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm55_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gm55_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gm55_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gm61_table(uint64_t *, cudaStream_t);
 prand_status_t gm61_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm61_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gm61_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gm61_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gm61_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gq58_1_table(uint64_t *, cudaStream_t);
 prand_status_t gq58_1_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gq58_1_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gq58_1_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gq58_1_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gq58_1_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 prand_status_t gq58_3_table(uint64_t *, cudaStream_t);
 prand_status_t gq58_3_seed(const uint64_t *, uint64_t *, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gq58_3_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
@@ -44,6 +50,7 @@ prand_status_t gq58_4_seed(const uint64_t *, uint64_t *, uint64_t, const Variant
 prand_status_t gq58_4_init(const uint64_t *, const uint64_t *, uint64_t *, uint64_t, uint64_t, const Variant &, cudaStream_t);
 prand_status_t gq58_4_skip(const uint64_t *, uint64_t *, uint64_t, const U256 &, cudaStream_t);
 prand_status_t gq58_4_gen(const DevTables *, uint64_t *, uint64_t *, StreamRange &, void *, int, uint64_t, cudaStream_t);
+prand_status_t gq58_4_batch(const DevTables *, const BatchTile *, uint32_t, const uint64_t *, cudaStream_t);
 
 static const GmParams kGmHost[8] = {
     { 15, 28, (1ull << 19) - 1, 0, 1, 32, 32, P19, 6000000ull, 1000ull },
@@ -141,6 +148,21 @@ prand_status_t gm_gen(int gen, const DevTables *T, void *d_state, void *d_spare,
     case PRAND_GQ58_1: return gq58_1_gen(T, s, sp, R, out, dtype, nper, st);
     case PRAND_GQ58_3: return gq58_3_gen(T, s, sp, R, out, dtype, nper, st);
     case PRAND_GQ58_4: return gq58_4_gen(T, s, sp, R, out, dtype, nper, st);
+    default: return PRAND_ERR_ARG;
+    }
+}
+
+prand_status_t gm_batch(int gen, const DevTables *T, const BatchTile *tiles, uint32_t n, const void *base, cudaStream_t st)
+{
+    const uint64_t *b = (const uint64_t *)base;
+    switch (gen) {
+    case PRAND_GM19: return gm19_batch(T, tiles, n, b, st);
+    case PRAND_GM29: return gm29_batch(T, tiles, n, b, st);
+    case PRAND_GM31: return gm31_batch(T, tiles, n, b, st);
+    case PRAND_GM55: return gm55_batch(T, tiles, n, b, st);
+    case PRAND_GM61: return gm61_batch(T, tiles, n, b, st);
+    case PRAND_GQ58_1: return gq58_1_batch(T, tiles, n, b, st);
+    case PRAND_GQ58_4: return gq58_4_batch(T, tiles, n, b, st);
     default: return PRAND_ERR_ARG;
     }
 }

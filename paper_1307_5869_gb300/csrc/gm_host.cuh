@@ -72,6 +72,18 @@ struct GmHost {
         if (nper > 65536) return true;
         return 100 * ((nper + kTcSteps - 1) / kTcSteps * kTcSteps + 56) < ratio * (nper + 14);
     }
+    // A batch's tiles (plan_request) from the seeded base.
+    static prand_status_t batch(const uint64_t *tab, const GmTcTable *tc, volatile uint32_t *failed, const BatchTile *tiles,
+                                uint32_t n, const uint64_t *base, cudaStream_t st)
+    {
+        if constexpr (GmTc<GEN>::kUse) {
+            if (*failed) return PRAND_ERR_TIMEOUT;
+            const uint32_t ctas = (uint32_t)device_sm_count() * kTcCtas;
+            gm_tc_batch_kernel<GEN><<<n < ctas ? n : ctas, kTcThreads, kTcSmem, st>>>(tc, tab, TcBatch<GEN>{ tiles, n, base }, failed);
+            return launch_check();
+        }
+        return PRAND_ERR_ARG;  // not a generator of this form
+    }
     template <typename OutT>
     static prand_status_t gen(const uint64_t *tab, const GmTcTable *tc, volatile uint32_t *failed, uint64_t *state,
                               uint64_t *spare, StreamRange &R, OutT *out, uint64_t nper, cudaStream_t st)
@@ -94,9 +106,13 @@ struct GmHost {
                     const bool vec = (uintptr_t)out % (sizeof(OutT) * V) == 0 && nper % V == 0;
                     const uint64_t tiles = (units + GmTc<GEN>::kStreams - 1) / GmTc<GEN>::kStreams;
                     const unsigned grid = (unsigned)(tiles < ctas ? tiles : ctas);
-                    const auto k = vec ? gm_tc_kernel<GEN, OutT, true> : gm_tc_kernel<GEN, OutT, false>;
-                    k<<<grid, kTcThreads, kTcSmem, st>>>(tc, tab, sin, sout, (uint32_t)R.count, R.stride, nper, (uint32_t)units,
-                                                         seclen, out, failed);
+                    auto launch = [&](auto v) {
+                        constexpr bool VEC = decltype(v)::value;
+                        const TcFill<GEN, OutT, VEC> fill = { sin, sout, R.stride, nper, seclen, (uint32_t)R.count, (uint32_t)units, out };
+                        gm_tc_kernel<GEN, OutT, VEC><<<grid, kTcThreads, kTcSmem, st>>>(tc, tab, fill, failed);
+                    };
+                    if (vec) launch(std::true_type{});
+                    else launch(std::false_type{});
                     return launch_check();
                 }
             }
@@ -145,6 +161,12 @@ struct GmHost {
                                cudaStream_t st)                                                               \
     {                                                                                                         \
         return GmHost<GEN>::skip(tab, state, n, off, st);                                                     \
+    }                                                                                                         \
+    prand_status_t NAME##_batch(const DevTables *T, const BatchTile *tiles, uint32_t n, const uint64_t *base,   \
+                                cudaStream_t st)                                                              \
+    {                                                                                                         \
+        return GmHost<GEN>::batch(T->gm[GEN - PRAND_GM19], T->gm_tc[GEN - PRAND_GM19], T->wait_failed, tiles,  \
+                                  n, base, st);                                                               \
     }                                                                                                         \
     prand_status_t NAME##_gen(const DevTables *T, uint64_t *state, uint64_t *spare, StreamRange &R,            \
                               void *out, int dtype, uint64_t nper, cudaStream_t st)                            \

@@ -39,6 +39,7 @@
 // 64 with a warp group per half, 64 registers, 107 / 95; this form without the next
 // tile's product behind the last block, 139 / 119.
 #pragma once
+#include "batch.cuh"
 #include "gm_impl.cuh"
 #include "gm_tc_table.h"
 
@@ -373,6 +374,152 @@ __device__ __noinline__ uint4 tc_exact_half(const uint64_t *al_s, const uint64_t
     return acc;
 }
 
+// A block's words to `to` (this lane's first word): w[half][register], `words` of them
+// in the whole block, `first` the lane's first.  VEC: rows are aligned for stores of
+// two (v = 1) or four (v = 4) elements.
+template <int GEN, typename OutT, bool VEC>
+__device__ __forceinline__ void tc_put(const uint32_t (&w)[2][GmTc<GEN>::kRegs], OutT *to, uint32_t words, uint32_t first)
+{
+    constexpr int V = GmT<GEN>::v;
+    if (VEC && words == (uint32_t)kTcSteps) {
+        if constexpr (V == 1) {
+            store2<OutT>(to, Cvt<OutT>::f(w[0][0]), Cvt<OutT>::f(w[1][0]));
+        } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                store4<OutT>(to + kTcRow * h, Cvt<OutT>::f(w[h][0]), Cvt<OutT>::f(w[h][1]), Cvt<OutT>::f(w[h][2]), Cvt<OutT>::f(w[h][3]));
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int r = 0; r < GmTc<GEN>::kRegs; ++r) {
+                const int at = V == 1 ? h : kTcRow * h + r;
+                if (first + at < words) to[at] = Cvt<OutT>::f(w[h][r]);
+            }
+    }
+}
+
+// ------------------------------------------------------------------ sections
+// Where a kernel's sections come from: tiles of kStreams sections of nearly equal
+// length, `at` a section's place in its tile (0: the longest).
+
+// A fill's: unit g is section g / nstreams of stream g % nstreams (in order, so only
+// the last section of a stream is shorter).  units = nstreams x nsec < 2^32, seclen <
+// 2^32.  The last section of a stream leaves its next state in state_out.
+template <int GEN, typename OutT, bool VEC>
+struct TcFill {
+    using P = GmT<GEN>;
+    static constexpr int S = P::s, N = GmTc<GEN>::kStreams;
+    static constexpr bool kNextState = true;
+    const uint64_t *state_in;
+    uint64_t *state_out;
+    uint64_t stride, nper, seclen;
+    uint32_t nstreams, units;
+    OutT *out;
+    struct Section {
+        uint64_t start = 0;
+        uint32_t j = 0, len = 0;
+    };
+    __device__ __forceinline__ uint32_t tiles() const { return (units + N - 1) / N; }
+    __device__ __forceinline__ Section section(uint32_t tile, int at) const
+    {
+        Section s;
+        const uint32_t g = tile * N + at;
+        if (g >= units) return s;
+        const uint32_t sec = units == nstreams ? 0 : g / nstreams;
+        s.j = g - sec * nstreams;
+        s.start = sec * seclen;
+        s.len = s.start < nper ? (uint32_t)min(seclen, nper - s.start) : 0u;
+        return s;
+    }
+    __device__ __forceinline__ void load(const Section &s, int li, uint64_t &prev, uint64_t &cur) const
+    {
+        prev = cur = 0;
+        if (!s.len) return;
+        prev = state_in[(uint64_t)s.j * S + li];
+        cur = state_in[(stride + s.j) * S + li];
+    }
+    __device__ __forceinline__ void advance(const uint64_t *jump, const Section &s, uint64_t &zc, uint64_t &zp) const
+    {
+        if (s.start && s.len) gm_jump128<GEN>(jump, s.start, 0, zc, zp);
+    }
+    __device__ __forceinline__ unsigned char *row(const Section &s) const
+    {
+        return reinterpret_cast<unsigned char *>(out + s.j * nper + s.start);
+    }
+    __device__ __forceinline__ int form(const Section &) const { return 0; }
+    __device__ __forceinline__ static uint32_t bytes(int) { return sizeof(OutT); }
+    __device__ __forceinline__ static void put(const uint32_t (&w)[2][GmTc<GEN>::kRegs], unsigned char *to, uint32_t words, uint32_t first, int)
+    {
+        tc_put<GEN, OutT, VEC>(w, reinterpret_cast<OutT *>(to), words, first);
+    }
+    __device__ __forceinline__ bool ends(const Section &s) const { return s.len && s.start + s.len == nper; }
+    __device__ __forceinline__ void next_state(const Section &s, int li, uint64_t zp, uint64_t zc) const
+    {
+        state_out[(uint64_t)s.j * S + li] = zp << P::t;
+        state_out[(stride + s.j) * S + li] = zc << P::t;
+    }
+};
+
+// A batch's: a tile is up to kStreams sections of one request, from the seeded base
+// advanced by stream x L + the section's offset (an exponent of up to 128 bits).
+template <int GEN>
+struct TcBatch {
+    using P = GmT<GEN>;
+    static constexpr int S = P::s;
+    static constexpr bool kNextState = false;
+    const BatchTile *list;
+    uint32_t n;
+    const uint64_t *base;
+    struct Section {
+        uint64_t lo = 0, hi = 0;
+        unsigned char *out = nullptr;
+        uint32_t len = 0;
+        int form = 0;
+    };
+    __device__ __forceinline__ uint32_t tiles() const { return n; }
+    __device__ __forceinline__ Section section(uint32_t tile, int at) const
+    {
+        const BatchTile &T = list[tile];
+        Section s;
+        const uint64_t off = (uint64_t)at * T.seclen;
+        if (off >= T.len) return s;
+        s.len = (uint32_t)min((uint64_t)T.seclen, T.len - off);
+        const uint64_t add = T.start + off, klo = T.stream * P::L_;
+        s.lo = klo + add;
+        s.hi = __umul64hi(T.stream, P::L_) + (s.lo < klo ? 1u : 0u);
+        s.form = T.dtype + (T.flags & kTileVec ? 4 : 0);
+        s.out = reinterpret_cast<unsigned char *>(T.out) + off * bytes(s.form);
+        return s;
+    }
+    __device__ __forceinline__ void load(const Section &s, int li, uint64_t &prev, uint64_t &cur) const
+    {
+        prev = base[li];
+        cur = base[S + li];
+    }
+    __device__ __forceinline__ void advance(const uint64_t *jump, const Section &s, uint64_t &zc, uint64_t &zp) const
+    {
+        if (s.len) gm_jump128<GEN>(jump, s.lo, s.hi, zc, zp);
+    }
+    __device__ __forceinline__ unsigned char *row(const Section &s) const { return s.out; }
+    __device__ __forceinline__ int form(const Section &s) const { return s.form; }
+    __device__ __forceinline__ static uint32_t bytes(int form) { return (form & 3) == PRAND_DTYPE_F64 ? 8 : 4; }
+    __device__ __forceinline__ static void put(const uint32_t (&w)[2][GmTc<GEN>::kRegs], unsigned char *to, uint32_t words, uint32_t first, int form)
+    {
+        auto as = [&](auto *p) {
+            using T = typename std::remove_pointer<decltype(p)>::type;
+            if (form & 4) tc_put<GEN, T, true>(w, p, words, first);
+            else tc_put<GEN, T, false>(w, p, words, first);
+        };
+        if ((form & 3) == PRAND_DTYPE_U32) as(reinterpret_cast<uint32_t *>(to));
+        else if ((form & 3) == PRAND_DTYPE_F32) as(reinterpret_cast<float *>(to));
+        else as(reinterpret_cast<double *>(to));
+    }
+    __device__ __forceinline__ bool ends(const Section &) const { return false; }
+    __device__ __forceinline__ void next_state(const Section &, int, uint64_t, uint64_t) const {}
+};
+
 // ------------------------------------------------------------------ kernel
 // Persistent blocks of 128 threads; a tile is kStreams sections (one per warp
 // for v = 1, one per 8 lanes for v = 4), thread = point.  Per block of 64 steps a
@@ -385,16 +532,11 @@ __device__ __noinline__ uint4 tc_exact_half(const uint64_t *al_s, const uint64_t
 // tensor cores run on from tile to tile.  The strips are transposed across the
 // lanes, so lane l ends with words 2 l and 2 l + 1 (v = 1) or words 4 i .. 4 i + 3 of
 // either half of its stream's block (v = 4), and rows leave 256 or 128 bytes at a time.
-// units: sections of all streams (below 2^32), nstreams x nsec; seclen below 2^32.
 // err: a word in host memory, set if a wait ran out (the caller's next call
 // reports it).
-template <int GEN, typename OutT, bool VEC>
-__global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTable *__restrict__ tab,
-                                                                   const uint64_t *__restrict__ jump,
-                                                                   const uint64_t *state_in, uint64_t *state_out,
-                                                                   uint32_t nstreams, uint64_t stride, uint64_t nper,
-                                                                   uint32_t units, uint64_t seclen,
-                                                                   OutT *__restrict__ out, volatile uint32_t *err)
+template <int GEN, typename Src>
+__device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, const uint64_t *__restrict__ jump, const Src &src,
+                                          volatile uint32_t *err)
 {
     using P = GmT<GEN>;
     using C = GmTc<GEN>;
@@ -432,46 +574,23 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
         count_s = 0;
     }
 
-    // A tile's section of this thread: unit gid is section gid / nstreams of stream
-    // gid % nstreams.  A section's length, and from its state X0 and X1.
-    auto section = [&](uint32_t tile, uint32_t &j, uint64_t &start) -> uint64_t {
-        const uint32_t gid = tile * C::kStreams + tid / S;
-        j = 0;
-        start = nper;
-        if (gid >= units) return 0;
-        const uint32_t sec = units == nstreams ? 0 : gid / nstreams;
-        j = gid - sec * nstreams;
-        start = sec * seclen;
-        return start < nper ? min(seclen, nper - start) : 0;
-    };
-    // the blocks of a tile: those of its first section (the sections of a stream are
-    // in order, and only the last one is shorter)
-    auto tile_blocks = [&](uint32_t tile) -> uint32_t {
-        const uint64_t start = units == nstreams ? 0 : (uint64_t)(tile * C::kStreams / nstreams) * seclen;
-        return (uint32_t)((min(seclen, nper - start) + M - 1) / M);
-    };
-    auto load = [&](uint32_t j, uint64_t len, uint64_t &p, uint64_t &c) {  // the section's stream's state
-        p = c = 0;
-        if (!len) return;
-        p = state_in[(uint64_t)j * S + li];
-        c = state_in[(stride + j) * S + li];
-    };
-    auto pair = [&](uint64_t start, uint64_t len, uint64_t &zc, uint64_t &zm) {  // in: state, out: X0 and X1
+    // X0 and X1 of a section from its stream's state (prev, cur) = (zm, zc)
+    auto pair = [&](const typename Src::Section &sec, uint64_t &zc, uint64_t &zm) {
         uint64_t zp = reduce_prod<P::kind>(zm >> P::t, 0);
         zc = reduce_prod<P::kind>(zc >> P::t, 0);
-        if (start && len) gm_jump128<GEN>(jump, start, 0, zc, zp);
+        src.advance(jump, sec, zc, zp);
         zm = tc_lin<GEN>(to_a, zc, to_b, zp);
     };
 
-    const uint32_t tiles = (units + C::kStreams - 1) / C::kStreams;
-    uint32_t tile = blockIdx.x, j;
-    uint64_t start, len = section(tile, j, start);
+    const uint32_t tiles = src.tiles();
+    uint32_t tile = blockIdx.x;
+    typename Src::Section sec = src.section(tile, tid / S);
     Val x0, x1;
     TcLimbs<GEN> limbs;
     {
         uint64_t zc, zm;
-        load(j, len, zm, zc);
-        pair(start, len, zc, zm);
+        src.load(sec, li, zm, zc);
+        pair(sec, zc, zm);
         TcLimbs<GEN>(zc).store(myA, 0);
         limbs = TcLimbs<GEN>(zm);
         limbs.store(myA, 1);
@@ -498,53 +617,40 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
     for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int r = 0; r < C::kRegs; ++r) T[h].acc[r] = 0;
-    // the block whose strips are in T: where its words go (this lane's first) and how many it has
+    // the block whose strips are in T: where its words go (this lane's first), how many
+    // it has, and in which form
     const uint32_t first = P::v == 1 ? 2 * lane : 4 * li;
-    OutT *to = nullptr;
+    unsigned char *to = nullptr;
     uint32_t words = 0;
+    int to_form = 0;
     auto emit = [&]() {
         uint32_t w[2][C::kRegs];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int r = 0; r < C::kRegs; ++r) w[h][r] = transpose(T[h].acc[r]);
-        if (VEC && words == (uint32_t)M) {
-            if constexpr (P::v == 1) {
-                store2<OutT>(to, Cvt<OutT>::f(w[0][0]), Cvt<OutT>::f(w[1][0]));
-            } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    store4<OutT>(to + kTcRow * h, Cvt<OutT>::f(w[h][0]), Cvt<OutT>::f(w[h][1]), Cvt<OutT>::f(w[h][2]), Cvt<OutT>::f(w[h][3]));
-            }
-        } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int r = 0; r < C::kRegs; ++r) {
-                    const int at = P::v == 1 ? h : kTcRow * h + r;
-                    if (first + at < words) to[at] = Cvt<OutT>::f(w[h][r]);
-                }
-        }
+        src.put(w, to, words, first, to_form);
     };
 
-    OutT *o = out + j * nper + start + first;
-    uint32_t left = (uint32_t)len;         // outputs of the section not yet made
-    bool ends = len && start + len == nper;  // the section is its stream's last in this fill
-    uint32_t next = 0;                     // (in a tile's last block) the next tile, if any
+    int form = src.form(sec);
+    unsigned char *o = src.row(sec) + first * src.bytes(form);
+    uint32_t left = sec.len;       // outputs of the section not yet made
+    bool ends = src.ends(sec);     // the stream's next state is due after them
+    uint32_t next = 0;             // (in a tile's last block) the next tile, if any
     bool on = true;
     // One block; LAST: the tile's last one.
     auto block = [&](auto last_block) {
         constexpr bool LAST = decltype(last_block)::value;
         const uint64_t z2 = next_pair(x1, x0);
         const Val x2(z2);
-        uint32_t nj = 0;
-        uint64_t nstart = 0, nlen = 0, zc = 0, zm = 0;
+        typename Src::Section nsec;
+        uint64_t zc = 0, zm = 0;
         if constexpr (LAST) {
             next = tile + gridDim.x;
             on = next < tiles;
             if (on) {  // the next tile's states, on their way from here on
-                nlen = section(next, nj, nstart);
-                load(nj, nlen, zm, zc);
+                nsec = src.section(next, tid / S);
+                src.load(nsec, li, zm, zc);
             }
         }
         uint32_t d0[32], d1[32];
@@ -571,12 +677,13 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
         tc_ld_wait(d1);
         // this block's words (none once the section has ended)
         to = o;
+        to_form = form;
         words = min((uint32_t)M, left);
         left -= words;
-        o += M;
+        o += M * src.bytes(form);
         if constexpr (LAST) {
             if (on) {  // A: the next tile's first pair
-                pair(nstart, nlen, zc, zm);
+                pair(nsec, zc, zm);
                 TcLimbs<GEN>(zc).store(myA, 0);
                 limbs = TcLimbs<GEN>(zm);
                 limbs.store(myA, 1);
@@ -601,19 +708,20 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
                 if constexpr (P::v != 1) { T[h].acc[1] = e.y; T[h].acc[2] = e.z; T[h].acc[3] = e.w; }
             }
         }
-        if (ends && left == 0) {
+        if (Src::kNextState && ends && left == 0) {
             // the stream ends here for this fill: x^(n + words - 1), x^(n + words)
-            state_out[(uint64_t)j * S + li] = tc_lin<GEN>(al_s[words], x1.whole(), be_s[words], z2) << P::t;
-            state_out[(stride + j) * S + li] = tc_lin<GEN>(al_s[words + 1], x1.whole(), be_s[words + 1], z2) << P::t;
+            src.next_state(sec, li, tc_lin<GEN>(al_s[words], x1.whole(), be_s[words], z2),
+                           tc_lin<GEN>(al_s[words + 1], x1.whole(), be_s[words + 1], z2));
             ends = false;
         }
         if constexpr (LAST) {
             if (!on) return;
             tile = next;
-            j = nj;
-            o = out + j * nper + nstart + first;
-            left = (uint32_t)nlen;
-            ends = nlen && nstart + nlen == nper;
+            sec = nsec;
+            form = src.form(sec);
+            o = src.row(sec) + first * src.bytes(form);
+            left = sec.len;
+            ends = src.ends(sec);
             x0 = Val(zc);
             x1 = Val(zm);
         } else {
@@ -622,7 +730,8 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
         }
     };
     while (on) {
-        for (uint32_t b = tile_blocks(tile); b > 1; --b) block(std::false_type{});
+        // (the tile's first section is its longest)
+        for (uint32_t b = (src.section(tile, 0).len + M - 1) / M; b > 1; --b) block(std::false_type{});
         block(std::true_type{});
     }
     emit();
@@ -632,6 +741,24 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTa
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(kTcTmem) : "memory");
     }
+}
+
+template <int GEN, typename OutT, bool VEC>
+__global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_kernel(const GmTcTable *__restrict__ tab,
+                                                                   const uint64_t *__restrict__ jump,
+                                                                   const __grid_constant__ TcFill<GEN, OutT, VEC> fill,
+                                                                   volatile uint32_t *err)
+{
+    gm_tc_run<GEN>(tab, jump, fill, err);
+}
+
+template <int GEN>
+__global__ void __launch_bounds__(kTcThreads, kTcCtas) gm_tc_batch_kernel(const GmTcTable *__restrict__ tab,
+                                                                         const uint64_t *__restrict__ jump,
+                                                                         const __grid_constant__ TcBatch<GEN> batch,
+                                                                         volatile uint32_t *err)
+{
+    gm_tc_run<GEN>(tab, jump, batch, err);
 }
 
 }  // namespace prand
