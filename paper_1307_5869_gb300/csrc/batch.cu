@@ -31,22 +31,17 @@ constexpr int kBatchThreads = 64;  // the wide build: small blocks (a warp on a 
 
 // One MT19937 stream for the per-request form: stream k = base advanced by
 // k 2^432, one window polynomial per nonzero byte of k (the same jump the
-// batched MT19937 tiles take), by one warp.
-__global__ void __launch_bounds__(32) mt_window_init_kernel(const uint32_t *base, const uint32_t *win, uint64_t k,
-                                                            uint32_t *dst)
+// batched MT19937 tiles take), by one block.
+__global__ void __launch_bounds__(32 * kMtTeam) mt_window_init_kernel(const uint32_t *base, const uint32_t *win, uint64_t k,
+                                                                      uint32_t *dst)
 {
-    __shared__ uint32_t seq[2 * kMtN], pbuf[kMtPolyWords];
-    const int lane = threadIdx.x;
-    bool first = true;
+    __shared__ __align__(16) MtJumpSmem S;
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) S.state[i] = base[i];
     for (int i = 0; i < kMtWinPositions; ++i) {
         const uint32_t d = (uint32_t)(k >> (kMtWinBits * i)) & (uint32_t)(kMtWinDigits - 1);
-        if (!d) continue;
-        mt_apply_poly_warp(win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords, first ? base : dst, dst, seq, pbuf,
-                           lane);
-        first = false;
-        __syncwarp();
+        if (d) mt_jump_block<kMtTeam>(S, win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords);
     }
-    if (first) mt_copy_state_warp(base, dst, lane);
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) dst[i] = S.state[i];
 }
 
 
@@ -663,7 +658,7 @@ prand_status_t prand_batch_run_per_request(const prand_request_t *reqs, size_t n
         R.stride = R.count = 1;
         uint32_t idx = kMtN;
         if (r.gen == PRAND_MT19937) {
-            mt_window_init_kernel<<<1, 32, 0, st>>>((const uint32_t *)ctx.base[r.gen], ctx.mt_win, r.stream,
+            mt_window_init_kernel<<<1, 32 * kMtTeam, 0, st>>>((const uint32_t *)ctx.base[r.gen], ctx.mt_win, r.stream,
                                                     (uint32_t *)a);
             s = launch_check();
             if (s == PRAND_OK) s = mt_gen(a, 1, &idx, r.dev_out, r.dtype, r.length, st);

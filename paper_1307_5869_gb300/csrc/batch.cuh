@@ -88,12 +88,9 @@ struct Branches {
     void destroy();
 };
 bool wide_tile_gen(int gen);
-// Warps per MT19937 tile: the team applies each jump polynomial together
-// (each warp takes a quarter of its coefficients) and then twists each output
-// block together (five rounds of four 32-word chunks), for batches and the
-// server alike (a batch of 10^4 mixed requests ran 16 % faster so than with
-// one warp per tile).
-constexpr int kMtTeam = 4;
+// Warps per MT19937 tile: one block applies each jump polynomial and twists each output
+// block together, for batches and the server alike.
+constexpr int kMtTeam = 12;
 
 prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter, const BatchCtx &ctx,
                             cudaStream_t st, const Branches *br = nullptr);

@@ -157,29 +157,24 @@ __device__ __forceinline__ void batch_gm(const BatchTile &T, const BatchCtx &C, 
 }
 
 // ------------------------------------------------------------------ MT19937 tiles
-// One tile = one request, run by a block of TEAM warps: the team applies the
-// jump polynomials together (each warp takes a range of the coefficients),
-// then makes the outputs together (batch_mt_emit_team).  Slot layout: 624 words of the current
-// block, then the index inside it.  ring: the team's per-warp rings (2 x 624
-// words each, warp w at ring + w * ring_stride words); tstate: 624 shared
-// words holding the state between polynomial applications; pbuf: 624 shared
-// words for the polynomial being applied; part: TEAM x 624 shared words for
-// the warps' partial results.
-// The outputs of an MT19937 tile made by the whole team: b0 holds the current
-// block (written by warp 0), idx the position inside it.  Each further block
-// is twisted by all TEAM warps (mt_twist_emit_team: TEAM chunks at a time
-// instead of one), so a long request's sequential work shrinks by about TEAM.
-template <typename OutT, int TEAM>
+// One tile = one request, run by a whole block of kMtTeam warps: it applies the jump
+// polynomials (mt_jump_block), then makes the outputs.  Slot layout: 624 words of the
+// current block, then the index inside it.
+//
+// The outputs: b0 holds the current block, idx the position inside it.  Each further
+// block is twisted by the whole team (mt_twist_emit_team), so a long request's
+// sequential work is three rounds per 624 outputs.
+template <typename OutT>
 __device__ __forceinline__ void batch_mt_emit_team(const BatchTile &T, const BatchCtx &C, uint32_t *b0, uint32_t *b1,
-                                                   uint32_t idx, int warp, int lane)
+                                                   uint32_t idx)
 {
-    __syncthreads();  // warp 0's copy of the current block is visible to the team
+    __syncthreads();  // the current block is visible to the team
     OutT *o = (OutT *)T.out;
     const uint64_t nper = T.len;
     uint64_t done = 0;
     if (idx < (uint32_t)kMtN) {
         const uint32_t cnt = (uint32_t)min((uint64_t)(kMtN - idx), nper);
-        for (uint32_t t = threadIdx.x; t < cnt; t += 32 * TEAM) o[t] = Cvt<OutT>::f(mt_temper(b0[idx + t]));
+        for (uint32_t t = threadIdx.x; t < cnt; t += 32 * kMtTeam) o[t] = Cvt<OutT>::f(mt_temper(b0[idx + t]));
         done = cnt;
         idx += cnt;
     }
@@ -187,53 +182,43 @@ __device__ __forceinline__ void batch_mt_emit_team(const BatchTile &T, const Bat
     while (done < nper) {
         const uint64_t rem = nper - done;
         const uint32_t emit = rem < (uint64_t)kMtN ? (uint32_t)rem : (uint32_t)kMtN;
-        if (in_b0) mt_twist_emit_team<OutT, TEAM>(b0, b1, warp, lane, o + done, emit);
-        else mt_twist_emit_team<OutT, TEAM>(b1, b0, warp, lane, o + done, emit);
+        mt_twist_emit_team<OutT, kMtTeam>(in_b0 ? b0 : b1, in_b0 ? b1 : b0, o + done, emit);
         done += emit;
         idx = emit;
         in_b0 = !in_b0;
     }
-    if ((T.flags & kTileLast) && warp == 0) {
+    if (T.flags & kTileLast) {
         const uint32_t *cur = in_b0 ? b0 : b1;
         uint32_t *d = (uint32_t *)C.slots[PRAND_MT19937] + (kMtN + 1) * (uint64_t)T.wslot;
-        mt_copy_state_warp(cur, d, lane);
-        if (lane == 0) d[kMtN] = idx;
+        for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) d[i] = cur[i];
+        if (threadIdx.x == 0) d[kMtN] = idx;
     }
     // every warp wrote outputs: each thread fences its own writes before the
     // block barrier after which one thread publishes the tile's completion
     __threadfence();
 }
 
-template <typename OutT, int TEAM>
-__device__ __forceinline__ void batch_mt(const BatchTile &T, const BatchCtx &C, uint32_t *ring, int ring_stride,
-                                         uint32_t *tstate, uint32_t *pbuf, uint32_t *part, int warp, int lane)
+template <typename OutT>
+__device__ __forceinline__ void batch_mt(const BatchTile &T, const BatchCtx &C, MtJumpSmem &S)
 {
-    uint32_t *b0 = ring, *b1 = ring + kMtN;  // warp 0's ring, for the outputs
+    uint32_t *b0 = S.x[0], *b1 = S.x[0] + kMtN;  // the outputs' two blocks
     uint32_t idx = kMtN;
-    if (T.flags & kTileFromSlot) {
-        const uint32_t *src = (const uint32_t *)C.slots[PRAND_MT19937] + (kMtN + 1) * (uint64_t)T.slot;
-        if (warp == 0) {
-            mt_copy_state_warp(src, b0, lane);
-            __syncwarp();
-        }
+    const bool from_slot = T.flags & kTileFromSlot;
+    const uint32_t *src = from_slot ? (const uint32_t *)C.slots[PRAND_MT19937] + (kMtN + 1) * (uint64_t)T.slot
+                                    : (const uint32_t *)C.base[PRAND_MT19937];
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) S.state[i] = src[i];
+    if (from_slot) {
         idx = src[kMtN];
     } else {
         // stream k = base advanced by k 2^432: one polynomial per nonzero byte of k
-        const uint32_t *src = (const uint32_t *)C.base[PRAND_MT19937];
-        bool first = true;
         for (int i = 0; i < kMtWinPositions; ++i) {
             const uint32_t d = (uint32_t)(T.stream >> (kMtWinBits * i)) & (uint32_t)(kMtWinDigits - 1);
-            if (!d) continue;
-            mt_apply_poly_team<TEAM>(C.mt_win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords, first ? src : tstate, tstate,
-                                     ring + warp * ring_stride, pbuf, part, warp, lane);
-            first = false;
-        }
-        if (warp == 0) {
-            mt_copy_state_warp(first ? src : tstate, b0, lane);
-            __syncwarp();
+            if (d) mt_jump_block<kMtTeam>(S, C.mt_win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords);
         }
     }
-    batch_mt_emit_team<OutT, TEAM>(T, C, b0, b1, idx, warp, lane);
+    // (a thread reads back the words it wrote, or those a jump's last barrier published)
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) b0[i] = S.state[i];
+    batch_mt_emit_team<OutT>(T, C, b0, b1, idx);
 }
 
 // ------------------------------------------------------------------ the persistent kernels
@@ -289,18 +274,13 @@ __device__ __forceinline__ void batch_tile_done(const BatchTile &T, const BatchC
 // build claims tiles per block (a team of BS / 32 warps per tile), the others
 // per warp.
 template <int MODE, int BS, int ROWB>
-__global__ void __launch_bounds__(BS, (MODE == kModeRest ? 1280 / BS : MODE == kModeWide ? 512 / BS : 1)) batch_kernel(
+__global__ void __launch_bounds__(BS, (MODE == kModeRest ? 1280 / BS : MODE == kModeWide ? 512 / BS : 1536 / BS)) batch_kernel(
     const BatchTile *__restrict__ tiles, uint32_t ntiles, uint32_t *counter, BatchCtx ctx)
 {
-    __shared__ __align__(16) unsigned char smem[BS / 32][WarpSmem<ROWB>::bytes];
     if constexpr (MODE == kModeMt) {
-        constexpr int TEAM = BS / 32;  // one team of warps per block
-        static_assert(TEAM == kMtTeam, "MT19937 build: one team of warps per tile");
-        __shared__ uint32_t tstate[kMtN];
-        __shared__ uint32_t pbuf[kMtPolyWords];
-        __shared__ uint32_t part[TEAM > 1 ? TEAM * kMtN : 1];
+        static_assert(BS == 32 * kMtTeam, "MT19937 build: one team of warps per tile");
+        __shared__ __align__(16) MtJumpSmem S;
         __shared__ uint32_t claimed;
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         for (;;) {
             if (threadIdx.x == 0) claimed = atomicAdd(counter, 1u);
             __syncthreads();
@@ -308,15 +288,14 @@ __global__ void __launch_bounds__(BS, (MODE == kModeRest ? 1280 / BS : MODE == k
             __syncthreads();
             if (t >= ntiles) return;
             const BatchTile T = tiles[t];
-            uint32_t *ring = reinterpret_cast<uint32_t *>(&smem[0][0]);
-            constexpr int stride = WarpSmem<ROWB>::bytes / 4;
-            if (T.dtype == PRAND_DTYPE_U32) batch_mt<uint32_t, TEAM>(T, ctx, ring, stride, tstate, pbuf, part, warp, lane);
-            else if (T.dtype == PRAND_DTYPE_F32) batch_mt<float, TEAM>(T, ctx, ring, stride, tstate, pbuf, part, warp, lane);
-            else batch_mt<double, TEAM>(T, ctx, ring, stride, tstate, pbuf, part, warp, lane);
+            if (T.dtype == PRAND_DTYPE_U32) batch_mt<uint32_t>(T, ctx, S);
+            else if (T.dtype == PRAND_DTYPE_F32) batch_mt<float>(T, ctx, S);
+            else batch_mt<double>(T, ctx, S);
             __syncthreads();
             if (threadIdx.x == 0) batch_tile_done(T, ctx);
         }
     } else {
+        __shared__ __align__(16) unsigned char smem[BS / 32][WarpSmem<ROWB>::bytes];
         const int lane = threadIdx.x & 31;
         unsigned char *wsm = smem[threadIdx.x >> 5];
         for (;;) {

@@ -16,7 +16,7 @@
 // Jump (Sec. 5.4): A^v Y = g_v(A) Y = sum_i a_i A^(i-1) Y with g_v = x^v mod phi.
 // With Y in window form (x_t..x_{t+623}), A^i Y is the window starting at
 // x_{t+i}, so the sum is a sliding-window XOR over the stream's next 20560
-// words, taken at the set coefficients of g_v.
+// words, taken at the set coefficients of g_v (mt_jump_block).
 #include "mt_dev.cuh"
 
 namespace prand {
@@ -95,36 +95,38 @@ __global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_gen_kernel(uint32_t 
 }
 
 // ------------------------------------------------------------------ jump
-// Doubling level: dst stream (off + j) := g(A) (src stream j), j < count.
-__global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_level_kernel(const uint32_t *poly, uint32_t *state,
-                                                                         uint64_t off, uint64_t count)
+// Blocks of 12 warps, four to an SM (40 registers): one wave holds 608 streams, and 65536
+// streams take 18.2 ms (6 warps 18.1, 3 warps 21.5, 15 warps 19.7, 30 warps 28.0) with the
+// small levels, which are latency, at 55 us each (6 warps 100, 3 warps 200, 30 warps 33).
+// The first stream of a handle is alone on the chip, in a chain of one jump per set bit:
+// 30 warps (0.60 ms for a chain of eight; 12 warps 0.80).
+constexpr int kMtLevelWarps = 12, kMtMultiWarps = 30;
+
+// Doubling level: dst stream (off + j) := g(A) (src stream j), one block per stream.
+__global__ void __launch_bounds__(32 * kMtLevelWarps, 4) mt_level_kernel(const uint32_t *poly, uint32_t *state, uint64_t off)
 {
-    __shared__ uint32_t seq[kMtWarpsPerBlock][2 * kMtN], pbuf[kMtWarpsPerBlock][kMtPolyWords];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint64_t j = (uint64_t)blockIdx.x * kMtWarpsPerBlock + w;
-    if (j >= count) return;
-    mt_apply_poly_warp(poly, state + j * kMtN, state + (off + j) * kMtN, seq[w], pbuf[w], lane);
+    __shared__ __align__(16) MtJumpSmem S;
+    const uint64_t j = blockIdx.x;
+    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) S.state[i] = state[j * kMtN + i];
+    mt_jump_block<kMtLevelWarps>(S, poly);
+    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) state[(off + j) * kMtN + i] = S.state[i];
 }
 
 // Every stream advanced by the set bits of a 512-bit offset (one polynomial
-// x^(2^b) mod phi per set bit b, applied one after another in place).
+// x^(2^b) mod phi per set bit b, applied one after another), one block per stream.
 struct MtBits { uint64_t w[8]; };
 
-__global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_multi_kernel(const uint32_t *polys, uint32_t *state,
-                                                                         uint64_t n, MtBits e, uint32_t *scratch)
+template <int NW, int MB>
+__global__ void __launch_bounds__(32 * NW, MB) mt_multi_kernel(const uint32_t *polys, uint32_t *state, MtBits e)
 {
-    __shared__ uint32_t seq[kMtWarpsPerBlock][2 * kMtN], pbuf[kMtWarpsPerBlock][kMtPolyWords];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint64_t j = (uint64_t)blockIdx.x * kMtWarpsPerBlock + w;
-    if (j >= n) return;
-    uint32_t *s = state + j * kMtN;
+    __shared__ __align__(16) MtJumpSmem S;
+    uint32_t *s = state + (uint64_t)blockIdx.x * kMtN;
+    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) S.state[i] = s[i];
     for (int b = 0; b < 512; ++b) {
         if (!((e.w[b >> 6] >> (b & 63)) & 1u)) continue;
-        // result goes to registers then back over s (src is copied to smem first)
-        mt_apply_poly_warp(polys + (size_t)b * kMtPolyWords, s, s, seq[w], pbuf[w], lane);
-        __syncwarp();
+        mt_jump_block<NW>(S, polys + (size_t)b * kMtPolyWords);
     }
-    (void)scratch;
+    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) s[i] = S.state[i];
 }
 
 // ------------------------------------------------------------------ host
@@ -150,15 +152,14 @@ prand_status_t mt_init(const DevTables *T, const void *d_base, void *d_state, ui
         // first * 2^shift: bits shift .. shift + 63
         for (int b = 0; b < 64; ++b)
             if ((first >> b) & 1u) e.w[(shift + b) >> 6] |= 1ull << ((shift + b) & 63);
-        mt_multi_kernel<<<1, 32 * kMtWarpsPerBlock, 0, st>>>(T->mt, state, 1, e, nullptr);
+        mt_multi_kernel<kMtMultiWarps, 1><<<1, 32 * kMtMultiWarps, 0, st>>>(T->mt, state, e);
         prand_status_t s = launch_check();
         if (s != PRAND_OK) return s;
     }
     for (int b = 0; b < 64 && (1ull << b) < n; ++b) {
         uint64_t have = 1ull << b;
         uint64_t count = min(have, n - have);
-        mt_level_kernel<<<grid_warps(count), 32 * kMtWarpsPerBlock, 0, st>>>(
-            T->mt + (size_t)(shift + b) * kMtPolyWords, state, have, count);
+        mt_level_kernel<<<(unsigned)count, 32 * kMtLevelWarps, 0, st>>>(T->mt + (size_t)(shift + b) * kMtPolyWords, state, have);
         prand_status_t s = launch_check();
         if (s != PRAND_OK) return s;
     }
@@ -190,7 +191,7 @@ prand_status_t mt_skip512(const DevTables *T, void *d_state, uint64_t n, uint32_
     bool any = false;
     for (int i = 0; i < 8; ++i) any = any || e.w[i];
     if (!any) return PRAND_OK;
-    mt_multi_kernel<<<grid_warps(n), 32 * kMtWarpsPerBlock, 0, st>>>(T->mt, (uint32_t *)d_state, n, e, nullptr);
+    mt_multi_kernel<kMtLevelWarps, 4><<<(unsigned)n, 32 * kMtLevelWarps, 0, st>>>(T->mt, (uint32_t *)d_state, e);
     return launch_check();
 }
 

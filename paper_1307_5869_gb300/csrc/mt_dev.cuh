@@ -1,7 +1,7 @@
 // Device routines of MT19937 (Matsumoto & Nishimura 1998; Sec. 5.4) shared by
 // the per-handle kernels and the batched persistent kernel: the recurrence
 // word, tempering, the fused twist-and-emit of one block, and the polynomial
-// jump of eq. (g_v) applied by one warp.
+// jump of eq. (g_v) applied by one block.
 #pragma once
 #include "devcommon.cuh"
 
@@ -71,25 +71,22 @@ __device__ __forceinline__ void mt_twist_emit_chunks(const uint32_t *__restrict_
     }
 }
 
-// The same twist by a team of TEAM warps that make up the whole block (TEAM
-// divides 20): in round r, warp w makes chunk TEAM r + w.  A chunk reads new
-// words only from chunks at least seven before it, i.e. from earlier rounds,
-// so one block barrier per round orders every such read after its write; a
-// final barrier publishes the new block.  All TEAM warps call it.
+// The same twist by a team of TEAM warps that make up the whole block, in rounds of 227
+// words (or of one per thread): a word reads new words 227 or more before it, i.e. from
+// earlier rounds, so one block barrier per round orders every such read after its
+// write; the last one publishes the new block.  All TEAM warps call it.
 template <typename OutT, int TEAM>
-__device__ __forceinline__ void mt_twist_emit_team(const uint32_t *__restrict__ ob, uint32_t *__restrict__ nb, int warp,
-                                                   int lane, OutT *o, uint32_t emit)
+__device__ __forceinline__ void mt_twist_emit_team(const uint32_t *__restrict__ ob, uint32_t *__restrict__ nb, OutT *o,
+                                                   uint32_t emit)
 {
-    static_assert(20 % TEAM == 0 && TEAM <= 4, "chunks per round");
+    constexpr int ROUND = 32 * TEAM < kMtN - kMtM ? 32 * TEAM : kMtN - kMtM;
 #pragma unroll
-    for (int r = 0; r < 20 / TEAM; ++r) {
-        const int c = TEAM * r + warp;
-        const int k = 32 * c + lane;
-        if (k < kMtN) {
-            const uint32_t a = ob[k];
-            const uint32_t b = k + 1 < kMtN ? ob[k + 1] : nb[0];
+    for (int a = 0; a < kMtN; a += ROUND) {
+        const int k = a + threadIdx.x;
+        if (threadIdx.x < ROUND && k < kMtN) {
+            const uint32_t nxt = k + 1 < kMtN ? ob[k + 1] : nb[0];
             const uint32_t p = k < kMtN - kMtM ? ob[k + kMtM] : nb[k - (kMtN - kMtM)];
-            const uint32_t x = mt_recur(a, b, p);
+            const uint32_t x = mt_recur(ob[k], nxt, p);
             nb[k] = x;
             if ((uint32_t)k < emit) o[k] = Cvt<OutT>::f(mt_temper(x));
         }
@@ -105,150 +102,153 @@ __device__ __forceinline__ void mt_twist_emit(const uint32_t *__restrict__ ob, u
     else mt_twist_emit_chunks<OutT, false>(ob, nb, lane, o, emit);
 }
 
-// Twist of one block out of place (no output): the 20-chunk in-order schedule
-// of mt_twist_emit_chunks, kept as a compact loop (it runs inside the jump's
-// unrolled sliding-window loop, where code size matters more than its cost).
-__device__ __forceinline__ void mt_twist_block(const uint32_t *ob, uint32_t *nb, int lane)
-{
-#pragma unroll 4
-    for (int c = 0; c < 20; ++c) {
-        const int k = 32 * c + lane;
-        if (k < kMtN) {
-            const uint32_t b = k + 1 < kMtN ? ob[k + 1] : nb[0];
-            const uint32_t p = k < 227 ? ob[k + 397] : nb[k - 227];
-            nb[k] = mt_recur(ob[k], b, p);
-        }
-        if ((c & 3) == 3) __syncwarp();
-    }
-}
-
-// dst := the part of g(A) src that coefficients [c0, c1) of g contribute to
-// result words [m0, m1), for one stream, by one warp (eq. (g_v)).  poly: g's
-// 624 coefficient words, staged in shared memory by the caller.
+// ------------------------------------------------------------------ jump
+// state := g(A) state for one stream, by one block (eq. (g_v)).
 //
-// With src in window form x_0..x_623, A^i src is the window x_i..x_{i+623}, so
-// result word m is the XOR of x_{i+m} over the set coefficients i of g.  Lane
-// l owns W consecutive result words m = mbase + j (mbase = m0 + W l, clamped to
-// m1 - W; a clamped lane writes only the words past the previous lane's) and
-// keeps the W sequence words x_{i+mbase..i+mbase+W-1} in registers as a window
-// that slides by one word per coefficient: one shared-memory load per
-// coefficient, and W register XORs per set coefficient (one three-input XOR
-// when two neighbouring coefficients are both set; W is even).  seq is this
-// warp's 1248-word ring holding two consecutive 624-word blocks of the
-// sequence (x at index i sits at seq[i mod 1248]): blocks 0 and 1 are made
-// from src, and the warp twists on to the blocks around c0 before its first
-// coefficient; block b then replaces block b - 2 at the first chunk of W
-// coefficients from which no lane loads below index 624 (b - 1) again (loads
-// from chunk start i0 on reach x_{i0+m0+W-1} and up).  c0 and c1 are multiples
-// of W.  src and dst may be the same buffer only when every warp that reads
-// src has copied it before any warp writes dst (sync: called between the two).
-template <int W, typename Sync>
-__device__ inline void mt_apply_poly_part(const uint32_t *__restrict__ poly, const uint32_t *src, uint32_t *dst,
-                                          uint32_t *seq, int lane, int m0, int m1, int c0, int c1, Sync &&sync)
+// With the state in window form x_0..x_623, A^i of it is the window x_i..x_{i+623}, so
+// result word m is R_m = sum over the set coefficients g_i of x_{i+m} over GF(2): a
+// product of a Toeplitz matrix with the coefficient vector.  It is split once in the
+// manner of Karatsuba.  Take coefficients and results in blocks of K = 320 (two blocks
+// of results, the last 16 unused); with G_q the q-th block of coefficients and
+// G_q * X_s the K results sum_r g_{Kq+r} x_{Ks+r+m}, a pair q, q + 1 (q even) adds
+//   to results 0..319:    G_q * X_q     + G_{q+1} * X_{q+1} = A + B
+//   to results 320..639:  G_q * X_{q+1} + G_{q+1} * X_{q+2} = A + C
+// with A = (G_q + G_{q+1}) * X_{q+1}, B = G_q * Y_q, C = G_{q+1} * Y_{q+1} and
+// Y_s = X_s + X_{s+1}, i.e. y_i = x_i ^ x_{i+320}: three products of half the size each
+// way instead of four.
+//
+// One warp computes (a share of the coefficients of) one of the three products: lane l
+// owns the W = 10 consecutive results from 10 l, and keeps the sequence words from
+// there on in registers as a window that slides by four words per group of four
+// coefficients (two 8-byte shared-memory loads, free of bank conflicts at this stride).
+// A group costs, per result, 1.25 logic operations on average over its 16 patterns of
+// coefficients (0, 1 or 2 three-input XORs), selected by a tree of branches that are
+// uniform over the warp.  The window's P = 16 registers come round every 16
+// coefficients, so the loop is unrolled over a chunk of 16; wider windows are slower,
+// because the 16 patterns of every group of the chunk no longer fit the instruction
+// caches (21 results per lane and groups of four: 30 KB of code, warps stalled on
+// instruction fetch for half of the time).
+// The block goes through the coefficients in steps of one pair (640): the next step's
+// 640 sequence words are made by the whole block (a word needs the one 227 before it,
+// so three rounds of 227) into the other buffer, then every warp takes its share of
+// the step.
+//
+// Bound by instruction issue: 32 steps x 3 products x 80 groups per stream, each 12.5
+// logic operations (two-cycle ones: 5.4 ms of the ALU pipe for 32768 streams), two loads
+// and about 20 instructions of branches, uniform tests and moves.  32768 streams: 8.6 ms
+// (82 % of the issue slots), where one warp per stream over the unsplit sum, in groups of
+// two coefficients, took 12.7 ms; one stream alone 55 us with 12 warps, where that took
+// 670 us.  Groups of two coefficients 10.1 ms; a switch instead of the tree 8.7 ms;
+// branches the compiler does not know to be uniform 9.7 ms.
+constexpr int kMtK = 320, kMtStep = 2 * kMtK, kMtSteps = (kMtDeg + kMtStep - 1) / kMtStep;  // 32 steps
+constexpr int kMtW = 10, kMtP = 16, kMtG = 4;
+
+struct MtJumpSmem {
+    uint32_t x[2][2 * kMtStep];       // x_{640 Q} .. x_{640 Q + 1279} of step Q, in buffer Q & 1
+    uint32_t y[2][3 * kMtK];          // y_i = x_i ^ x_{i + 320}
+    uint32_t poly[kMtStep / 32 * kMtSteps];
+    uint32_t state[kMtStep];
+};
+
+template <int U, int BIT, int PAT>
+__device__ __forceinline__ void mt_poly_tree(uint32_t bits, uint32_t (&acc)[kMtW], const uint32_t (&x)[kMtP])
 {
-    static_assert(W % 2 == 0 && W <= 32, "pairs of coefficients per step");
-    constexpr int RING = 2 * kMtN;
-    const int mwant = m0 + W * lane;
-    const int mbase = mwant + W <= m1 ? mwant : m1 - W;
-    uint32_t acc[W], win[W];
+    if constexpr (BIT >= 0) {
+        if (bits & (1u << (U + BIT))) mt_poly_tree<U, BIT - 1, PAT | (1 << BIT)>(bits, acc, x);
+        else mt_poly_tree<U, BIT - 1, PAT>(bits, acc, x);
+    } else if constexpr (PAT != 0) {
 #pragma unroll
-    for (int j = 0; j < W; ++j) acc[j] = 0;
-    mt_copy_state_warp(src, seq, lane);
-    __syncwarp();
-    sync();  // every warp holds its copy of src
-    mt_twist_block(seq, seq + kMtN, lane);  // block 1 into slot 1
-    const int b0 = c0 / kMtN;
-    for (int b = 2; b <= b0 + 1; ++b) {  // blocks b0 and b0 + 1 in the ring
-        __syncwarp();
-        mt_twist_block(seq + ((b - 1) & 1) * kMtN, seq + (b & 1) * kMtN, lane);
+        for (int j = 0; j < kMtW; ++j)
+#pragma unroll
+            for (int t = 0; t < kMtG; ++t)
+                if ((PAT >> t) & 1) acc[j] ^= x[(U + j + t) % kMtP];
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < W - 1; ++j) win[j] = seq[(c0 + mbase + j) % RING];
-    int next_block = b0 + 2;
-    int p0 = (c0 + mbase + W - 1) % RING;  // ring position of the word loaded at step i0
-    for (int i0 = c0; i0 < c1; i0 += W) {
-        if (next_block <= 32 && i0 >= kMtN * (next_block - 1) - m0 - W + 1) {
-            __syncwarp();
-            mt_twist_block(seq + ((next_block - 1) & 1) * kMtN, seq + (next_block & 1) * kMtN, lane);
-            ++next_block;
-        }
-        const int w = i0 >> 5, sh = i0 & 31;
-        const uint64_t two = (uint64_t)poly[w] | ((uint64_t)(w + 1 < kMtPolyWords ? poly[w + 1] : 0u) << 32);
-        const uint32_t bits = (uint32_t)(two >> sh) & (uint32_t)((1ull << W) - 1u);
-#pragma unroll
-        for (int u = 0; u < W; u += 2) {
-            // step u: window slots (u + j) % W hold x_{i0+u+mbase+j}; the newest,
-            // x_{i0+u+mbase+W-1}, goes into slot (u + W - 1) % W.  Step u + 1 needs
-            // x_{i0+u+1+mbase+W-1} as its j = W - 1 word (nx); it replaces the
-            // oldest word (slot u % W) only after both steps are applied.
-            int pa = p0 + u, pb = p0 + u + 1;
-            if (pa >= RING) pa -= RING;
-            if (pb >= RING) pb -= RING;
-            win[(u + W - 1) % W] = seq[pa];
-            const uint32_t nx = seq[pb];
-            const uint32_t pat = (bits >> u) & 3u;
-            if (pat == 1u) {
-#pragma unroll
-                for (int j = 0; j < W; ++j) acc[j] ^= win[(u + j) % W];
-            } else if (pat == 2u) {
-#pragma unroll
-                for (int j = 0; j < W; ++j) acc[j] ^= (j < W - 1 ? win[(u + 1 + j) % W] : nx);
-            } else if (pat == 3u) {
-#pragma unroll
-                for (int j = 0; j < W; ++j) acc[j] ^= win[(u + j) % W] ^ (j < W - 1 ? win[(u + 1 + j) % W] : nx);
-            }
-            win[u % W] = nx;
-        }
-        p0 += W;
-        if (p0 >= RING) p0 -= RING;
-    }
-    __syncwarp();
-    const int jfirst = mwant - mbase;  // words of this lane not already written by the previous lane
-#pragma unroll
-    for (int j = 0; j < W; ++j)
-        if (j >= jfirst) dst[mbase + j] = acc[j];
-    __syncwarp();
 }
 
-constexpr int kMtChunkW = 20;                                       // result words per lane, coefficients per chunk
-constexpr int kMtChunks = (kMtDeg + kMtChunkW - 1) / kMtChunkW;     // 997 chunks of coefficients
-
-// dst := g(A) src for one stream by one warp (lane l owns 20 result words);
-// poly in global memory, staged into pbuf (624 shared words of this warp).
-__device__ inline void mt_apply_poly_warp(const uint32_t *__restrict__ poly, const uint32_t *src, uint32_t *dst,
-                                          uint32_t *seq, uint32_t *pbuf, int lane)
+template <int U>
+__device__ __forceinline__ void mt_poly_groups(uint32_t bits, const uint32_t *run, uint32_t (&acc)[kMtW], uint32_t (&x)[kMtP])
 {
-    mt_copy_state_warp(poly, pbuf, lane);  // 624 words, as a state
-    __syncwarp();
-    mt_apply_poly_part<kMtChunkW>(pbuf, src, dst, seq, lane, 0, kMtN, 0, kMtChunkW * kMtChunks, [] {});
+    if constexpr (U < kMtP) {
+#pragma unroll
+        for (int t = 0; t < kMtG; t += 2) {  // words U + 10 .. U + 13; the last is ahead of its use
+            const uint2 v = *reinterpret_cast<const uint2 *>(run + U + kMtW + t);
+            x[(U + kMtW + t) % kMtP] = v.x;
+            x[(U + kMtW + t + 1) % kMtP] = v.y;
+        }
+        mt_poly_tree<U, kMtG - 1, 0>(bits, acc, x);
+        mt_poly_groups<U + kMtG>(bits, run, acc, x);
+    }
 }
 
-// The same by a team of T warps of one block (T = blockDim.x / 32), for one
-// stream's latency: the coefficients are split in T consecutive ranges, warp w
-// computes its range's contribution to all 624 result words into part[w]
-// (T x 624 shared words), each warp making its own copy of the sequence up to
-// its range, and the result is the XOR of the T parts (the sum of eq. (g_v) is
-// linear over GF(2)).  The team stages the polynomial into pbuf (624 shared
-// words) first; the block barrier after the copies of src lets dst alias src.
-template <int T>
-__device__ inline void mt_apply_poly_team(const uint32_t *__restrict__ poly, const uint32_t *src, uint32_t *dst,
-                                          uint32_t *seq, uint32_t *pbuf, uint32_t *part, int warp, int lane)
+// All 32 NW threads call it; S.state holds the state before and after (a barrier at the
+// end publishes it).  poly: g's 624 coefficient words.  NW is a multiple of 3 whose
+// third divides the 20 chunks of a block of coefficients.
+template <int NW>
+__device__ __forceinline__ void mt_jump_block(MtJumpSmem &S, const uint32_t *__restrict__ poly)
 {
-    const int c0 = kMtChunkW * (kMtChunks * warp / T), c1 = kMtChunkW * (kMtChunks * (warp + 1) / T);
-    for (int i = threadIdx.x; i < kMtPolyWords; i += 32 * T) pbuf[i] = poly[i];
-    mt_apply_poly_part<kMtChunkW>(pbuf, src, T == 1 ? dst : part + warp * kMtN, seq, lane, 0, kMtN, c0, c1,
-                                  [] { __syncthreads(); });
+    constexpr int NT = 32 * NW, SHARE = kMtK / (NW / 3), ROUND = NT < 227 ? NT : 227;
+    static_assert(NW % 3 == 0 && SHARE * (NW / 3) == kMtK && SHARE % kMtP == 0, "shares of whole chunks");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int role = warp % 3, c0 = SHARE * (warp / 3);
+    __syncthreads();  // S.state written by the caller, or by the last jump
+    for (int i = tid; i < kMtN; i += NT) S.x[0][i] = S.state[i];
+    for (int i = tid; i < (int)(sizeof(S.poly) / 4); i += NT) S.poly[i] = i < kMtPolyWords ? poly[i] : 0u;
     __syncthreads();
-    if constexpr (T > 1) {
-        for (int m = threadIdx.x; m < kMtN; m += 32 * T) {
-            uint32_t r = 0;
-#pragma unroll
-            for (int w = 0; w < T; ++w) r ^= part[w * kMtN + m];
-            dst[m] = r;
-        }
+    for (int i = tid; i < kMtStep; i += NT) S.state[i] = 0;
+    for (int a = kMtN; a < 2 * kMtStep; a += ROUND) {  // the rest of the first step's words
+        const int n = a + tid;
+        if (tid < ROUND && n < 2 * kMtStep)
+            S.x[0][n] = mt_recur(S.x[0][n - kMtN], S.x[0][n - kMtN + 1], S.x[0][n - (kMtN - kMtM)]);
         __syncthreads();
     }
+    for (int i = tid; i < 3 * kMtK; i += NT) S.y[0][i] = S.x[0][i] ^ S.x[0][i + kMtK];
+    uint32_t acc[kMtW], x[kMtP];
+#pragma unroll
+    for (int j = 0; j < kMtW; ++j) acc[j] = 0;
+#pragma unroll 1
+    for (int Q = 0; Q < kMtSteps; ++Q) {
+        const int b = Q & 1;
+        __syncthreads();  // this step's words are written; buffer b ^ 1 is read no more
+        if (Q + 1 < kMtSteps) {
+            const uint32_t *ob = S.x[b];
+            uint32_t *nb = S.x[b ^ 1];
+            for (int i = tid; i < kMtStep; i += NT) nb[i] = ob[kMtStep + i];
+            __syncthreads();
+#pragma unroll 1
+            for (int a = kMtStep; a < 2 * kMtStep; a += ROUND) {
+                const int n = a + tid;
+                if (tid < ROUND && n < 2 * kMtStep) nb[n] = mt_recur(nb[n - kMtN], nb[n - kMtN + 1], nb[n - (kMtN - kMtM)]);
+                __syncthreads();
+            }
+            for (int i = tid; i < 3 * kMtK; i += NT) S.y[b ^ 1][i] = nb[i] ^ nb[i + kMtK];
+        }
+        // coefficients 640 Q + (320 for C) + c, c0 <= c < c1, none past the polynomial's end
+        const int left = kMtDeg - (kMtStep * Q + (role == 2 ? kMtK : 0));
+        const int c1 = min(c0 + SHARE, left);
+        const uint32_t *run = (role == 0 ? S.x[b] + kMtK : role == 1 ? S.y[b] : S.y[b] + kMtK) + c0 + kMtW * lane;
+        const uint32_t *g = S.poly + (kMtStep / 32) * Q;
+#pragma unroll
+        for (int j = 0; j < kMtW; j += 2) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(run + j);
+            x[j] = v.x;
+            x[j + 1] = v.y;
+        }
+#pragma unroll 1
+        for (int c = c0; c < c1; c += kMtP) {
+            uint32_t bits = role < 2 ? g[c >> 5] : 0u;
+            if (role != 1) bits ^= g[(kMtK + c) >> 5];
+            // (a reduction's result is uniform to the compiler, and so are the branches on it)
+            bits = __reduce_or_sync(kFull, bits >> (c & 16));
+            mt_poly_groups<0>(bits, run, acc, x);
+            run += kMtP;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kMtW; ++j) {  // (result 640 and on do not exist: 320 + 319 is the last)
+        if (role != 2) atomicXor(&S.state[kMtW * lane + j], acc[j]);
+        if (role != 1) atomicXor(&S.state[kMtK + kMtW * lane + j], acc[j]);
+    }
+    __syncthreads();
 }
 
 }  // namespace prand
