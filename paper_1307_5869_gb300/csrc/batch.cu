@@ -219,9 +219,9 @@ uint64_t plan_tile_count(const prand_request_t &r, const BatchParams &P, uint32_
 // one block, each from its own jump, so a tile's sections are of one length, whole
 // blocks of 64 outputs, at most kTcSection: long enough that a jump is a small part of
 // a section, short enough that the longest requests still spread over tens of blocks
-// (10^4 mixed requests, the part's five larger generators alone: 6.1 ms at 512, 4.0 at
-// 1024, 3.0 at 2048, 2.5 at 4096, 2.3 at 8192; 100 requests without MT19937: 0.58,
-// 0.57, 0.57, 0.57, 0.62 ms).
+// (10^4 mixed requests, the part's five larger generators alone: 2.33 ms at 512, 2.11 at
+// 1024, 1.99 at 2048, 1.93 at 4096; 100 requests without MT19937: 0.56, 0.56, 0.59,
+// 0.58 ms).
 constexpr uint64_t kTcSection = 4096;
 
 bool tc_tile_gen(int gen) { return is_gm(gen) && gen != PRAND_GQ58_3; }

@@ -119,7 +119,7 @@ __device__ __forceinline__ void batch_gm(const BatchTile &T, const BatchCtx &C, 
         uint64_t zp = src[lane] >> P::t, zc = src[P::s + lane] >> P::t;
         uint64_t lo, hi;
         exponent(0, lo, hi);
-        gm_jump128<GEN>(tab, lo, hi, zc, zp);
+        gm_apply<GEN>(gm_pow_group<GEN, 32, true>(tab, lo, hi), zc, zp);
         OutT *o = (OutT *)T.out;
         uint32_t *myslot = reinterpret_cast<uint32_t *>(wsm) + 4 * lane;
         if (T.flags & kTileVec) gm_generate_section<GEN, OutT, true>(zc, zp, lane, o, len, myslot);

@@ -9,6 +9,7 @@ template <int GEN>
 inline prand_status_t gm_build_table_t(uint64_t *tab, cudaStream_t st)
 {
     gm_table_kernel<GEN><<<1, 32, 0, st>>>(tab);
+    gm_window_kernel<GEN><<<kGmDigits, 256, 0, st>>>(tab);
     return launch_check();
 }
 
@@ -24,8 +25,7 @@ struct GmHost {
     static prand_status_t init(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first, uint64_t n,
                                const Variant &V, cudaStream_t st)
     {
-        const unsigned B = 128;
-        gm_init_kernel<GEN><<<gm_grid_for(n * GmT<GEN>::s, B), B, 0, st>>>(tab, base, state, first, n, V.L[0], V.L[1]);
+        gm_init_kernel<GEN><<<gm_grid_for(n, kGmInitThreads), kGmInitThreads, 0, st>>>(tab, base, state, first, n, V.L[0], V.L[1]);
         return launch_check();
     }
     static prand_status_t skip(const uint64_t *tab, uint64_t *state, uint64_t n, const U256 &off, cudaStream_t st)

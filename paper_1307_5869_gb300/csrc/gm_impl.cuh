@@ -290,73 +290,123 @@ __device__ __forceinline__ uint32_t gm_strip_insert(GmZ<GEN> z, uint32_t w)
 }
 
 // ----------------------------------------------------------------- jumps
-// M = [[k, -q], [1, 0]] acting on (z^(n), z^(n-1)); tab[b] = M^(2^b) mod p.
+// a x + b y (mod p), canonical; every operand <= p.
 template <int GEN>
-__global__ void gm_table_kernel(uint64_t *tab)
+__device__ __forceinline__ uint64_t gm_lin(uint64_t a, uint64_t x, uint64_t b, uint64_t y)
 {
-    using P = GmT<GEN>;
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    uint64_t m0 = P::k % P::p, m1 = P::p - P::q % P::p, m2 = 1, m3 = 0;
-#pragma unroll 1
-    for (int b = 0; b < kJumpBits; ++b) {
-        tab[4 * b] = m0; tab[4 * b + 1] = m1; tab[4 * b + 2] = m2; tab[4 * b + 3] = m3;
-        uint64_t n0 = addmod_p<P::kind>(mulmod_p<P::kind>(m0, m0), mulmod_p<P::kind>(m1, m2));
-        uint64_t n1 = addmod_p<P::kind>(mulmod_p<P::kind>(m0, m1), mulmod_p<P::kind>(m1, m3));
-        uint64_t n2 = addmod_p<P::kind>(mulmod_p<P::kind>(m2, m0), mulmod_p<P::kind>(m3, m2));
-        uint64_t n3 = addmod_p<P::kind>(mulmod_p<P::kind>(m2, m1), mulmod_p<P::kind>(m3, m3));
-        m0 = n0; m1 = n1; m2 = n2; m3 = n3;
+    constexpr int K = GmT<GEN>::kind;
+    if constexpr (K == P51 || K == P61) {
+        const uint64_t l0 = a * x, l1 = b * y, lo = l0 + l1;
+        const uint64_t hi = __umul64hi(a, x) + __umul64hi(b, y) + (lo < l0 ? 1u : 0u);
+        return reduce_prod<K>(lo, hi);
+    } else {
+        return reduce_prod<K>((uint64_t)(uint32_t)a * (uint32_t)x + (uint64_t)(uint32_t)b * (uint32_t)y, 0);
     }
 }
 
+// A jump by e steps is M^e, M = [[k, -q], [1, 0]] on (z^(n), z^(n-1)), and the powers of M
+// are the elements u + w x of Z_p[x] / (x^2 - k x + q) with x for M: two words and five
+// modular products each instead of a matrix's four and eight.  The table of a
+// generator (tab): x^(2^b), b < kJumpBits (u, w), then by bytes x^(d 2^(8 i)),
+// i < kGmDigits, d < 256.  A jump of 64 set bits was a chain of 64 matrix applications at
+// every point of a stream; now it is one product per byte, or a tree of them over the
+// lanes that need it, and one application per point (10^4 batched requests 7.4 -> 6.4 ms).
+struct __align__(16) GmPow { uint64_t u, w; };
+constexpr int kGmDigits = kJumpBits / 8;
+
 template <int GEN>
-__device__ __forceinline__ void gm_apply(const uint64_t *M, uint64_t &zc, uint64_t &zp)
+__device__ __forceinline__ GmPow gm_pow_mul(const GmPow &a, const GmPow &b)
 {
     using P = GmT<GEN>;
-    uint64_t c = addmod_p<P::kind>(mulmod_p<P::kind>(M[0], zc), mulmod_p<P::kind>(M[1], zp));
-    uint64_t q = addmod_p<P::kind>(mulmod_p<P::kind>(M[2], zc), mulmod_p<P::kind>(M[3], zp));
-    zc = c; zp = q;
+    constexpr uint64_t k = P::k % P::p, q = P::p - P::q % P::p;
+    const uint64_t t = mulmod_p<P::kind>(a.w, b.w);
+    return { gm_lin<GEN>(a.u, b.u, q, t), addmod_p<P::kind>(gm_lin<GEN>(a.u, b.w, a.w, b.u), mulmod_p<P::kind>(k, t)) };
 }
 
-// Jump by the 128-bit exponent (hi, lo), and by a third word w2 (bits 128..191).
 template <int GEN>
-__device__ __forceinline__ void gm_jump128(const uint64_t *tab, uint64_t lo, uint64_t hi, uint64_t &zc, uint64_t &zp,
-                                           uint64_t w2 = 0)
+__global__ void gm_table_kernel(uint64_t *tab)
+{
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    GmPow x = { 0, 1 };
+#pragma unroll 1
+    for (int b = 0; b < kJumpBits; ++b) {
+        reinterpret_cast<GmPow *>(tab)[b] = x;
+        x = gm_pow_mul<GEN>(x, x);
+    }
+}
+// One block of 256 threads per byte position.
+template <int GEN>
+__global__ void gm_window_kernel(uint64_t *tab)
+{
+    const GmPow *bit = reinterpret_cast<const GmPow *>(tab) + 8 * blockIdx.x;
+    GmPow r = { 1, 0 };
+#pragma unroll 1
+    for (int b = 0; b < 8; ++b)
+        if ((threadIdx.x >> b) & 1u) r = gm_pow_mul<GEN>(r, bit[b]);
+    reinterpret_cast<GmPow *>(tab)[kJumpBits + 256 * blockIdx.x + threadIdx.x] = r;
+}
+
+// x^(d 2^(8 i)), d the low byte.
+__device__ __forceinline__ GmPow gm_digit(const uint64_t *tab, int i, uint32_t d)
+{
+    return reinterpret_cast<const GmPow *>(tab)[kJumpBits + 256 * i + (d & 255u)];
+}
+
+// r x^(e 2^(64 at)), one product per nonzero byte of e (each thread its own e).
+template <int GEN>
+__device__ __forceinline__ void gm_pow_word(const uint64_t *tab, int at, uint64_t e, GmPow &r)
 {
 #pragma unroll 1
-    for (int b = 0; b < 64; ++b)
-        if ((lo >> b) & 1u) gm_apply<GEN>(tab + 4 * b, zc, zp);
-#pragma unroll 1
-    for (int b = 0; b < 64; ++b)
-        if ((hi >> b) & 1u) gm_apply<GEN>(tab + 4 * (64 + b), zc, zp);
-#pragma unroll 1
-    for (int b = 0; w2 && b < 64; ++b)
-        if ((w2 >> b) & 1u) gm_apply<GEN>(tab + 4 * (128 + b), zc, zp);
+    for (int i = 8 * at; e; ++i, e >>= 8)
+        if (e & 255u) r = gm_pow_mul<GEN>(r, gm_digit(tab, i, (uint32_t)e));
+}
+template <int GEN>
+__device__ __forceinline__ GmPow gm_pow128(const uint64_t *tab, uint64_t lo, uint64_t hi)
+{
+    GmPow r = { 1, 0 };
+    gm_pow_word<GEN>(tab, 0, lo, r);
+    gm_pow_word<GEN>(tab, 1, hi, r);
+    return r;
 }
 
-// R = A B (2x2, row-major, mod p).
+// The product of a value per lane over groups of G lanes, in every lane.
+template <int GEN, int G>
+__device__ __forceinline__ GmPow gm_pow_reduce(GmPow r)
+{
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        const GmPow other = { __shfl_xor_sync(kFull, r.u, o), __shfl_xor_sync(kFull, r.w, o) };
+        r = gm_pow_mul<GEN>(r, other);
+    }
+    return r;
+}
+// x^(lo + 2^64 hi) by groups of 8 lanes with an exponent of their own (WIDE: hi may be
+// nonzero), or by the whole warp (then in groups of 16 lanes, one byte each).  Four
+// products one after another, three for 64 bits by 8 lanes, where a lane alone would
+// take one per byte; every lane of the warp takes part.
+template <int GEN, int LANES, bool WIDE>
+__device__ __forceinline__ GmPow gm_pow_group(const uint64_t *tab, uint64_t lo, uint64_t hi)
+{
+    const int l = threadIdx.x & 7;
+    if constexpr (LANES == 32 && WIDE) {
+        const bool up = threadIdx.x & 8;
+        return gm_pow_reduce<GEN, 16>(gm_digit(tab, up ? 8 + l : l, (uint32_t)((up ? hi : lo) >> (8 * l))));
+    } else {
+        GmPow r = gm_digit(tab, l, (uint32_t)(lo >> (8 * l)));
+        if constexpr (WIDE) r = gm_pow_mul<GEN>(r, gm_digit(tab, 8 + l, (uint32_t)(hi >> (8 * l))));
+        return gm_pow_reduce<GEN, 8>(r);
+    }
+}
+
+// (z^(n), z^(n-1)) advanced by the power r.
 template <int GEN>
-__device__ __forceinline__ void gm_mat_mul(uint64_t R[4], const uint64_t A[4], const uint64_t *B)
+__device__ __forceinline__ void gm_apply(const GmPow &r, uint64_t &zc, uint64_t &zp)
 {
     using P = GmT<GEN>;
-    const uint64_t r0 = addmod_p<P::kind>(mulmod_p<P::kind>(A[0], B[0]), mulmod_p<P::kind>(A[1], B[2]));
-    const uint64_t r1 = addmod_p<P::kind>(mulmod_p<P::kind>(A[0], B[1]), mulmod_p<P::kind>(A[1], B[3]));
-    const uint64_t r2 = addmod_p<P::kind>(mulmod_p<P::kind>(A[2], B[0]), mulmod_p<P::kind>(A[3], B[2]));
-    const uint64_t r3 = addmod_p<P::kind>(mulmod_p<P::kind>(A[2], B[1]), mulmod_p<P::kind>(A[3], B[3]));
-    R[0] = r0; R[1] = r1; R[2] = r2; R[3] = r3;
-}
-
-// M^e mod p for the exponent (hi, lo) from the table (M^(2^b) for each set
-// bit; powers of one matrix commute, so the order of the products is free).
-template <int GEN>
-__device__ __forceinline__ void gm_matpow128(const uint64_t *tab, uint64_t lo, uint64_t hi, uint64_t R[4])
-{
-    R[0] = 1; R[1] = 0; R[2] = 0; R[3] = 1;
-#pragma unroll 1
-    for (int b = 0; b < 64; ++b)
-        if ((lo >> b) & 1u) gm_mat_mul<GEN>(R, R, tab + 4 * b);
-#pragma unroll 1
-    for (int b = 0; hi && b < 64; ++b)
-        if ((hi >> b) & 1u) gm_mat_mul<GEN>(R, R, tab + 4 * (64 + b));
+    constexpr uint64_t k = P::k % P::p, q = P::p - P::q % P::p;
+    const uint64_t zn = gm_lin<GEN>(k, zc, q, zp);
+    zp = gm_lin<GEN>(r.w, zc, r.u, zp);
+    zc = gm_lin<GEN>(r.w, zn, r.u, zc);
 }
 
 __device__ __forceinline__ void mul64x64(uint64_t a, uint64_t b, uint64_t &lo, uint64_t &hi)
@@ -382,48 +432,65 @@ __global__ void gm_seed_kernel(const uint64_t *tab, uint64_t *base, uint64_t see
     uint64_t elo, ehi;
     mul64x64(dlo, (uint64_t)i, elo, ehi);
     ehi += dhi * (uint64_t)i;
-    gm_jump128<GEN>(tab, elo, ehi, zc, zp);
+    gm_apply<GEN>(gm_pow128<GEN>(tab, elo, ehi), zc, zp);
     base[i] = zp << P::t;          // x^(n-1)
     base[P::s + i] = zc << P::t;   // x^(n)
 }
 
 // Stream j of the handle = base advanced by (first + j) * L, L of 128 bits (the
-// exponent, of up to 192 bits, is exact).  One thread per point of a stream.
+// exponent, of up to 192 bits, is exact).  A block takes one stream per thread: the
+// thread forms its stream's power, then the block applies the powers to the streams'
+// points, in the order of the state, so that the stores are whole lines.  (A thread per
+// point with its own chain of bits: 10^6 streams of GQ58.3 4.8 ms, now 0.2.)
+constexpr int kGmInitThreads = 128;
+
 template <int GEN>
-__global__ void gm_init_kernel(const uint64_t *tab, const uint64_t *base, uint64_t *state, uint64_t first, uint64_t n,
-                               uint64_t llo, uint64_t lhi)
+__global__ void __launch_bounds__(kGmInitThreads) gm_init_kernel(const uint64_t *tab, const uint64_t *base, uint64_t *state,
+                                                                 uint64_t first, uint64_t n, uint64_t llo, uint64_t lhi)
 {
     using P = GmT<GEN>;
-    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t g = tid / P::s;
-    const int i = (int)(tid % P::s);
-    if (g >= n) return;
-    uint64_t zp = base[i] >> P::t, zc = base[P::s + i] >> P::t;
-    const uint64_t k = first + g;
-    uint64_t e0, c0, e1, c1;
-    mul64x64(k, llo, e0, c0);
-    mul64x64(k, lhi, e1, c1);
-    e1 += c0;
-    const uint64_t e2 = c1 + (e1 < c0 ? 1u : 0u);
-    gm_jump128<GEN>(tab, e0, e1, zc, zp, e2);
-    state[g * P::s + i] = zp << P::t;
-    state[(n + g) * P::s + i] = zc << P::t;
+    __shared__ GmPow pow[kGmInitThreads];
+    __shared__ uint64_t zp_s[P::s], zc_s[P::s];
+    const uint64_t g0 = (uint64_t)blockIdx.x * kGmInitThreads;
+    const int streams = (int)min((uint64_t)kGmInitThreads, n - g0);
+    if (threadIdx.x < P::s) {
+        zp_s[threadIdx.x] = base[threadIdx.x] >> P::t;
+        zc_s[threadIdx.x] = base[P::s + threadIdx.x] >> P::t;
+    }
+    if ((int)threadIdx.x < streams) {
+        const uint64_t k = first + g0 + threadIdx.x;
+        uint64_t e0, c0, e1, c1;
+        mul64x64(k, llo, e0, c0);
+        mul64x64(k, lhi, e1, c1);
+        e1 += c0;
+        const uint64_t e2 = c1 + (e1 < c0 ? 1u : 0u);
+        GmPow r = gm_pow128<GEN>(tab, e0, e1);
+        gm_pow_word<GEN>(tab, 2, e2, r);
+        pow[threadIdx.x] = r;
+    }
+    __syncthreads();
+    for (int at = threadIdx.x; at < streams * P::s; at += kGmInitThreads) {
+        uint64_t zp = zp_s[at % P::s], zc = zc_s[at % P::s];
+        gm_apply<GEN>(pow[at / P::s], zc, zp);
+        state[g0 * P::s + at] = zp << P::t;
+        state[(n + g0) * P::s + at] = zc << P::t;
+    }
 }
 
+// Every stream advanced by off: each warp forms the power, a byte per lane.
 template <int GEN>
 __global__ void gm_skip_kernel(const uint64_t *tab, uint64_t *state, uint64_t n, U256 off)
 {
     using P = GmT<GEN>;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t g = tid / P::s;
-    const int i = (int)(tid % P::s);
-    if (g >= n) return;
-    uint64_t zp = state[g * P::s + i] >> P::t, zc = state[(n + g) * P::s + i] >> P::t;
-#pragma unroll 1
-    for (int b = 0; b < kJumpBits; ++b)
-        if (u256_bit(off, b)) gm_apply<GEN>(tab + 4 * b, zc, zp);
-    state[g * P::s + i] = zp << P::t;
-    state[(n + g) * P::s + i] = zc << P::t;
+    const int lane = threadIdx.x & 31;
+    const uint64_t word = lane < 8 ? off.w[0] : lane < 16 ? off.w[1] : lane < 24 ? off.w[2] : off.w[3];
+    const GmPow r = gm_pow_reduce<GEN, 32>(gm_digit(tab, lane, (uint32_t)(word >> (8 * (lane & 7)))));
+    if (tid >= n * P::s) return;
+    uint64_t zp = state[tid] >> P::t, zc = state[n * P::s + tid] >> P::t;
+    gm_apply<GEN>(r, zc, zp);
+    state[tid] = zp << P::t;
+    state[n * P::s + tid] = zc << P::t;
 }
 
 // ----------------------------------------------------------------- generation
@@ -535,7 +602,7 @@ __global__ void __launch_bounds__(256, gm_blocks_per_sm<GEN>()) gm_gen_kernel(co
     const uint64_t len = min(seclen, nper - start);
     uint64_t zp = state_in[j * P::s + li] >> P::t;
     uint64_t zc = state_in[(stride + j) * P::s + li] >> P::t;
-    if (start) gm_jump128<GEN>(tab, start, 0, zc, zp);
+    if (start) gm_apply<GEN>(gm_pow_group<GEN, 32, false>(tab, start, 0), zc, zp);  // (uniform over the warp)
     gm_generate_section<GEN, OutT, VEC>(zc, zp, li, out + j * nper + start, len, slots + 4 * threadIdx.x);
     if (start + len == nper) {
         state_out[j * P::s + li] = zp << P::t;
@@ -567,7 +634,7 @@ __device__ __forceinline__ uint32_t gmt_next_word(GmZ<GEN> *zc, GmZ<GEN> *zp)
 }
 
 // Load one stream's points (x >> t) from xp, xc and advance them by the
-// exponent (hi, lo) with one matrix M^e applied to every point; canonical
+// exponent (hi, lo) with one power applied to every point; canonical
 // residues in and out.
 template <int GEN>
 __device__ __forceinline__ void gmt_load(const uint64_t *tab, const uint64_t *xp, const uint64_t *xc, uint64_t lo,
@@ -578,10 +645,9 @@ __device__ __forceinline__ void gmt_load(const uint64_t *tab, const uint64_t *xp
 #pragma unroll
     for (int i = 0; i < P::s; ++i) { q[i] = xp[i] >> P::t; c[i] = xc[i] >> P::t; }
     if (lo | hi) {
-        uint64_t M[4];
-        gm_matpow128<GEN>(tab, lo, hi, M);
+        const GmPow r = gm_pow128<GEN>(tab, lo, hi);
 #pragma unroll
-        for (int i = 0; i < P::s; ++i) gm_apply<GEN>(M, c[i], q[i]);
+        for (int i = 0; i < P::s; ++i) gm_apply<GEN>(r, c[i], q[i]);
     }
 #pragma unroll
     for (int i = 0; i < P::s; ++i) { zc[i] = (GmZ<GEN>)c[i]; zp[i] = (GmZ<GEN>)q[i]; }

@@ -157,20 +157,6 @@ __device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32])
 }
 
 // ------------------------------------------------------------------ pieces
-// a x + b y (mod p), canonical; every operand <= p.
-template <int GEN>
-__device__ __forceinline__ uint64_t tc_lin(uint64_t a, uint64_t x, uint64_t b, uint64_t y)
-{
-    constexpr int K = GmT<GEN>::kind;
-    if constexpr (K == P51 || K == P61) {
-        const uint64_t l0 = a * x, l1 = b * y, lo = l0 + l1;
-        const uint64_t hi = __umul64hi(a, x) + __umul64hi(b, y) + (lo < l0 ? 1u : 0u);
-        return reduce_prod<K>(lo, hi);
-    } else {
-        return reduce_prod<K>((uint64_t)(uint32_t)a * (uint32_t)x + (uint64_t)(uint32_t)b * (uint32_t)y, 0);
-    }
-}
-
 // A value as the block recurrence takes it: for the 51- and 61-bit primes split at
 // bit 26 or 31, where every sum of partial products fits 64 bits (at bit 32 the
 // low one would not).  Lazy residues: below p + 8 (p + 2^18 for GM55).
@@ -354,7 +340,7 @@ __device__ __noinline__ uint4 tc_exact_half(const uint64_t *al_s, const uint64_t
         TcValue<GEN> a, b;
         a.lo = __shfl_sync(kFull, v1.lo, l); a.hi = __shfl_sync(kFull, v1.hi, l);
         b.lo = __shfl_sync(kFull, v2.lo, l); b.hi = __shfl_sync(kFull, v2.hi, l);
-        const uint64_t x = tc_lin<GEN>(al, a.whole(), be, b.whole());
+        const uint64_t x = gm_lin<GEN>(al, a.whole(), be, b.whole());
         uint4 r = make_uint4(0, 0, 0, 0);
         if constexpr (P::v == 1) {
             r.x = __ballot_sync(kFull, x >= (P::p + 1) / 2);
@@ -442,7 +428,7 @@ struct TcFill {
     }
     __device__ __forceinline__ void advance(const uint64_t *jump, const Section &s, uint64_t &zc, uint64_t &zp) const
     {
-        if (s.start && s.len) gm_jump128<GEN>(jump, s.start, 0, zc, zp);
+        if (units != nstreams) gm_apply<GEN>(gm_pow_group<GEN, S, false>(jump, s.start, 0), zc, zp);
     }
     __device__ __forceinline__ unsigned char *row(const Section &s) const
     {
@@ -500,7 +486,7 @@ struct TcBatch {
     }
     __device__ __forceinline__ void advance(const uint64_t *jump, const Section &s, uint64_t &zc, uint64_t &zp) const
     {
-        if (s.len) gm_jump128<GEN>(jump, s.lo, s.hi, zc, zp);
+        gm_apply<GEN>(gm_pow_group<GEN, S, true>(jump, s.lo, s.hi), zc, zp);
     }
     __device__ __forceinline__ unsigned char *row(const Section &s) const { return s.out; }
     __device__ __forceinline__ int form(const Section &s) const { return s.form; }
@@ -579,7 +565,7 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
         uint64_t zp = reduce_prod<P::kind>(zm >> P::t, 0);
         zc = reduce_prod<P::kind>(zc >> P::t, 0);
         src.advance(jump, sec, zc, zp);
-        zm = tc_lin<GEN>(to_a, zc, to_b, zp);
+        zm = gm_lin<GEN>(to_a, zc, to_b, zp);
     };
 
     const uint32_t tiles = src.tiles();
@@ -710,8 +696,8 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
         }
         if (Src::kNextState && ends && left == 0) {
             // the stream ends here for this fill: x^(n + words - 1), x^(n + words)
-            src.next_state(sec, li, tc_lin<GEN>(al_s[words], x1.whole(), be_s[words], z2),
-                           tc_lin<GEN>(al_s[words + 1], x1.whole(), be_s[words + 1], z2));
+            src.next_state(sec, li, gm_lin<GEN>(al_s[words], x1.whole(), be_s[words], z2),
+                           gm_lin<GEN>(al_s[words + 1], x1.whole(), be_s[words + 1], z2));
             ends = false;
         }
         if constexpr (LAST) {

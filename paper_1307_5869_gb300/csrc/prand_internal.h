@@ -116,7 +116,7 @@ struct DevTables {
     int device = -1;
     uint32_t *mrg = nullptr;      // [kJumpBits][18]: A^(2^b) mod m1 (9 words), B^(2^b) mod m2 (9 words)
     uint32_t *lfsr = nullptr;     // [4][kJumpBits][32]: column images of T_c^(2^b)
-    uint64_t *gm[8] = {};         // per GM/GQ generator: [kJumpBits][4] = M^(2^b) mod p
+    uint64_t *gm[8] = {};         // per GM/GQ generator: powers of its step, by bits and by bytes (gm_impl.cuh)
     struct GmTcTable *gm_tc[8] = {};      // the tensor-core generation's constants (null: not used by the generator)
     volatile uint32_t *wait_failed = nullptr;  // mapped host memory: set by a kernel whose bounded wait ran out
     uint32_t *mt = nullptr;       // [kMtPolyCount][kMtPolyWords]: x^(2^b) mod phi
