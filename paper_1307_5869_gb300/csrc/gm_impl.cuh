@@ -664,6 +664,39 @@ __device__ __forceinline__ void gmt_store(const GmZ<GEN> *zc, const GmZ<GEN> *zp
     }
 }
 
+// The states of a warp's 32 consecutive streams (rows of them exist), through shared
+// memory so that global memory sees whole lines: a stream's points are 64 or 96 bytes
+// apart, and a thread reading its own touches every line of the warp at every load.
+// tile: 32 rows of an odd number of words each, so the lanes' rows meet no bank conflicts.
+template <int GEN>
+__device__ __forceinline__ void gmt_stage_in(const uint64_t *from, int rows, uint64_t *tile, int lane, uint64_t *v)
+{
+    constexpr int S = GmT<GEN>::s, PITCH = S | 1;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+        const int at = 32 * i + lane;
+        if (at < rows * S) tile[at / S * PITCH + at % S] = from[at];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < S; ++i) v[i] = lane < rows ? tile[lane * PITCH + i] : 0;
+    __syncwarp();
+}
+template <int GEN>
+__device__ __forceinline__ void gmt_stage_out(const uint64_t *v, int rows, uint64_t *tile, int lane, uint64_t *to)
+{
+    constexpr int S = GmT<GEN>::s, PITCH = S | 1;
+#pragma unroll
+    for (int i = 0; i < S; ++i) tile[lane * PITCH + i] = v[i];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+        const int at = 32 * i + lane;
+        if (at < rows * S) to[at] = tile[at / S * PITCH + at % S];
+    }
+    __syncwarp();
+}
+
 // One thread = one section of one stream (sections reached by M^start).
 // ROWS: every row start is 16-byte aligned, so rows leave through the staged
 // 128-byte row stores (every lane of a warp takes part); else one store per
@@ -681,8 +714,24 @@ __global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict
     const uint64_t j = live ? tid % nstreams : 0;
     const uint64_t start = live ? (tid / nstreams) * seclen : 0;
     const uint64_t len = (live && start < nper) ? min(seclen, nper - start) : 0;
+    __shared__ __align__(16) unsigned char tiles[256 / 32][kTileBytes];
+    static_assert(32 * (P::s | 1) * 8 <= kTileBytes, "a warp's states fit its tile");
+    const int lane = threadIdx.x & 31;
+    uint64_t *const tile = reinterpret_cast<uint64_t *>(tiles[threadIdx.x >> 5]);
+    // whole streams: the warp's states are one run of memory (2^22 streams of GQ58.3, one
+    // output each: 482 us for a thread's own loads and stores, 305 through the tile, of
+    // which 240 for the bytes; 2^16 streams of 4096: 1637 and 1474 us)
+    const uint64_t j0 = tid - lane;
+    const int rows = nsec == 1 ? (int)min((uint64_t)32, nstreams > j0 ? nstreams - j0 : 0) : 0;
     Z zc[P::s], zp[P::s];
-    if (len) {
+    if (nsec == 1) {
+        if (!rows) return;  // whole warp
+        uint64_t q[P::s], c[P::s];
+        gmt_stage_in<GEN>(state_in + j0 * P::s, rows, tile, lane, q);
+        gmt_stage_in<GEN>(state_in + (stride + j0) * P::s, rows, tile, lane, c);
+#pragma unroll
+        for (int i = 0; i < P::s; ++i) { zp[i] = (Z)(q[i] >> P::t); zc[i] = (Z)(c[i] >> P::t); }
+    } else if (len) {
         gmt_load<GEN>(tab, state_in + j * P::s, state_in + (stride + j) * P::s, start, 0, zc, zp);
     } else {
 #pragma unroll
@@ -691,14 +740,21 @@ __global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict
     }
     OutT *o = out + j * nper + start;
     if constexpr (ROWS) {
-        __shared__ __align__(16) unsigned char tiles[256 / 32][kTileBytes];
         fill_rows<OutT, 128, true>([&]() { return gmt_next_word<GEN>(zc, zp); },
-                                   [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len, tiles[threadIdx.x >> 5],
-                                   threadIdx.x & 31);
+                                   [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len, tiles[threadIdx.x >> 5], lane);
     } else {
         for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(gmt_next_word<GEN>(zc, zp));
     }
-    if (len && start + len == nper) gmt_store<GEN>(zc, zp, state_out + j * P::s, state_out + (stride + j) * P::s);
+    if (nsec == 1) {
+        __syncwarp();
+        uint64_t q[P::s], c[P::s];
+#pragma unroll
+        for (int i = 0; i < P::s; ++i) { q[i] = gm_canon<GEN>(zp[i]) << P::t; c[i] = gm_canon<GEN>(zc[i]) << P::t; }
+        gmt_stage_out<GEN>(q, rows, tile, lane, state_out + j0 * P::s);
+        gmt_stage_out<GEN>(c, rows, tile, lane, state_out + (stride + j0) * P::s);
+    } else if (len && start + len == nper) {
+        gmt_store<GEN>(zc, zp, state_out + j * P::s, state_out + (stride + j) * P::s);
+    }
 }
 
 }  // namespace prand
