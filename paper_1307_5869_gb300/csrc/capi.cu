@@ -445,11 +445,20 @@ static prand_status_t init_layout(prand_handle_t h, int32_t layout, uint64_t fir
         h->base_variant = base_variant;
     }
     h->variant = layout;
-    free_states(h);
+    // as many streams as the handle has: its buffers serve again, after the wait for the
+    // device that freeing them would be (2^22 streams of GQ58.3, 1.6 GB: freeing and
+    // allocating 1.4 ms of an opening of 1.7)
+    const bool keep = h->d_state && h->n == n_streams;
+    if (keep) {
+        if (cudaDeviceSynchronize() != cudaSuccess) { free_states(h); return PRAND_ERR_CUDA; }
+        h->n = 0;
+    } else {
+        free_states(h);
+    }
     uint64_t bytes;
     if (mul_overflows(n_streams, state_bytes_per_stream(h->gen), &bytes)) return PRAND_ERR_ARG;
-    if (!dev_alloc(&h->d_state, bytes)) { h->d_state = nullptr; return PRAND_ERR_NOMEM; }
-    if (h->gen != PRAND_MT19937 && !dev_alloc(&h->d_spare, bytes)) {
+    if (!h->d_state && !dev_alloc(&h->d_state, bytes)) { h->d_state = nullptr; return PRAND_ERR_NOMEM; }
+    if (!h->d_spare && h->gen != PRAND_MT19937 && !dev_alloc(&h->d_spare, bytes)) {
         h->d_spare = nullptr;
         free_states(h);
         return PRAND_ERR_NOMEM;
