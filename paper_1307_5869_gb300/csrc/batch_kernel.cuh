@@ -157,8 +157,8 @@ __device__ __forceinline__ void batch_gm(const BatchTile &T, const BatchCtx &C, 
 }
 
 // ------------------------------------------------------------------ MT19937 tiles
-// One tile = one request, run by a whole block of kMtTeam warps: it applies the jump
-// polynomials (mt_jump_block), then makes the outputs.  Slot layout: 624 words of the
+// One tile = one request, run by a whole block of kMtTeam warps, or by a cluster of CS of
+// them: it applies the jump polynomials (mt_jump_block), then makes the outputs.  Slot layout: 624 words of the
 // current block, then the index inside it.
 //
 // The outputs: b0 holds the current block, idx the position inside it.  Each further
@@ -198,7 +198,7 @@ __device__ __forceinline__ void batch_mt_emit_team(const BatchTile &T, const Bat
     __threadfence();
 }
 
-template <typename OutT>
+template <typename OutT, int CS>
 __device__ __forceinline__ void batch_mt(const BatchTile &T, const BatchCtx &C, MtJumpSmem &S)
 {
     uint32_t *b0 = S.x[0], *b1 = S.x[0] + kMtN;  // the outputs' two blocks
@@ -213,9 +213,10 @@ __device__ __forceinline__ void batch_mt(const BatchTile &T, const BatchCtx &C, 
         // stream k = base advanced by k 2^432: one polynomial per nonzero byte of k
         for (int i = 0; i < kMtWinPositions; ++i) {
             const uint32_t d = (uint32_t)(T.stream >> (kMtWinBits * i)) & (uint32_t)(kMtWinDigits - 1);
-            if (d) mt_jump_block<kMtTeam>(S, C.mt_win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords);
+            if (d) mt_jump_block<kMtTeam, CS>(S, C.mt_win + ((size_t)i * kMtWinDigits + d) * kMtPolyWords);
         }
     }
+    if (mt_cluster_rank<CS>() != 0) return;  // (whole block) one block makes the outputs
     // (a thread reads back the words it wrote, or those a jump's last barrier published)
     for (int i = threadIdx.x; i < kMtN; i += 32 * kMtTeam) b0[i] = S.state[i];
     batch_mt_emit_team<OutT>(T, C, b0, b1, idx);
@@ -271,9 +272,9 @@ __device__ __forceinline__ void batch_tile_done(const BatchTile &T, const BatchC
 // allow (the rest: 40 warps per SM at 48 registers; thread-per-stream GM/GQ:
 // 16 warps at 128; MT19937: whatever its jump chains need).  ROWB: the staged
 // row size of the thread-per-section tiles (MRG32K3A, LFSR113).  The MT19937
-// build claims tiles per block (a team of BS / 32 warps per tile), the others
+// build claims tiles per block or cluster (teams of BS / 32 warps), the others
 // per warp.
-template <int MODE, int BS, int ROWB>
+template <int MODE, int BS, int ROWB, int CS = 1>
 __global__ void __launch_bounds__(BS, (MODE == kModeRest ? 1280 / BS : MODE == kModeWide ? 512 / BS : 1536 / BS)) batch_kernel(
     const BatchTile *__restrict__ tiles, uint32_t ntiles, uint32_t *counter, BatchCtx ctx)
 {
@@ -282,17 +283,17 @@ __global__ void __launch_bounds__(BS, (MODE == kModeRest ? 1280 / BS : MODE == k
         __shared__ __align__(16) MtJumpSmem S;
         __shared__ uint32_t claimed;
         for (;;) {
-            if (threadIdx.x == 0) claimed = atomicAdd(counter, 1u);
-            __syncthreads();
-            const uint32_t t = claimed;
-            __syncthreads();
+            if (threadIdx.x == 0 && mt_cluster_rank<CS>() == 0) claimed = atomicAdd(counter, 1u);
+            mt_cluster_sync<CS>();
+            const uint32_t t = mt_cluster_word<CS>(&claimed, 0);
+            mt_cluster_sync<CS>();
             if (t >= ntiles) return;
             const BatchTile T = tiles[t];
-            if (T.dtype == PRAND_DTYPE_U32) batch_mt<uint32_t>(T, ctx, S);
-            else if (T.dtype == PRAND_DTYPE_F32) batch_mt<float>(T, ctx, S);
-            else batch_mt<double>(T, ctx, S);
+            if (T.dtype == PRAND_DTYPE_U32) batch_mt<uint32_t, CS>(T, ctx, S);
+            else if (T.dtype == PRAND_DTYPE_F32) batch_mt<float, CS>(T, ctx, S);
+            else batch_mt<double, CS>(T, ctx, S);
             __syncthreads();
-            if (threadIdx.x == 0) batch_tile_done(T, ctx);
+            if (threadIdx.x == 0 && mt_cluster_rank<CS>() == 0) batch_tile_done(T, ctx);
         }
     } else {
         __shared__ __align__(16) unsigned char smem[BS / 32][WarpSmem<ROWB>::bytes];

@@ -96,41 +96,56 @@ __global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_gen_kernel(uint32_t 
 
 // ------------------------------------------------------------------ jump
 // Blocks of 12 warps, four to an SM (40 registers): one wave holds 608 streams, and 65536
-// streams take 18.2 ms (6 warps 18.1, 3 warps 21.5, 15 warps 19.7, 30 warps 28.0) with the
-// small levels, which are latency, at 55 us each (6 warps 100, 3 warps 200, 30 warps 33).
-// The first stream of a handle is alone on the chip, in a chain of one jump per set bit:
-// 30 warps (0.60 ms for a chain of eight; 12 warps 0.80).
-constexpr int kMtLevelWarps = 12, kMtMultiWarps = 30;
+// streams take 17.4 ms (before the rounds of the next step's words were three instead of
+// four: 18.2; 6 warps 18.1, 3 warps 21.5, 15 warps 19.7, 30 warps 28.0).  Few streams are
+// latency, so each takes a cluster of blocks (kMtCluster): the first stream of a
+// handle, a chain of one jump per set bit, 0.22 ms for nine jumps (one block 0.80,
+// clusters of four 0.30; 15 or 30 warps a block the same), a level of up to 16 streams
+// 26 us (90).
+constexpr int kMtJumpWarps = 12;
 
-// Doubling level: dst stream (off + j) := g(A) (src stream j), one block per stream.
-__global__ void __launch_bounds__(32 * kMtLevelWarps, 4) mt_level_kernel(const uint32_t *poly, uint32_t *state, uint64_t off)
+// Doubling level: dst stream (off + j) := g(A) (src stream j), one block or cluster per stream.
+template <int NW, int MB, int CS>
+__global__ void __launch_bounds__(32 * NW, MB) mt_level_kernel(const uint32_t *poly, uint32_t *state, uint64_t off)
 {
     __shared__ __align__(16) MtJumpSmem S;
-    const uint64_t j = blockIdx.x;
-    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) S.state[i] = state[j * kMtN + i];
-    mt_jump_block<kMtLevelWarps>(S, poly);
-    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) state[(off + j) * kMtN + i] = S.state[i];
+    const uint64_t j = blockIdx.x / CS;
+    for (int i = threadIdx.x; i < kMtN; i += 32 * NW) S.state[i] = state[j * kMtN + i];
+    mt_jump_block<NW, CS>(S, poly);
+    if (mt_cluster_rank<CS>() == 0)
+        for (int i = threadIdx.x; i < kMtN; i += 32 * NW) state[(off + j) * kMtN + i] = S.state[i];
 }
 
 // Every stream advanced by the set bits of a 512-bit offset (one polynomial
-// x^(2^b) mod phi per set bit b, applied one after another), one block per stream.
+// x^(2^b) mod phi per set bit b, applied one after another), one block or cluster per stream.
 struct MtBits { uint64_t w[8]; };
 
-template <int NW, int MB>
+template <int NW, int MB, int CS>
 __global__ void __launch_bounds__(32 * NW, MB) mt_multi_kernel(const uint32_t *polys, uint32_t *state, MtBits e)
 {
     __shared__ __align__(16) MtJumpSmem S;
-    uint32_t *s = state + (uint64_t)blockIdx.x * kMtN;
-    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) S.state[i] = s[i];
-    for (int b = 0; b < 512; ++b) {
-        if (!((e.w[b >> 6] >> (b & 63)) & 1u)) continue;
-        mt_jump_block<NW>(S, polys + (size_t)b * kMtPolyWords);
-    }
-    for (int i = threadIdx.x; i < kMtN; i += blockDim.x) s[i] = S.state[i];
+    uint32_t *s = state + (uint64_t)(blockIdx.x / CS) * kMtN;
+    for (int i = threadIdx.x; i < kMtN; i += 32 * NW) S.state[i] = s[i];
+    for (int b = 0; b < 512; ++b)
+        if ((e.w[b >> 6] >> (b & 63)) & 1u) mt_jump_block<NW, CS>(S, polys + (size_t)b * kMtPolyWords);
+    // (every block of a cluster has read the state before the first jump's barrier)
+    if (mt_cluster_rank<CS>() == 0)
+        for (int i = threadIdx.x; i < kMtN; i += 32 * NW) s[i] = S.state[i];
 }
 
 // ------------------------------------------------------------------ host
 static unsigned grid_warps(uint64_t n) { return (unsigned)((n + kMtWarpsPerBlock - 1) / kMtWarpsPerBlock); }
+
+// One block per stream, or a cluster of them when every block then has an SM to itself.
+template <typename... Args>
+static prand_status_t mt_jump_launch(void (*block)(Args...), void (*cluster)(Args...), uint64_t n, cudaStream_t st, Args... args)
+{
+    if (n * kMtCluster > (uint64_t)device_sm_count()) {
+        block<<<(unsigned)n, 32 * kMtJumpWarps, 0, st>>>(args...);
+        return launch_check();
+    }
+    return mt_cluster_launch(cluster, (unsigned)n * kMtCluster, 32 * kMtJumpWarps, kMtCluster, st, args...);
+}
 
 prand_status_t mt_seed(uint64_t seed, void *d_base, cudaStream_t st)
 {
@@ -152,15 +167,14 @@ prand_status_t mt_init(const DevTables *T, const void *d_base, void *d_state, ui
         // first * 2^shift: bits shift .. shift + 63
         for (int b = 0; b < 64; ++b)
             if ((first >> b) & 1u) e.w[(shift + b) >> 6] |= 1ull << ((shift + b) & 63);
-        mt_multi_kernel<kMtMultiWarps, 1><<<1, 32 * kMtMultiWarps, 0, st>>>(T->mt, state, e);
-        prand_status_t s = launch_check();
+        prand_status_t s = mt_jump_launch(mt_multi_kernel<kMtJumpWarps, 4, 1>, mt_multi_kernel<kMtJumpWarps, 1, kMtCluster>, 1, st, (const uint32_t *)T->mt, state, e);
         if (s != PRAND_OK) return s;
     }
     for (int b = 0; b < 64 && (1ull << b) < n; ++b) {
         uint64_t have = 1ull << b;
         uint64_t count = min(have, n - have);
-        mt_level_kernel<<<(unsigned)count, 32 * kMtLevelWarps, 0, st>>>(T->mt + (size_t)(shift + b) * kMtPolyWords, state, have);
-        prand_status_t s = launch_check();
+        prand_status_t s = mt_jump_launch(mt_level_kernel<kMtJumpWarps, 4, 1>, mt_level_kernel<kMtJumpWarps, 1, kMtCluster>, count, st,
+                                          (const uint32_t *)T->mt + (size_t)(shift + b) * kMtPolyWords, state, have);
         if (s != PRAND_OK) return s;
     }
     return PRAND_OK;
@@ -191,8 +205,8 @@ prand_status_t mt_skip512(const DevTables *T, void *d_state, uint64_t n, uint32_
     bool any = false;
     for (int i = 0; i < 8; ++i) any = any || e.w[i];
     if (!any) return PRAND_OK;
-    mt_multi_kernel<kMtLevelWarps, 4><<<(unsigned)n, 32 * kMtLevelWarps, 0, st>>>(T->mt, (uint32_t *)d_state, e);
-    return launch_check();
+    return mt_jump_launch(mt_multi_kernel<kMtJumpWarps, 4, 1>, mt_multi_kernel<kMtJumpWarps, 1, kMtCluster>, n, st, (const uint32_t *)T->mt,
+                          (uint32_t *)d_state, e);
 }
 
 prand_status_t mt_skip(const DevTables *T, void *d_state, uint64_t n, uint32_t *idx, const U256 &off, cudaStream_t st)

@@ -135,13 +135,15 @@ __device__ __forceinline__ void mt_twist_emit(const uint32_t *__restrict__ ob, u
 //
 // Bound by instruction issue: 32 steps x 3 products x 80 groups per stream, each 12.5
 // logic operations (two-cycle ones: 5.4 ms of the ALU pipe for 32768 streams), two loads
-// and about 20 instructions of branches, uniform tests and moves.  32768 streams: 8.6 ms
+// and about 20 instructions of branches, uniform tests and moves.  32768 streams: 8.4 ms
 // (82 % of the issue slots), where one warp per stream over the unsplit sum, in groups of
-// two coefficients, took 12.7 ms; one stream alone 55 us with 12 warps, where that took
-// 670 us.  Groups of two coefficients 10.1 ms; a switch instead of the tree 8.7 ms;
-// branches the compiler does not know to be uniform 9.7 ms.
+// two coefficients, took 12.7 ms; one stream alone 85 us with 12 warps and 24 us by a
+// cluster of eight blocks, where that took 670 us.  Groups of two coefficients 10.1 ms; a
+// switch instead of the tree 8.7 ms; branches the compiler does not know to be uniform
+// 9.7 ms.
 constexpr int kMtK = 320, kMtStep = 2 * kMtK, kMtSteps = (kMtDeg + kMtStep - 1) / kMtStep;  // 32 steps
 constexpr int kMtW = 10, kMtP = 16, kMtG = 4;
+constexpr int kMtCluster = 8;  // blocks per stream when the streams are few
 
 struct MtJumpSmem {
     uint32_t x[2][2 * kMtStep];       // x_{640 Q} .. x_{640 Q + 1279} of step Q, in buffer Q & 1
@@ -180,16 +182,53 @@ __device__ __forceinline__ void mt_poly_groups(uint32_t bits, const uint32_t *ru
     }
 }
 
-// All 32 NW threads call it; S.state holds the state before and after (a barrier at the
-// end publishes it).  poly: g's 624 coefficient words.  NW is a multiple of 3 whose
-// third divides the 20 chunks of a block of coefficients.
-template <int NW>
+// Barrier over the CS blocks of a cluster (the block alone for CS = 1), and a word of a
+// shared variable of one of its blocks.
+template <int CS>
+__device__ __forceinline__ void mt_cluster_sync()
+{
+    if constexpr (CS == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+template <int CS>
+__device__ __forceinline__ uint32_t mt_cluster_rank()
+{
+    uint32_t r = 0;
+    if constexpr (CS > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+template <int CS>
+__device__ __forceinline__ uint32_t mt_cluster_word(const uint32_t *p, uint32_t rank)
+{
+    if constexpr (CS == 1) {
+        return *p;
+    } else {
+        uint32_t at, v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+        return v;
+    }
+}
+
+// All 32 NW threads of the block call it, and of all CS blocks of the cluster: each takes
+// a run of the steps (making the words before it on its own), the parts are summed
+// through distributed shared memory, and every block ends with the new state.
+// S.state holds the state before and after (a barrier at the end publishes it).
+// poly: g's 624 coefficient words.  NW is a multiple of 3 whose third divides the 20
+// chunks of a block of coefficients.
+template <int NW, int CS = 1>
 __device__ __forceinline__ void mt_jump_block(MtJumpSmem &S, const uint32_t *__restrict__ poly)
 {
     constexpr int NT = 32 * NW, SHARE = kMtK / (NW / 3), ROUND = NT < 227 ? NT : 227;
     static_assert(NW % 3 == 0 && SHARE * (NW / 3) == kMtK && SHARE % kMtP == 0, "shares of whole chunks");
+    static_assert(kMtSteps % CS == 0, "whole steps per block");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int role = warp % 3, c0 = SHARE * (warp / 3);
+    const int q0 = kMtSteps / CS * (int)mt_cluster_rank<CS>(), q1 = q0 + kMtSteps / CS;
     __syncthreads();  // S.state written by the caller, or by the last jump
     for (int i = tid; i < kMtN; i += NT) S.x[0][i] = S.state[i];
     for (int i = tid; i < (int)(sizeof(S.poly) / 4); i += NT) S.poly[i] = i < kMtPolyWords ? poly[i] : 0u;
@@ -201,26 +240,39 @@ __device__ __forceinline__ void mt_jump_block(MtJumpSmem &S, const uint32_t *__r
             S.x[0][n] = mt_recur(S.x[0][n - kMtN], S.x[0][n - kMtN + 1], S.x[0][n - (kMtN - kMtM)]);
         __syncthreads();
     }
-    for (int i = tid; i < 3 * kMtK; i += NT) S.y[0][i] = S.x[0][i] ^ S.x[0][i + kMtK];
+    // the words of step Q + 1 from those of step Q (each other's buffer): the first 640 are
+    // step Q's last, and the first round of the others reads those where they are
+    auto advance = [&](int Q) {
+        const uint32_t *ob = S.x[Q & 1] + kMtStep;
+        uint32_t *nb = S.x[(Q & 1) ^ 1];
+        if (tid < ROUND) nb[kMtStep + tid] = mt_recur(ob[kMtStep - kMtN + tid], ob[kMtStep - kMtN + 1 + tid], ob[kMtStep - (kMtN - kMtM) + tid]);
+        for (int i = tid; i < kMtStep; i += NT) nb[i] = ob[i];
+        __syncthreads();
+#pragma unroll 1
+        for (int a = kMtStep + ROUND; a < 2 * kMtStep; a += ROUND) {
+            const int n = a + tid;
+            if (tid < ROUND && n < 2 * kMtStep) nb[n] = mt_recur(nb[n - kMtN], nb[n - kMtN + 1], nb[n - (kMtN - kMtM)]);
+            __syncthreads();
+        }
+    };
+    auto sums = [&](int b) {
+        for (int i = tid; i < 3 * kMtK; i += NT) S.y[b][i] = S.x[b][i] ^ S.x[b][i + kMtK];
+    };
+    if constexpr (CS > 1) {
+#pragma unroll 1
+        for (int Q = 0; Q < q0; ++Q) advance(Q);
+    }
+    sums(q0 & 1);
     uint32_t acc[kMtW], x[kMtP];
 #pragma unroll
     for (int j = 0; j < kMtW; ++j) acc[j] = 0;
 #pragma unroll 1
-    for (int Q = 0; Q < kMtSteps; ++Q) {
+    for (int Q = q0; Q < q1; ++Q) {
         const int b = Q & 1;
         __syncthreads();  // this step's words are written; buffer b ^ 1 is read no more
-        if (Q + 1 < kMtSteps) {
-            const uint32_t *ob = S.x[b];
-            uint32_t *nb = S.x[b ^ 1];
-            for (int i = tid; i < kMtStep; i += NT) nb[i] = ob[kMtStep + i];
-            __syncthreads();
-#pragma unroll 1
-            for (int a = kMtStep; a < 2 * kMtStep; a += ROUND) {
-                const int n = a + tid;
-                if (tid < ROUND && n < 2 * kMtStep) nb[n] = mt_recur(nb[n - kMtN], nb[n - kMtN + 1], nb[n - (kMtN - kMtM)]);
-                __syncthreads();
-            }
-            for (int i = tid; i < 3 * kMtK; i += NT) S.y[b ^ 1][i] = nb[i] ^ nb[i + kMtK];
+        if (Q + 1 < q1) {
+            advance(Q);
+            sums(b ^ 1);
         }
         // coefficients 640 Q + (320 for C) + c, c0 <= c < c1, none past the polynomial's end
         const int left = kMtDeg - (kMtStep * Q + (role == 2 ? kMtK : 0));
@@ -248,7 +300,37 @@ __device__ __forceinline__ void mt_jump_block(MtJumpSmem &S, const uint32_t *__r
         if (role != 2) atomicXor(&S.state[kMtW * lane + j], acc[j]);
         if (role != 1) atomicXor(&S.state[kMtK + kMtW * lane + j], acc[j]);
     }
-    __syncthreads();
+    mt_cluster_sync<CS>();
+    if constexpr (CS > 1) {
+        constexpr int R = (kMtN + NT - 1) / NT;
+        uint32_t sum[R] = {};
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (tid + NT * r < kMtN)
+                for (uint32_t k = 0; k < CS; ++k) sum[r] ^= mt_cluster_word<CS>(&S.state[tid + NT * r], k);
+        mt_cluster_sync<CS>();  // every block has read every part
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (tid + NT * r < kMtN) S.state[tid + NT * r] = sum[r];
+        __syncthreads();
+    }
+}
+
+// Launch of a kernel whose blocks are in clusters of CS.
+template <typename... Args>
+inline prand_status_t mt_cluster_launch(void (*kernel)(Args...), unsigned blocks, unsigned threads, unsigned cs, cudaStream_t st, Args... args)
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = cs;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(blocks);
+    c.blockDim = dim3(threads);
+    c.stream = st;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, args...) == cudaSuccess ? launch_check() : PRAND_ERR_CUDA;
 }
 
 }  // namespace prand
