@@ -31,12 +31,12 @@ __device__ __forceinline__ void batch_mrg(const BatchTile &T, const BatchCtx &C,
                                     : (const uint32_t *)C.base[PRAND_MRG32K3A];
     for (int i = 0; i < 3; ++i) { x[i] = src[i]; y[i] = src[3 + i]; }
     if (len) {
-        if (!from_slot)
-            for (int b = 0; b < 64; ++b)
-                if ((T.stream >> b) & 1u) mrg_apply_bit(C.mrg_tab, kMrgStreamShift + b, x, y);
-        const uint64_t s = T.start + off;
-        for (int b = 0; b < 64; ++b)
-            if ((s >> b) & 1u) mrg_apply_bit(C.mrg_tab, b, x, y);
+        static_assert(kMrgStreamShift == 127, "a stream is 2^127 steps: bits 127 on of the exponent");
+        if (!from_slot) {
+            mrg_apply_word(C.mrg_tab, 1, T.stream << 63, x, y);
+            mrg_apply_word(C.mrg_tab, 2, T.stream >> 1, x, y);
+        }
+        mrg_apply_word(C.mrg_tab, 0, T.start + off, x, y);
     }
     uint32_t x0 = x[0], x1 = x[1], x2 = x[2], y0 = y[0], y1 = y[1], y2 = y[2];
     OutT *o = (OutT *)T.out + off;

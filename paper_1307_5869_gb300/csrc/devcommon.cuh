@@ -228,10 +228,15 @@ struct RowFill {
 };
 constexpr int kTileBytes = RowFill<uint32_t, 128>::TILE;  // per warp, 128-byte segments
 
-// Emits `len` outputs of this lane's stream to dst (16-byte aligned rows), all
+// Emits `len` outputs of this lane's stream to dst (aligned to an output), all
 // 32 lanes of the warp taking part (lanes with len 0 only help store).
 // next() returns the next 32-bit output; cvt converts it.  tile: the warp's
 // RowFill<OutT, ROWB>::TILE bytes of shared memory.
+// Rows on 16-byte boundaries are cut from their start.  Where a row of the warp is not on
+// one, every row is cut at multiples of ROWB in memory, so that every chunk but its first
+// and last leaves as whole lines in 16-byte stores (2^20 rows of 777: LFSR113 f32 813 us,
+// MRG32K3A u32 945, by each thread's own stores 3436 and 3385).  The chunks that every
+// lane has whole are a loop of their own; tests in it cost MRG32K3A 2 % of its bulk fill.
 // ROLL: keep the loop over a chunk's 16-byte pieces rolled (for generators
 // whose next() is long, where unrolling a whole chunk would outgrow the
 // instruction cache).
@@ -240,20 +245,52 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 {
     using RF = RowFill<OutT, ROWB>;
     constexpr int K = RF::K, E = RF::E, PITCH = RF::PITCH, PIECES = RF::PIECES, ROWS = RF::ROWS;
-    uint64_t maxlen = len;
+    const bool on_vectors = __all_sync(kFull, len == 0 || (uintptr_t)dst % 16 == 0);
+    const uint32_t phase = on_vectors ? 0u : (uint32_t)((uintptr_t)dst % ROWB) / (uint32_t)sizeof(OutT);
+    OutT *const base = dst - phase;          // the row in whole chunks, from its first output's
+    const uint64_t end = len ? phase + len : 0;
+    uint64_t maxend = end, minend = end;
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) maxlen = max(maxlen, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)maxlen, d));
-    const uint64_t nch = (maxlen + K - 1) / K;
+    for (int d = 16; d >= 1; d >>= 1) {
+        maxend = max(maxend, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)maxend, d));
+        minend = min(minend, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)minend, d));
+    }
+    const uint64_t nch = (maxend + K - 1) / K;
+    const uint64_t whole0 = on_vectors ? 0 : 1, whole1 = minend / K;  // the chunks every lane has whole
     unsigned char *myrow = tile + lane * PITCH;
     const int piece = lane % PIECES;
     for (uint64_t ch = 0; ch < nch; ++ch) {
-        const uint32_t cnt = len > ch * K ? (uint32_t)min((uint64_t)K, len - ch * K) : 0u;
-        const unsigned long long mydst = (unsigned long long)(dst + ch * K);
-        if (__all_sync(kFull, cnt == (uint32_t)K)) {
-            // every lane has a whole chunk: no per-output tests, and every row
-            // segment of the tile is stored whole
+        if (ch >= whole0 && ch < whole1) {
+            // no per-output tests, and every row segment of the tile is stored whole
+            do {
+                const unsigned long long mydst = (unsigned long long)(base + ch * K);
 #pragma unroll (ROLL ? 1 : PIECES)
-            for (int v = 0; v < PIECES; ++v) {
+                for (int v = 0; v < PIECES; ++v) {
+                    OutT vals[E];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) vals[e] = cvt(next());
+                    *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    const int r = ROWS * i + lane / PIECES;
+                    OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
+                    *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
+                }
+                __syncwarp();
+            } while (++ch < whole1);
+            if (ch >= nch) return;
+        }
+        // this lane's outputs of the chunk: columns lo .. hi - 1
+        const uint32_t lo = ch ? 0u : phase;
+        const uint32_t hi = end > ch * K ? (uint32_t)min((uint64_t)K, end - ch * K) : 0u;
+        const unsigned long long mydst = (unsigned long long)(base + ch * K);
+        const uint32_t hi0 = __shfl_sync(kFull, hi, 0);
+        if (hi0 % E == 0 && __all_sync(kFull, lo == 0 && hi == hi0)) {
+            // every lane has the same whole pieces: short rows, or the end of rows
+#pragma unroll 4
+            for (int v = 0; v < (int)(hi0 / E); ++v) {
                 OutT vals[E];
 #pragma unroll
                 for (int e = 0; e < E; ++e) vals[e] = cvt(next());
@@ -264,38 +301,52 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
             for (int i = 0; i < PIECES; ++i) {
                 const int r = ROWS * i + lane / PIECES;
                 OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
-                *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
+                if (piece * E < (int)hi0)
+                    *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
             }
             __syncwarp();
             continue;
         }
-#pragma unroll
+        // a row's first or last chunk, or rows of several lengths: rolled (a warp comes here
+        // once or twice a row, with cold code: unrolled it took 2 us a chunk)
+#pragma unroll 1
         for (int v = 0; v < PIECES; ++v) {
-            if ((uint32_t)(v * E) < cnt) {
-                OutT vals[E];
+            if ((uint32_t)(v * E) >= hi) continue;
+            OutT vals[E];
 #pragma unroll
-                for (int e = 0; e < E; ++e) vals[e] = (uint32_t)(v * E + e) < cnt ? cvt(next()) : OutT(0);
-                *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
-            }
+            for (uint32_t e = 0; e < E; ++e) vals[e] = v * E + e >= lo && v * E + e < hi ? cvt(next()) : OutT(0);
+            *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
         }
         __syncwarp();
-#pragma unroll
+#pragma unroll 1
         for (int i = 0; i < PIECES; ++i) {
             const int r = ROWS * i + lane / PIECES;
             OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
-            const uint32_t rc = __shfl_sync(kFull, cnt, r);
-            const int col = piece * E;
+            const uint32_t rl = __shfl_sync(kFull, lo, r), rh = __shfl_sync(kFull, hi, r), col = piece * E;
             const unsigned char *src = tile + r * PITCH + 16 * piece;
-            if ((uint32_t)(col + E) <= rc) {
+            if (col >= rl && col + E <= rh) {
                 *reinterpret_cast<uint4 *>(rd + col) = *reinterpret_cast<const uint4 *>(src);
             } else {
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    if ((uint32_t)(col + e) < rc) rd[col + e] = reinterpret_cast<const OutT *>(src)[e];
+                    if (col + e >= rl && col + e < rh) rd[col + e] = reinterpret_cast<const OutT *>(src)[e];
             }
         }
         __syncwarp();
     }
+}
+
+// Whether a fill of n rows of nper outputs leaves through fill_rows: rows that all start
+// on 16 bytes, and others when the fill is too large for L2 to put the lines of each
+// thread's own stores together (MRG32K3A u32, 2^20 rows of 47 outputs, 197 MB: 162 us
+// staged, 152 by own stores; of 63, 264 MB: 180 and 212; of 777: 945 and 3385; 65536 of
+// 777, 204 MB: 88 and 187; of 301, 79 MB: 47 and 32).
+template <typename OutT>
+inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint64_t seclen)
+{
+    constexpr uint64_t E = RowFill<OutT>::E;
+    return ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0) ||
+           (nper >= 64 && n * nper >= (144ull << 20) / sizeof(OutT));
 }
 
 // Resident threads of a kernel launched with BS-thread blocks on the current

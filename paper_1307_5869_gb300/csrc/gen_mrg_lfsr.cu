@@ -33,16 +33,9 @@ struct LfsrSecJumps {
     static constexpr int kCount = kSecJumps;
     uint32_t col[kSecJumps][4][32];  // [s - 1][component][bit]: image of bit i under T_c^(s seclen)
 };
-// MRG32K3A: section s < 16^4 reached by one matrix per nonzero base-16 digit
-// d_j of s (A^(d_j 16^j seclen) commute, so their order does not matter): at
-// most four 3x3 products however many sections a fill has, so a single stream
-// can be split into sections of 64 outputs (one table entry per set bit of the
-// offset would cost up to 14 dependent products per section).
-struct MrgSecJumps {
-    static constexpr int kLevels = 4;
-    static constexpr uint32_t kMaxSections = 1u << (4 * kLevels);
-    uint32_t m[kLevels][15][18];  // [j][d - 1]: A^(d 16^j seclen) mod m1, B^(...) mod m2, row-major
-};
+// MRG32K3A: by the bytes of the section's offset (mrg_apply_word), at most three 3x3
+// products however many sections a fill has.
+struct MrgByteJumps {};
 
 template <typename SJ>
 __device__ __forceinline__ void lfsr_jump_section(const uint32_t *tab, const SJ &sj, uint64_t sec, uint64_t start,
@@ -59,24 +52,14 @@ __device__ __forceinline__ void lfsr_jump_section(const uint32_t *tab, const SJ 
 }
 
 template <typename SJ>
-__device__ __forceinline__ void mrg_jump_section(const uint32_t *tab, const SJ &sj, uint64_t sec, uint64_t start,
-                                                 uint32_t x[3], uint32_t y[3])
+__device__ __forceinline__ void mrg_jump_section(const uint32_t *tab, const SJ &, uint64_t start, uint32_t x[3], uint32_t y[3])
 {
-    if constexpr (!std::is_same<SJ, NoSecJumps>::value) {
-        if (sec < (uint64_t)SJ::kMaxSections) {
-#pragma unroll
-            for (int j = 0; j < SJ::kLevels; ++j) {
-                const uint32_t d = (uint32_t)(sec >> (4 * j)) & 15u;
-                if (d) {
-                    mat3_vec<209>(sj.m[j][d - 1], x);
-                    mat3_vec<22853>(sj.m[j][d - 1] + 9, y);
-                }
-            }
-            return;
-        }
+    if constexpr (std::is_same<SJ, MrgByteJumps>::value) {
+        mrg_apply_word(tab, 0, start, x, y);
+    } else {
+        for (int b = 0; b < 64; ++b)
+            if ((start >> b) & 1u) mrg_apply_bit(tab, b, x, y);
     }
-    for (int b = 0; b < 64; ++b)
-        if ((start >> b) & 1u) mrg_apply_bit(tab, b, x, y);
 }
 
 // =========================================================== MRG32K3A
@@ -91,6 +74,26 @@ __global__ void mrg_table_kernel(uint32_t *tab)
         mat3_sqr<209>(A);
         mat3_sqr<22853>(B);
     }
+}
+
+// The table's bytes, from its bits: one block per position, one thread per digit.
+__global__ void __launch_bounds__(256) mrg_window_kernel(uint32_t *tab)
+{
+    uint32_t A[9] = { 1, 0, 0, 0, 1, 0, 0, 0, 1 }, B[9] = { 1, 0, 0, 0, 1, 0, 0, 0, 1 };
+#pragma unroll 1
+    for (int b = 0; b < 8; ++b) {
+        if (!((threadIdx.x >> b) & 1u)) continue;
+        const uint32_t *m = tab + 18 * (8 * blockIdx.x + b);
+        for (int c = 0; c < 3; ++c) {  // column by column: m times the product so far
+            uint32_t x[3] = { A[c], A[3 + c], A[6 + c] }, y[3] = { B[c], B[3 + c], B[6 + c] };
+            mat3_vec<209>(m, x);
+            mat3_vec<22853>(m + 9, y);
+            for (int i = 0; i < 3; ++i) { A[3 * i + c] = x[i]; B[3 * i + c] = y[i]; }
+        }
+    }
+    uint32_t *row = tab + mrg_byte_row(blockIdx.x, threadIdx.x);
+    for (int i = 0; i < 9; ++i) { row[i] = A[i]; row[9 + i] = B[i]; }
+    row[18] = row[19] = 0;
 }
 
 // Default state: all six words 12345 (the paper does not print it; L'Ecuyer's
@@ -128,9 +131,7 @@ __global__ void mrg_init_kernel(const uint32_t *tab, const uint32_t *base, uint3
     uint32_t x[3] = { base[0], base[1], base[2] }, y[3] = { base[3], base[4], base[5] };
     uint64_t e[3];
     mul_64x128(first + j, llo, lhi, e);
-    for (int w = 0; w < 3; ++w)
-        for (int b = 0; e[w] && b < 64; ++b)
-            if ((e[w] >> b) & 1u) mrg_apply_bit(tab, 64 * w + b, x, y);
+    for (int w = 0; w < 3; ++w) mrg_apply_word(tab, w, e[w], x, y);
     for (int i = 0; i < 3; ++i) { state[i * n + j] = x[i]; state[(3 + i) * n + j] = y[i]; }
 }
 
@@ -140,8 +141,7 @@ __global__ void mrg_skip_kernel(const uint32_t *tab, uint32_t *state, uint64_t n
     if (j >= n) return;
     uint32_t x[3], y[3];
     for (int i = 0; i < 3; ++i) { x[i] = state[i * n + j]; y[i] = state[(3 + i) * n + j]; }
-    for (int b = 0; b < kJumpBits; ++b)
-        if (u256_bit(off, b)) mrg_apply_bit(tab, b, x, y);
+    for (int w = 0; w < kJumpBits / 64; ++w) mrg_apply_word(tab, w, off.w[w], x, y);
     for (int i = 0; i < 3; ++i) { state[i * n + j] = x[i]; state[(3 + i) * n + j] = y[i]; }
 }
 
@@ -150,7 +150,7 @@ __global__ void mrg_skip_kernel(const uint32_t *tab, uint32_t *state, uint64_t n
 // next state to sout, a separate buffer when a stream has several sections (so
 // no thread reads a state that another thread has already replaced).
 template <typename OutT, bool ROWS = false, typename SJ = NoSecJumps>
-__global__ void __launch_bounds__(256) mrg_gen_kernel(const uint32_t *__restrict__ tab, const uint32_t *state, uint32_t *sout, uint64_t nstreams,
+__global__ void __launch_bounds__(256, 4) mrg_gen_kernel(const uint32_t *__restrict__ tab, const uint32_t *state, uint32_t *sout, uint64_t nstreams,
                                                       uint64_t stride, uint64_t nper, uint32_t nsec, uint64_t seclen,
                                                       OutT *__restrict__ out, int vec, const __grid_constant__ SJ sj)
 {
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) mrg_gen_kernel(const uint32_t *__restrict
             y0 = state[3 * stride + j]; y1 = state[4 * stride + j]; y2 = state[5 * stride + j];
             if (start) {
                 uint32_t x[3] = { x0, x1, x2 }, y[3] = { y0, y1, y2 };
-                mrg_jump_section(tab, sj, tid / nstreams, start, x, y);
+                mrg_jump_section(tab, sj, start, x, y);
                 x0 = x[0]; x1 = x[1]; x2 = x[2]; y0 = y[0]; y1 = y[1]; y2 = y[2];
             }
         }
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(256) mrg_gen_kernel(const uint32_t *__restrict
     uint32_t y0 = state[3 * stride + j], y1 = state[4 * stride + j], y2 = state[5 * stride + j];
     if (start) {
         uint32_t x[3] = { x0, x1, x2 }, y[3] = { y0, y1, y2 };
-        mrg_jump_section(tab, sj, sec, start, x, y);
+        mrg_jump_section(tab, sj, start, x, y);
         x0 = x[0]; x1 = x[1]; x2 = x[2]; y0 = y[0]; y1 = y[1]; y2 = y[2];
     }
     OutT *o = out + j * nper + start;
@@ -340,6 +340,7 @@ static unsigned grid_for(uint64_t n, unsigned block) { return (unsigned)((n + bl
 prand_status_t mrg_build_table(uint32_t *tab, cudaStream_t st)
 {
     mrg_table_kernel<<<1, 32, 0, st>>>(tab);
+    mrg_window_kernel<<<kMrgBytes, 256, 0, st>>>(tab);
     return launch_check();
 }
 
@@ -405,20 +406,6 @@ uint32_t lfsr_comp_step_host(int c, uint32_t z)
     }
 }
 
-using Mat3 = std::array<uint64_t, 9>;
-
-Mat3 mat3_mul(const Mat3 &X, const Mat3 &Y, uint64_t m)
-{
-    Mat3 R;
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            uint64_t s = 0;
-            for (int k = 0; k < 3; ++k) s = (s + X[3 * i + k] * Y[3 * k + j] % m) % m;
-            R[3 * i + j] = s;
-        }
-    return R;
-}
-
 template <typename M, typename Mul>
 M mat_pow(M base, uint64_t e, M one, Mul mul)
 {
@@ -433,7 +420,6 @@ M mat_pow(M base, uint64_t e, M one, Mul mul)
 
 std::mutex g_sj_mu;
 std::map<std::tuple<int, uint64_t, uint32_t>, LfsrSecJumps> g_sj_lfsr;
-std::map<std::tuple<int, uint64_t, uint32_t>, MrgSecJumps> g_sj_mrg;
 constexpr size_t kSecJumpCacheMax = 256;
 
 void build_sec_jumps(uint64_t seclen, uint32_t nsec, LfsrSecJumps *out)
@@ -449,30 +435,6 @@ void build_sec_jumps(uint64_t seclen, uint32_t nsec, LfsrSecJumps *out)
             for (int i = 0; i < 32; ++i) out->col[s - 1][c][i] = J[i];
             J = gf2_mul(J, A);
         }
-    }
-}
-
-void build_sec_jumps(uint64_t seclen, uint32_t nsec, MrgSecJumps *out)
-{
-    const Mat3 one = { 1, 0, 0, 0, 1, 0, 0, 0, 1 };
-    const Mat3 a = { 0, 1403580, kM1 - 810728, 1, 0, 0, 0, 1, 0 };
-    const Mat3 b = { 527612, 0, kM2 - 1370589, 1, 0, 0, 0, 1, 0 };
-    auto mul1 = [](const Mat3 &X, const Mat3 &Y) { return mat3_mul(X, Y, kM1); };
-    auto mul2 = [](const Mat3 &X, const Mat3 &Y) { return mat3_mul(X, Y, kM2); };
-    (void)nsec;
-    Mat3 A = mat_pow(a, seclen, one, mul1), B = mat_pow(b, seclen, one, mul2);  // A^(16^j seclen)
-    for (int j = 0; j < MrgSecJumps::kLevels; ++j) {
-        Mat3 JA = A, JB = B;
-        for (int d = 1; d < 16; ++d) {
-            for (int i = 0; i < 9; ++i) {
-                out->m[j][d - 1][i] = (uint32_t)JA[i];
-                out->m[j][d - 1][9 + i] = (uint32_t)JB[i];
-            }
-            JA = mul1(JA, A);
-            JB = mul2(JB, B);
-        }
-        A = JA;  // (A^(16^j seclen))^16
-        B = JB;
     }
 }
 
@@ -498,7 +460,8 @@ void sec_jumps(std::map<std::tuple<int, uint64_t, uint32_t>, SJ> &cache, int gen
 // Sections per stream: whole waves of the kernel's resident threads (cap),
 // sections no shorter than min_len outputs (256 for LFSR113, whose section
 // jumps beyond the 15 tabulated ones take one table entry per set bit of the
-// offset; 64 for MRG32K3A, whose take at most four products) and starting on
+// offset; 32 for MRG32K3A, whose take one product per byte: one stream of 10^6
+// doubles 10.3 us, by sections of 64 and matrices passed with the launch 16.4) and starting on
 // multiples of 32 outputs, so the staged 128-byte row stores of every section
 // fill whole cache lines.
 static void pick_sections(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t min_len, uint32_t *nsec,
@@ -522,7 +485,7 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
         // size by the rows form (the other form has the same footprint or less)
         const uint64_t cap = gen == PRAND_MRG32K3A ? resident_threads<1>(mrg_gen_kernel<OutT, true>)
                                                    : resident_threads<2, kLfsrBlock>(lfsr_gen_kernel<OutT, true>);
-        pick_sections(R.count, nper, cap, gen == PRAND_MRG32K3A ? 64 : 256, &R.nsec, &R.seclen);
+        pick_sections(R.count, nper, cap, gen == PRAND_MRG32K3A ? 32 : 256, &R.nsec, &R.seclen);
     }
     const uint32_t nsec = R.nsec;
     const uint64_t seclen = R.seclen, nstreams = R.count;
@@ -530,22 +493,13 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
     const unsigned B = 256;
     uint64_t threads = nstreams * nsec;
     uint32_t *sin = (uint32_t *)d_state + R.j0, *sout = (nsec > 1 ? (uint32_t *)d_spare : (uint32_t *)d_state) + R.j0;
-    // staged row stores need every row start 16-byte aligned
-    constexpr uint64_t E = RowFill<OutT>::E;
-    const bool rows = ((uintptr_t)out % 16) == 0 && nper % E == 0 && seclen % E == 0;
+    const bool rows = staged_rows(out, nstreams, nper, seclen);
     // section jumps as one matrix per section when there are few sections
-    const bool sj = nsec > 1 && (gen == PRAND_MRG32K3A ? nsec <= MrgSecJumps::kMaxSections : nsec <= (uint32_t)kSecJumps + 1);
+    const bool sj = nsec > 1 && nsec <= (uint32_t)kSecJumps + 1;
     if (gen == PRAND_MRG32K3A) {
         const unsigned g = grid_for(threads, B);
-        if (sj) {
-            MrgSecJumps J;
-            sec_jumps(g_sj_mrg, gen, seclen, nsec, &J);
-            if (rows) mrg_gen_kernel<OutT, true, MrgSecJumps><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, J);
-            else mrg_gen_kernel<OutT, false, MrgSecJumps><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, J);
-        } else {
-            if (rows) mrg_gen_kernel<OutT, true><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, NoSecJumps{});
-            else mrg_gen_kernel<OutT><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, NoSecJumps{});
-        }
+        if (rows) mrg_gen_kernel<OutT, true, MrgByteJumps><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, MrgByteJumps{});
+        else mrg_gen_kernel<OutT, false, MrgByteJumps><<<g, B, 0, st>>>(T->mrg, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, vec, MrgByteJumps{});
     } else {
         const unsigned BL = kLfsrBlock, g = grid_for(threads, BL);
         if (sj) {
@@ -684,14 +638,12 @@ extern "C" prand_status_t prand_mrg32k3a_generate_u32_noalloc(uint32_t *dev_stat
     if (n_per_stream == 0) return PRAND_OK;
     uint32_t nsec;
     uint64_t seclen;
-    // the store form of prand_generate_u32 on a handle (staged 128-byte row
-    // stores whenever every row start is 16-byte aligned); sections of at least
+    // the store form of prand_generate_u32 on a handle; sections of at least
     // 256 outputs, since this path builds no section matrices (that would
     // allocate host memory) and jumps by one table entry per set bit
     pick_sections(n_streams, n_per_stream, resident_threads<1>(mrg_gen_kernel<uint32_t, true>), 256, &nsec, &seclen);
     int vec = ((uintptr_t)dev_out % 16) == 0;
-    constexpr uint64_t E = RowFill<uint32_t>::E;
-    const bool rows = vec && n_per_stream % E == 0 && seclen % E == 0;
+    const bool rows = staged_rows(dev_out, n_streams, n_per_stream, seclen);
     const unsigned B = 256;
     const unsigned grid = grid_for(n_streams * nsec, B);
     uint32_t *sout = nsec > 1 ? D->next : dev_state;

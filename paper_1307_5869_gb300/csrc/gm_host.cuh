@@ -133,8 +133,7 @@ struct GmHost {
             const uint32_t nsec = R.nsec;
             const uint64_t seclen = R.seclen, nstreams = R.count;
             uint64_t *sout = (nsec > 1 ? spare : state) + off;
-            constexpr uint64_t E = RowFill<OutT>::E;
-            const bool rows = ((uintptr_t)out % 16) == 0 && nper % E == 0 && seclen % E == 0;
+            const bool rows = staged_rows(out, nstreams, nper, seclen);
             const unsigned grid = gm_grid_for(nstreams * nsec, B);
             if (rows) gmt_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
             else gmt_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);

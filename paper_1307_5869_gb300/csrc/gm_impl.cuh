@@ -669,7 +669,7 @@ __device__ __forceinline__ void gmt_store(const GmZ<GEN> *zc, const GmZ<GEN> *zp
 // apart, and a thread reading its own touches every line of the warp at every load.
 // tile: 32 rows of an odd number of words each, so the lanes' rows meet no bank conflicts.
 template <int GEN>
-__device__ __forceinline__ void gmt_stage_in(const uint64_t *from, int rows, uint64_t *tile, int lane, uint64_t *v)
+__device__ __forceinline__ void gmt_stage_in(const uint64_t *from, int rows, uint64_t *tile, int lane, GmZ<GEN> *z)
 {
     constexpr int S = GmT<GEN>::s, PITCH = S | 1;
 #pragma unroll
@@ -679,15 +679,15 @@ __device__ __forceinline__ void gmt_stage_in(const uint64_t *from, int rows, uin
     }
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < S; ++i) v[i] = lane < rows ? tile[lane * PITCH + i] : 0;
+    for (int i = 0; i < S; ++i) z[i] = lane < rows ? (GmZ<GEN>)(tile[lane * PITCH + i] >> GmT<GEN>::t) : 0;
     __syncwarp();
 }
 template <int GEN>
-__device__ __forceinline__ void gmt_stage_out(const uint64_t *v, int rows, uint64_t *tile, int lane, uint64_t *to)
+__device__ __forceinline__ void gmt_stage_out(const GmZ<GEN> *z, int rows, uint64_t *tile, int lane, uint64_t *to)
 {
     constexpr int S = GmT<GEN>::s, PITCH = S | 1;
 #pragma unroll
-    for (int i = 0; i < S; ++i) tile[lane * PITCH + i] = v[i];
+    for (int i = 0; i < S; ++i) tile[lane * PITCH + i] = (uint64_t)gm_canon<GEN>(z[i]) << GmT<GEN>::t;
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < S; ++i) {
@@ -702,7 +702,7 @@ __device__ __forceinline__ void gmt_stage_out(const uint64_t *v, int rows, uint6
 // 128-byte row stores (every lane of a warp takes part); else one store per
 // output.  The thread of the last section writes the next state to state_out.
 template <int GEN, typename OutT, bool ROWS>
-__global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict__ tab, const uint64_t *state_in,
+__global__ void __launch_bounds__(256, 3) gmt_gen_kernel(const uint64_t *__restrict__ tab, const uint64_t *state_in,
                                                       uint64_t *state_out, uint64_t nstreams, uint64_t stride,
                                                       uint64_t nper, uint32_t nsec, uint64_t seclen,
                                                       OutT *__restrict__ out)
@@ -726,11 +726,8 @@ __global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict
     Z zc[P::s], zp[P::s];
     if (nsec == 1) {
         if (!rows) return;  // whole warp
-        uint64_t q[P::s], c[P::s];
-        gmt_stage_in<GEN>(state_in + j0 * P::s, rows, tile, lane, q);
-        gmt_stage_in<GEN>(state_in + (stride + j0) * P::s, rows, tile, lane, c);
-#pragma unroll
-        for (int i = 0; i < P::s; ++i) { zp[i] = (Z)(q[i] >> P::t); zc[i] = (Z)(c[i] >> P::t); }
+        gmt_stage_in<GEN>(state_in + j0 * P::s, rows, tile, lane, zp);
+        gmt_stage_in<GEN>(state_in + (stride + j0) * P::s, rows, tile, lane, zc);
     } else if (len) {
         gmt_load<GEN>(tab, state_in + j * P::s, state_in + (stride + j) * P::s, start, 0, zc, zp);
     } else {
@@ -747,11 +744,8 @@ __global__ void __launch_bounds__(256) gmt_gen_kernel(const uint64_t *__restrict
     }
     if (nsec == 1) {
         __syncwarp();
-        uint64_t q[P::s], c[P::s];
-#pragma unroll
-        for (int i = 0; i < P::s; ++i) { q[i] = gm_canon<GEN>(zp[i]) << P::t; c[i] = gm_canon<GEN>(zc[i]) << P::t; }
-        gmt_stage_out<GEN>(q, rows, tile, lane, state_out + j0 * P::s);
-        gmt_stage_out<GEN>(c, rows, tile, lane, state_out + (stride + j0) * P::s);
+        gmt_stage_out<GEN>(zp, rows, tile, lane, state_out + j0 * P::s);
+        gmt_stage_out<GEN>(zc, rows, tile, lane, state_out + (stride + j0) * P::s);
     } else if (len && start + len == nper) {
         gmt_store<GEN>(zc, zp, state_out + j * P::s, state_out + (stride + j) * P::s);
     }

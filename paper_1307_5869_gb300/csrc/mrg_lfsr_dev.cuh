@@ -49,6 +49,31 @@ __device__ __forceinline__ void mrg_apply_bit(const uint32_t *tab, int b, uint32
     mat3_vec<22853>(tab + 18 * b + 9, y);
 }
 
+// The same jumps by bytes of the exponent: entry (i, d) of the table's second part is the
+// pair of matrices of d 2^(8 i) steps, in five 16-byte vectors.
+constexpr int kMrgRow = 20, kMrgBytes = kJumpBits / 8;
+constexpr size_t kMrgTabWords = (size_t)kJumpBits * 18 + (size_t)kMrgBytes * 256 * kMrgRow;
+
+__host__ __device__ __forceinline__ constexpr size_t mrg_byte_row(int i, uint32_t d)
+{
+    return (size_t)kJumpBits * 18 + ((size_t)i * 256 + d) * kMrgRow;
+}
+
+// Advance (x, y) by e 2^(64 at) steps: one application per nonzero byte of e.
+__device__ __forceinline__ void mrg_apply_word(const uint32_t *tab, int at, uint64_t e, uint32_t x[3], uint32_t y[3])
+{
+#pragma unroll 1
+    for (int i = 8 * at; e; ++i, e >>= 8) {
+        if (!(e & 255u)) continue;
+        const uint4 *row = reinterpret_cast<const uint4 *>(tab + mrg_byte_row(i, (uint32_t)e & 255u));
+        uint32_t m[kMrgRow];
+#pragma unroll
+        for (int k = 0; k < kMrgRow / 4; ++k) *reinterpret_cast<uint4 *>(m + 4 * k) = row[k];
+        mat3_vec<209>(m, x);
+        mat3_vec<22853>(m + 9, y);
+    }
+}
+
 // One MRG32K3A step (x_n = a x_{n-2} - b x_{n-3} mod m1, y_n = c y_{n-1} -
 // d y_{n-3} mod m2, Sec. 5.2) on canonical residues, in 32-bit limbs:
 // t = m - v (no borrow), S = A u + B t < 2^54 by two wide multiply-adds; with
