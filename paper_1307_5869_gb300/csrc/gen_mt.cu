@@ -17,6 +17,8 @@
 // With Y in window form (x_t..x_{t+623}), A^i Y is the window starting at
 // x_{t+i}, so the sum is a sliding-window XOR over the stream's next 20560
 // words, taken at the set coefficients of g_v (mt_jump_block).
+#include <type_traits>
+
 #include "mt_dev.cuh"
 
 namespace prand {
@@ -92,6 +94,36 @@ __global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_gen_kernel(uint32_t 
     const uint32_t *cur = in_b0 ? b0 : b1;
     uint32_t *dst = state + j * kMtN;
     mt_copy_state_warp(cur, dst, lane);
+}
+
+// Few streams: a block per stream, which makes each block of words in three rounds
+// (mt_twist_emit_team) where one warp takes twenty steps: 96 streams of 1001 f32 4.1 us
+// (5.7), one of 10^6 u32 415 (1376).  With six streams or more per SM the warps fill it by
+// themselves (10^4 outputs of 608 streams 12.3 and 18.5 us, of 1216 20.5 and 20.5, of 2432
+// 35.9 and 27.6).
+constexpr int kMtGenTeam = 8;
+constexpr uint64_t kMtTeamStreams = 6;
+
+template <typename OutT>
+__global__ void __launch_bounds__(32 * kMtGenTeam) mt_gen_team_kernel(uint32_t *state, uint32_t idx0, uint64_t nper, OutT *__restrict__ out)
+{
+    __shared__ uint32_t sm[2][kMtN];
+    uint32_t *s = state + blockIdx.x * (uint64_t)kMtN;
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtGenTeam) sm[0][i] = s[i];
+    __syncthreads();
+    OutT *o = out + blockIdx.x * nper;
+    uint64_t done = 0;
+    if (idx0 < (uint32_t)kMtN) {  // the rest of the current block
+        done = min((uint64_t)(kMtN - idx0), nper);
+        for (uint32_t t = threadIdx.x; t < (uint32_t)done; t += 32 * kMtGenTeam) o[t] = Cvt<OutT>::f(mt_temper(sm[0][idx0 + t]));
+    }
+    int cur = 0;
+    for (; done < nper; cur ^= 1) {
+        const uint32_t emit = (uint32_t)min(nper - done, (uint64_t)kMtN);
+        mt_twist_emit_team<OutT, kMtGenTeam>(sm[cur], sm[cur ^ 1], o + done, emit);
+        done += emit;
+    }
+    for (int i = threadIdx.x; i < kMtN; i += 32 * kMtGenTeam) s[i] = sm[cur][i];
 }
 
 // ------------------------------------------------------------------ jump
@@ -218,10 +250,16 @@ prand_status_t mt_skip(const DevTables *T, void *d_state, uint64_t n, uint32_t *
 prand_status_t mt_gen(void *d_state, uint64_t nstreams, uint32_t *idx, void *out, int dtype, uint64_t nper, cudaStream_t st)
 {
     uint32_t *state = (uint32_t *)d_state;
-    unsigned grid = grid_warps(nstreams);
-    if (dtype == PRAND_DTYPE_U32) mt_gen_kernel<uint32_t><<<grid, 32 * kMtWarpsPerBlock, 0, st>>>(state, nstreams, *idx, nper, (uint32_t *)out);
-    else if (dtype == PRAND_DTYPE_F32) mt_gen_kernel<float><<<grid, 32 * kMtWarpsPerBlock, 0, st>>>(state, nstreams, *idx, nper, (float *)out);
-    else mt_gen_kernel<double><<<grid, 32 * kMtWarpsPerBlock, 0, st>>>(state, nstreams, *idx, nper, (double *)out);
+    const auto launch = [&](auto *o) {
+        using OutT = std::remove_pointer_t<decltype(o)>;
+        if (nstreams <= kMtTeamStreams * (uint64_t)device_sm_count())
+            mt_gen_team_kernel<<<(unsigned)nstreams, 32 * kMtGenTeam, 0, st>>>(state, *idx, nper, o);
+        else
+            mt_gen_kernel<OutT><<<grid_warps(nstreams), 32 * kMtWarpsPerBlock, 0, st>>>(state, nstreams, *idx, nper, o);
+    };
+    if (dtype == PRAND_DTYPE_U32) launch((uint32_t *)out);
+    else if (dtype == PRAND_DTYPE_F32) launch((float *)out);
+    else launch((double *)out);
     prand_status_t s = launch_check();
     if (s != PRAND_OK) return s;
     // the index after nper outputs: the rest of the current block, then whole blocks
