@@ -309,7 +309,7 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
         }
         // a row's first or last chunk, or rows of several lengths: rolled (a warp comes here
         // once or twice a row, with cold code: unrolled it took 2 us a chunk)
-#pragma unroll 1
+#pragma unroll 2
         for (int v = 0; v < PIECES; ++v) {
             if ((uint32_t)(v * E) >= hi) continue;
             OutT vals[E];
@@ -336,17 +336,25 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
     }
 }
 
-// Whether a fill of n rows of nper outputs leaves through fill_rows: rows that all start
-// on 16 bytes, and others when the fill is too large for L2 to put the lines of each
-// thread's own stores together (MRG32K3A u32, 2^20 rows of 47 outputs, 197 MB: 162 us
-// staged, 152 by own stores; of 63, 264 MB: 180 and 212; of 777: 945 and 3385; 65536 of
-// 777, 204 MB: 88 and 187; of 301, 79 MB: 47 and 32).
+// Whether a fill of n rows of nper outputs (nsec sections of seclen each) leaves through
+// fill_rows or by each thread's own stores, whose lines L2 puts together while the fill
+// fits there.  Rows on 16-byte boundaries: staged from 96 MiB on, and below if sections
+// are own_len or longer (32 for the lighter steps; never for MRG32K3A, whose stores then
+// hide behind its steps), but not for less than a warp of sections.  Others: staged when
+// long and beyond L2.  Measured, us, staged / own:
+//   on 16 bytes: MRG32K3A one stream of 10^6 f64 10.3 / 8.2, 65536 x 300 u32 32.7 / 30.8,
+//     x 500 f32 51 / 71; LFSR113 f32 2^20 x 16 30.8 / 22.6, 2^18 x 32 12.6 / 13.3, 65536 x
+//     320 26.7 / 32.8; one stream of 64: LFSR113 u32 8.2 / 4.2, GQ58.3 18.5 / 12.3
+//   others: MRG32K3A u32 2^20 x 47 162 / 152, x 63 180 / 212, x 777 945 / 3385, 65536 x
+//     777 88 / 187, x 301 47 / 32
 template <typename OutT>
-inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint64_t seclen)
+inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len)
 {
     constexpr uint64_t E = RowFill<OutT>::E;
-    return ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0) ||
-           (nper >= 64 && n * nper >= (144ull << 20) / sizeof(OutT));
+    const uint64_t mib = n * nper / ((1ull << 20) / sizeof(OutT));
+    if ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0)
+        return mib >= 96 || (seclen >= own_len && n * nsec >= 32);
+    return nper >= 64 && mib >= 144;
 }
 
 // Resident threads of a kernel launched with BS-thread blocks on the current

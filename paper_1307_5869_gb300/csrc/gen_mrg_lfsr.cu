@@ -458,10 +458,11 @@ void sec_jumps(std::map<std::tuple<int, uint64_t, uint32_t>, SJ> &cache, int gen
 }  // namespace
 
 // Sections per stream: whole waves of the kernel's resident threads (cap),
-// sections no shorter than min_len outputs (256 for LFSR113, whose section
+// sections no shorter than min_len outputs (64 for LFSR113, whose section
 // jumps beyond the 15 tabulated ones take one table entry per set bit of the
-// offset; 32 for MRG32K3A, whose take one product per byte: one stream of 10^6
-// doubles 10.3 us, by sections of 64 and matrices passed with the launch 16.4) and starting on
+// offset: one stream of 10^6 u32 16.4 us, by sections of 128 27.1, of 256 36.9;
+// 32 for MRG32K3A, whose take one product per byte: one stream of 10^6 doubles
+// 10.3 us staged, by sections of 64 and matrices passed with the launch 16.4) and starting on
 // multiples of 32 outputs, so the staged 128-byte row stores of every section
 // fill whole cache lines.
 static void pick_sections(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t min_len, uint32_t *nsec,
@@ -485,7 +486,7 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
         // size by the rows form (the other form has the same footprint or less)
         const uint64_t cap = gen == PRAND_MRG32K3A ? resident_threads<1>(mrg_gen_kernel<OutT, true>)
                                                    : resident_threads<2, kLfsrBlock>(lfsr_gen_kernel<OutT, true>);
-        pick_sections(R.count, nper, cap, gen == PRAND_MRG32K3A ? 32 : 256, &R.nsec, &R.seclen);
+        pick_sections(R.count, nper, cap, gen == PRAND_MRG32K3A ? 32 : 64, &R.nsec, &R.seclen);
     }
     const uint32_t nsec = R.nsec;
     const uint64_t seclen = R.seclen, nstreams = R.count;
@@ -493,7 +494,7 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
     const unsigned B = 256;
     uint64_t threads = nstreams * nsec;
     uint32_t *sin = (uint32_t *)d_state + R.j0, *sout = (nsec > 1 ? (uint32_t *)d_spare : (uint32_t *)d_state) + R.j0;
-    const bool rows = staged_rows(out, nstreams, nper, seclen);
+    const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, gen == PRAND_MRG32K3A ? UINT64_MAX : 32);
     // section jumps as one matrix per section when there are few sections
     const bool sj = nsec > 1 && nsec <= (uint32_t)kSecJumps + 1;
     if (gen == PRAND_MRG32K3A) {
@@ -643,7 +644,7 @@ extern "C" prand_status_t prand_mrg32k3a_generate_u32_noalloc(uint32_t *dev_stat
     // allocate host memory) and jumps by one table entry per set bit
     pick_sections(n_streams, n_per_stream, resident_threads<1>(mrg_gen_kernel<uint32_t, true>), 256, &nsec, &seclen);
     int vec = ((uintptr_t)dev_out % 16) == 0;
-    const bool rows = staged_rows(dev_out, n_streams, n_per_stream, seclen);
+    const bool rows = staged_rows(dev_out, n_streams, n_per_stream, nsec, seclen, UINT64_MAX);
     const unsigned B = 256;
     const unsigned grid = grid_for(n_streams * nsec, B);
     uint32_t *sout = nsec > 1 ? D->next : dev_state;
