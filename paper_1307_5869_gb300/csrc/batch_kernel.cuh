@@ -76,17 +76,17 @@ __device__ __forceinline__ void batch_lfsr(const BatchTile &T, const BatchCtx &C
         for (int b = 0; b < 64; ++b)
             if ((hi >> b) & 1u) lfsr_apply_bit(C.lfsr_tab, 64 + b, z);
     }
-    uint32_t z0 = z[0], z1 = z[1], z2 = z[2], z3 = z[3];
+    LfsrRun run(z[0], z[1], z[2], z[3]);
     OutT *o = (OutT *)T.out + off;
     if (T.flags & kTileVec) {
-        fill_rows<OutT, ROWB>([&]() { return lfsr_next(z0, z1, z2, z3); }, [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len,
+        fill_rows<OutT, ROWB>(run, [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len,
                         wsm, lane);
     } else {
-        for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(lfsr_next(z0, z1, z2, z3));
+        for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(run());
     }
     if ((T.flags & kTileLast) && len && off + len == T.len) {
         uint32_t *d = (uint32_t *)C.slots[PRAND_LFSR113] + 4 * (uint64_t)T.wslot;
-        d[0] = z0; d[1] = z1; d[2] = z2; d[3] = z3;
+        d[0] = run.z0; d[1] = run.z1; d[2] = run.z2; d[3] = run.z3;
     }
 }
 

@@ -3,6 +3,7 @@
 // float epilogue, and vectorised output emission.
 #pragma once
 
+#include <type_traits>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -239,7 +240,8 @@ constexpr int kTileBytes = RowFill<uint32_t, 128>::TILE;  // per warp, 128-byte 
 // lane has whole are a loop of their own; tests in it cost MRG32K3A 2 % of its bulk fill.
 // ROLL: keep the loop over a chunk's 16-byte pieces rolled (for generators
 // whose next() is long, where unrolling a whole chunk would outgrow the
-// instruction cache).
+// instruction cache).  A generator may offer next(k) as well, for output k of a
+// whole chunk (k a constant, in order from 0).
 template <typename OutT, int ROWB = 128, bool ROLL = false, typename Next, typename Conv>
 __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, uint64_t len, unsigned char *tile, int lane)
 {
@@ -268,7 +270,10 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
                 for (int v = 0; v < PIECES; ++v) {
                     OutT vals[E];
 #pragma unroll
-                    for (int e = 0; e < E; ++e) vals[e] = cvt(next());
+                    for (int e = 0; e < E; ++e) {
+                        if constexpr (std::is_invocable<Next, int>::value) vals[e] = cvt(next(v * E + e));
+                        else vals[e] = cvt(next());
+                    }
                     *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
                 }
                 __syncwarp();

@@ -299,10 +299,11 @@ __global__ void __launch_bounds__(kLfsrBlock) lfsr_gen_kernel(const uint32_t *__
                 z0 = z[0]; z1 = z[1]; z2 = z[2]; z3 = z[3];
             }
         }
-        fill_rows<OutT, kLfsrRowBytes>([&]() { return lfsr_next(z0, z1, z2, z3); }, [](uint32_t u) { return Cvt<OutT>::f(u); },
+        LfsrRun run(z0, z1, z2, z3);
+        fill_rows<OutT, kLfsrRowBytes>(run, [](uint32_t u) { return Cvt<OutT>::f(u); },
                         out + j * nper + start, len, tiles[threadIdx.x >> 5], threadIdx.x & 31);
         if (len && start + len == nper) {
-            sout[j] = z0; sout[stride + j] = z1; sout[2 * stride + j] = z2; sout[3 * stride + j] = z3;
+            sout[j] = run.z0; sout[stride + j] = run.z1; sout[2 * stride + j] = run.z2; sout[3 * stride + j] = run.z3;
         }
         return;
     }
