@@ -126,8 +126,15 @@ struct GmHost {
             // when the output is aligned and n_per_stream is a multiple of 4
             const bool vec = ((uintptr_t)out % (sizeof(OutT) == 8 ? 32 : 16)) == 0 && nper % 4 == 0;
             const unsigned grid = gm_grid_for(nstreams * nsec * 32, B);
-            if (vec) gm_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-            else gm_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+            auto launch = [&](auto v, auto few) {
+                gm_gen_kernel<GEN, OutT, decltype(v)::value, decltype(few)::value><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+            };
+            auto by_vec = [&](auto few) {
+                if (vec) launch(std::true_type{}, few);
+                else launch(std::false_type{}, few);
+            };
+            if (gm_blocks_per_sm<GEN>() > 6 && grid <= 3 * (unsigned)device_sm_count()) by_vec(std::integral_constant<bool, (gm_blocks_per_sm<GEN>() > 6)>{});
+            else by_vec(std::false_type{});
         } else {
             if (R.nsec == 0) pick(R.count, nper, resident_threads<200 + GEN>(gmt_gen_kernel<GEN, OutT, true>), 32, 256, 128, &R.nsec, &R.seclen);
             const uint32_t nsec = R.nsec;
