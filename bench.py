@@ -43,13 +43,15 @@ STATE_BYTES = {"MT19937": 624 * 4, "MRG32K3A": 24, "LFSR113": 16, "GM19": 32 * 1
                "GQ58_4": 8 * 16}
 # Algorithmic int32 operations per output word of the integer-bound generators,
 # counted from each kernel's arithmetic on 32-bit lanes (a 32x32->64 product or
-# multiply-add counts as two operations): GM/GQ = the points' steps (the
-# recurrence and its fold), strips and word assembly; MRG32K3A = its two
-# component steps and the combination.  Per point step: GM19, GM29 7; GM31,
-# GQ58.1 10; GM61 16; GM55 20; GQ58.3 12, GQ58.4 13 (a 7-operation step and a
-# 32-bit strip of 5 or 6; GQ58.3's point 11 steps without a strip: 7).
-OPS_PER_WORD = {"GM19": 32 * 7, "GM29": 32 * 7, "GM31": 32 * 10, "GM55": 8 * 20, "GM61": 32 * 16,
-                "GQ58_1": 32 * 10, "GQ58_3": 11 * 12 + 7, "GQ58_4": 8 * 13, "MRG32K3A": 28}
+# multiply-add counts as two operations): GQ58.3 = its points' steps (12 each: a
+# 7-operation step and a 32-bit strip of 5; point 11 steps without a strip);
+# MRG32K3A = its two component steps and the combination.
+OPS_PER_WORD = {"GQ58_3": 11 * 12 + 7, "MRG32K3A": 28}
+# Tensor-core operations per output word of the other GM/GQ generators: a block of 64
+# steps of 128 points is a product 128 x K x 128 (K = 16 slots for the 32-bit primes'
+# bytes, 32 for nibbles) and makes 64 words of 4 (v = 1) or 16 (v = 4) streams.
+TENSOR_FLOP_PER_WORD = {"GM19": 2048, "GM29": 2048, "GM31": 2048, "GQ58_1": 2048, "GM61": 4096, "GM55": 1024,
+                        "GQ58_4": 1024}
 # int32 lanes per SM: four schedulers, each issuing one 32-lane warp instruction per
 # cycle (the issue-slot bound of an integer kernel; the SM count and clock are
 # queried at run time)
@@ -57,9 +59,9 @@ LANES_PER_SM = 128
 # DRAM bytes (read + write) per stream of one fill of 1024 outputs, from ncu
 # captures (dram__bytes_read.sum + dram__bytes_write.sum) of the current kernels
 # at 2^18 streams x 2^10 outputs, scaled per stream; None for other shapes.
-TRAFFIC_PER_STREAM_1024 = {"MT19937.u32": 2.322e9 / 2**18, "MT19937.f32": 2.319e9 / 2**18,
-                           "LFSR113.u32": 1.025e9 / 2**18, "LFSR113.f32": 1.022e9 / 2**18,
-                           "GM61.u32": 1.396e9 / 2**18, "GM61.f32": 1.395e9 / 2**18}
+TRAFFIC_PER_STREAM_1024 = {"MT19937.u32": 2.322e9 / 2**18, "MT19937.f32": 2.322e9 / 2**18,
+                           "LFSR113.u32": 1.025e9 / 2**18, "LFSR113.f32": 1.026e9 / 2**18,
+                           "GM61.u32": 1.284e9 / 2**18, "GM61.f32": 1.283e9 / 2**18}
 # Output arena of the serving leg: 32 GiB of the GPU's HBM holds every request's
 # output until it is read (at 1.9e10 samples/s of 4-8 byte samples, about a
 # third of a second of demand).
@@ -89,6 +91,15 @@ def _peaks():
         return float(d["hbm_gbs"]), "measured"
     except Exception:
         return 6800.0, "fallback"
+
+
+def _tensor_peak():
+    """16-bit tensor rate (TFLOP/s): the measured bf16 GEMM burst."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured"
+    except Exception:
+        return 1900.0, "fallback"
 
 
 class ClockSampler:
@@ -343,7 +354,12 @@ def run_gpu(args):
     for g in gens:
         for dt, ms in (("u32", ms_u[g]), ("f32", ms_f[g])):
             key = f"{g}.{dt}"
-            if g.startswith("GM") or g.startswith("GQ"):
+            if g in TENSOR_FLOP_PER_WORD:
+                # (bound by the issue of what follows the products: profiles/gm_tc_mt_jump_lfsr.md)
+                rooflines[key] = {"bound": "tensor", "achieved": nS * nP * TENSOR_FLOP_PER_WORD[g] / (ms * 1e-3) / 1e12,
+                                  "peak": _tensor_peak()[0], "unit": "TFLOP/s",
+                                  "ms": ms, "gsamples_per_s": nS * nP / (ms * 1e-3) / 1e9}
+            elif g.startswith("GM") or g.startswith("GQ"):
                 ops = nS * nP * OPS_PER_WORD[g]
                 rooflines[key] = {"bound": "alu", "achieved": ops / (ms * 1e-3) / 1e12,
                                   "peak": int_peak, "unit": "Tops/s",
@@ -364,7 +380,8 @@ def run_gpu(args):
     R = rooflines[dom]
     roofline = {"bound": R["bound"], "achieved": R["achieved"], "peak": R["peak"], "unit": R["unit"],
                 "frac": R["frac"], "traffic": R.get("traffic"), "kernel": dom,
-                "peak_source": int_src if R["bound"] == "alu" else f"{peak_src} HBM copy GB/s"}
+                "peak_source": int_src if R["bound"] == "alu" else f"{_tensor_peak()[1]} bf16 GEMM TFLOP/s"
+                if R["bound"] == "tensor" else f"{peak_src} HBM copy GB/s"}
     per_gen = {g: 2 * nS * nP / ((ms_u[g] + ms_f[g]) * 1e-3) / 1e9 for g in gens}
 
     # ----- end to end: same step through host buffers (device -> pinned host copies inside)
@@ -533,6 +550,9 @@ def run_table(P, torch, sp, args):
             byts = nS * nP * 4 + 2 * nS * STATE_BYTES[g]
             res[dt] = {"ms": ms, "gsamples_per_s": nS * nP / (ms * 1e-3) / 1e9,
                        "hbm_frac": byts / (ms * 1e-3) / 1e9 / hbm_peak}
+            if g in TENSOR_FLOP_PER_WORD:
+                res[dt]["tensor_tflops"] = nS * nP * TENSOR_FLOP_PER_WORD[g] / (ms * 1e-3) / 1e12
+                res[dt]["tensor_frac"] = res[dt]["tensor_tflops"] / _tensor_peak()[0]
             if g in OPS_PER_WORD:
                 tops = nS * nP * OPS_PER_WORD[g] / (ms * 1e-3) / 1e12
                 res[dt]["int_tops"] = tops

@@ -29,7 +29,7 @@
 // What bounds it: the arithmetic after the product, per point step two multiply-adds
 // (FMA-heavy pipe, 2 cycles each), one funnel shift and half a three-input minimum
 // (ALU, 2 cycles each), against four 32x32->64 products and a fold (about 24 cycles)
-// by the recurrence; issue slots 70 % busy, both pipes 57 %, the tensor pipe 12 %.
+// by the recurrence; issue slots 70 % busy, both pipes 57 %, the tensor pipe 12 to 22 %.
 // GB300, 65536 streams x 4096 u32, G words/s, lane-per-point or thread-per-stream
 // kernel (gm_impl.cuh) / this one: GM61 51 / 126, GM31 88 / 145, GQ58.1 74 / 143, GM55
 // 134 / 387, GQ58.4 250 / 462, GM19 128 / 146, GM29 135 / 143.  Measured on the way
