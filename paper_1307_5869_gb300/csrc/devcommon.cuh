@@ -235,8 +235,8 @@ constexpr int kTileBytes = RowFill<uint32_t, 128>::TILE;  // per warp, 128-byte 
 // RowFill<OutT, ROWB>::TILE bytes of shared memory.
 // Rows on 16-byte boundaries are cut from their start.  Where a row of the warp is not on
 // one, every row is cut at multiples of ROWB in memory, so that every chunk but its first
-// and last leaves as whole lines in 16-byte stores (2^20 rows of 777: LFSR113 f32 813 us,
-// MRG32K3A u32 945, by each thread's own stores 3436 and 3385).  The chunks that every
+// and last leaves as whole lines in 16-byte stores (2^20 rows of 777: LFSR113 f32 742 us,
+// MRG32K3A u32 920, by each thread's own stores 3436 and 3385).  The chunks that every
 // lane has whole are a loop of their own; tests in it cost MRG32K3A 2 % of its bulk fill.
 // ROLL: keep the loop over a chunk's 16-byte pieces rolled (for generators
 // whose next() is long, where unrolling a whole chunk would outgrow the
@@ -251,21 +251,17 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
     const uint32_t phase = on_vectors ? 0u : (uint32_t)((uintptr_t)dst % ROWB) / (uint32_t)sizeof(OutT);
     OutT *const base = dst - phase;          // the row in whole chunks, from its first output's
     const uint64_t end = len ? phase + len : 0;
-    uint64_t maxend = end, minend = end;
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        maxend = max(maxend, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)maxend, d));
-        minend = min(minend, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)minend, d));
-    }
-    const uint64_t nch = (maxend + K - 1) / K;
-    const uint64_t whole0 = on_vectors ? 0 : 1, whole1 = minend / K;  // the chunks every lane has whole
+    // (a row in memory is fewer than 2^32 chunks; 64-bit lengths by shuffles took 1 to 2 % of
+    // the bulk fills)
+    const uint32_t nch = __reduce_max_sync(kFull, (uint32_t)((end + K - 1) / K));
+    const uint32_t whole0 = on_vectors ? 0 : 1, whole1 = __reduce_min_sync(kFull, (uint32_t)(end / K));  // the chunks every lane has whole
     unsigned char *myrow = tile + lane * PITCH;
     const int piece = lane % PIECES;
-    for (uint64_t ch = 0; ch < nch; ++ch) {
+    for (uint32_t ch = 0; ch < nch; ++ch) {
         if (ch >= whole0 && ch < whole1) {
             // no per-output tests, and every row segment of the tile is stored whole
             do {
-                const unsigned long long mydst = (unsigned long long)(base + ch * K);
+                const unsigned long long mydst = (unsigned long long)(base + (uint64_t)ch * K);
 #pragma unroll (ROLL ? 1 : PIECES)
                 for (int v = 0; v < PIECES; ++v) {
                     OutT vals[E];
@@ -289,8 +285,8 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
         }
         // this lane's outputs of the chunk: columns lo .. hi - 1
         const uint32_t lo = ch ? 0u : phase;
-        const uint32_t hi = end > ch * K ? (uint32_t)min((uint64_t)K, end - ch * K) : 0u;
-        const unsigned long long mydst = (unsigned long long)(base + ch * K);
+        const uint32_t hi = end > (uint64_t)ch * K ? (uint32_t)min((uint64_t)K, end - (uint64_t)ch * K) : 0u;
+        const unsigned long long mydst = (unsigned long long)(base + (uint64_t)ch * K);
         const uint32_t hi0 = __shfl_sync(kFull, hi, 0);
         if (hi0 % E == 0 && __all_sync(kFull, lo == 0 && hi == hi0)) {
             // every lane has the same whole pieces: short rows, or the end of rows
@@ -350,7 +346,7 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 //   on 16 bytes: MRG32K3A one stream of 10^6 f64 10.3 / 8.2, 65536 x 300 u32 32.7 / 30.8,
 //     x 500 f32 51 / 71; LFSR113 f32 2^20 x 16 30.8 / 22.6, 2^18 x 32 12.6 / 13.3, 65536 x
 //     320 26.7 / 32.8; one stream of 64: LFSR113 u32 8.2 / 4.2, GQ58.3 18.5 / 12.3
-//   others: MRG32K3A u32 2^20 x 47 162 / 152, x 63 180 / 212, x 777 945 / 3385, 65536 x
+//   others: MRG32K3A u32 2^20 x 47 162 / 152, x 63 180 / 212, x 777 920 / 3385, 65536 x
 //     777 88 / 187, x 301 47 / 32
 template <typename OutT>
 inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len)

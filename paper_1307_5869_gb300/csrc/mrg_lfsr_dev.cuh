@@ -222,7 +222,7 @@ __device__ __forceinline__ uint32_t lfsr_next(uint32_t &z0, uint32_t &z1, uint32
 // the current word and the next 32 bits: one funnel shift each, where a step of its own is
 // a multiply and three operations of the ALU pipe, which bounds the fill.  operator()(k)
 // is output k of a whole chunk (a multiple of sixteen outputs), operator()() any other.
-// 2^20 x 1024 f32: 879 us before, now 784 (792 with two of the other components' shifts
+// 2^20 x 1024 f32: 879 us before, with this 784 (792 with two of the other components' shifts
 // as high multiplies, as in lfsr_next, 796 with three).
 struct LfsrRun {
     uint32_t z0, z1, z2, z3, ahead;
