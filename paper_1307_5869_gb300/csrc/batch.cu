@@ -50,16 +50,11 @@ namespace {
 
 size_t esize(int dtype) { return dtype == PRAND_DTYPE_F64 ? 8 : 4; }
 
-struct SeedBases {
-    uint64_t seed = 0;
-    void *dev = nullptr;
-    size_t off[PRAND_NUM_GENERATORS] = {};
-};
-
 struct Engine {
     int device = -1;
     DevTables *T = nullptr;
-    std::vector<SeedBases> bases;  // small cache, most recent last
+    std::mutex bases_mu;
+    std::vector<BasesRef> bases;  // small cache, most recent last
     BatchTile *d_tiles = nullptr;
     size_t d_cap = 0;
     BatchTile *h_tiles = nullptr;  // pinned staging
@@ -76,7 +71,7 @@ struct Engine {
 };
 
 constexpr int kMaxDev = 64;
-Engine g_eng[kMaxDev];
+Engine *const g_eng = new Engine[kMaxDev];  // never destroyed: its device memory may outlive CUDA at exit
 std::mutex g_eng_mu;
 
 prand_status_t engine_get(Engine **out)
@@ -127,48 +122,55 @@ prand_status_t engine_get(Engine **out)
     return PRAND_OK;
 }
 
-// Base states of all eleven generators for one seed (computed on the device).
-prand_status_t engine_bases(Engine &E, uint64_t seed, cudaStream_t st, const SeedBases **out)
+// Base states of all eleven generators for one seed (computed on the device).  The
+// cache keeps the last four seeds'; what was handed out stays until its last user (a
+// plan, a server, a call under way) lets go of it.
+prand_status_t engine_bases(Engine &E, uint64_t seed, cudaStream_t st, BasesRef *out)
 {
-    for (size_t i = 0; i < E.bases.size(); ++i)
-        if (E.bases[i].seed == seed) { *out = &E.bases[i]; return PRAND_OK; }
-    SeedBases B;
-    B.seed = seed;
+    BasesRef dropped;  // freed after the lock is: cudaFree waits for the device, and so for batches that read it
+    std::lock_guard<std::mutex> lk(E.bases_mu);
+    for (const BasesRef &b : E.bases)
+        if (b->seed == seed) { *out = b; return PRAND_OK; }
+    const std::shared_ptr<SeedBases> B = std::make_shared<SeedBases>();
+    B->seed = seed;
     size_t total = 0;
     for (int g = 0; g < PRAND_NUM_GENERATORS; ++g) {
-        B.off[g] = total;
+        B->off[g] = total;
         total += (state_bytes_per_stream(g) + 255) & ~(size_t)255;
     }
-    if (!dev_alloc(&B.dev, total)) return PRAND_ERR_NOMEM;
+    if (!dev_alloc(&B->dev, total)) { B->dev = nullptr; return PRAND_ERR_NOMEM; }
     prand_status_t s = PRAND_OK;
     for (int g = 0; g < PRAND_NUM_GENERATORS && s == PRAND_OK; ++g) {
-        void *p = (char *)B.dev + B.off[g];
+        void *p = (char *)B->dev + B->off[g];
         if (g == PRAND_MT19937) s = mt_seed(seed, p, st);
         else if (is_gm(g)) { Variant V; variant_params(g, 0, &V); s = gm_seed(g, E.T, seed, V, p, st); }
         else s = mrg_lfsr_seed(g, seed, p, st);
     }
     // wait once, so later batches on any stream see the bases
     if (s == PRAND_OK && cudaStreamSynchronize(st) != cudaSuccess) s = PRAND_ERR_CUDA;
-    if (s != PRAND_OK) { cudaFree(B.dev); return s; }
+    if (s != PRAND_OK) return s;
     if (E.bases.size() >= 4) {
-        cudaStreamSynchronize(st);
-        cudaFree(E.bases.front().dev);
+        dropped = std::move(E.bases.front());
         E.bases.erase(E.bases.begin());
     }
     E.bases.push_back(B);
-    *out = &E.bases.back();
+    *out = B;
     return PRAND_OK;
 }
 
 }  // namespace
 
-prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, DevTables **T)
+SeedBases::~SeedBases()
+{
+    if (dev) cudaFree(dev);
+}
+
+prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, BasesRef *bases, DevTables **T)
 {
     Engine *E;
     prand_status_t s = engine_get(&E);
     if (s != PRAND_OK) return s;
-    const SeedBases *B;
-    if ((s = engine_bases(*E, seed, st, &B)) != PRAND_OK) return s;
+    if ((s = engine_bases(*E, seed, st, bases)) != PRAND_OK) return s;
     memset(ctx, 0, sizeof *ctx);
     ctx->mrg_tab = E->T->mrg;
     ctx->lfsr_tab = E->T->lfsr;
@@ -176,7 +178,7 @@ prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, DevTable
     if ((s = get_mt_window(E->T)) != PRAND_OK) return s;
     ctx->mt_win = E->T->mt_win;
     for (int g = 0; g < 8; ++g) ctx->gm_tab[g] = E->T->gm[g];
-    for (int g = 0; g < PRAND_NUM_GENERATORS; ++g) ctx->base[g] = (const char *)B->dev + B->off[g];
+    for (int g = 0; g < PRAND_NUM_GENERATORS; ++g) ctx->base[g] = (const char *)(*bases)->dev + (*bases)->off[g];
     if (T) *T = E->T;
     return PRAND_OK;
 }
@@ -459,6 +461,7 @@ struct prand_batch_plan_s {
     Branches br;  // the side branches while capturing
     uint32_t *d_counter = nullptr;
     BatchCtx ctx;
+    BasesRef bases;  // ctx's base states
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -471,7 +474,8 @@ prand_status_t prand_batch_run(const prand_request_t *reqs, size_t n, uint64_t s
     if (s != PRAND_OK || n == 0) return s;
     cudaStream_t st = (cudaStream_t)stream;
     BatchCtx ctx;
-    if ((s = batch_ctx(seed, st, &ctx, nullptr)) != PRAND_OK) return s;
+    BasesRef bases;
+    if ((s = batch_ctx(seed, st, &ctx, &bases, nullptr)) != PRAND_OK) return s;
     const BatchParams P = batch_params();
     std::vector<BatchTile> tiles;
     tiles.reserve(n * 2);
@@ -507,7 +511,7 @@ prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_requ
         delete p;
         return e;
     };
-    if ((s = batch_ctx(seed, 0, &p->ctx, nullptr)) != PRAND_OK) return fail(s);
+    if ((s = batch_ctx(seed, 0, &p->ctx, &p->bases, nullptr)) != PRAND_OK) return fail(s);
     const BatchParams P = batch_params();
     std::vector<BatchTile> tiles;
     for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles, 0, true);
@@ -658,8 +662,9 @@ prand_status_t prand_batch_run_per_request(const prand_request_t *reqs, size_t n
     if (s != PRAND_OK || n == 0) return s;
     cudaStream_t st = (cudaStream_t)stream;
     BatchCtx ctx;
+    BasesRef bases;
     DevTables *T;
-    if ((s = batch_ctx(seed, st, &ctx, &T)) != PRAND_OK) return s;
+    if ((s = batch_ctx(seed, st, &ctx, &bases, &T)) != PRAND_OK) return s;
     size_t maxb = 0;
     for (int g = 0; g < PRAND_NUM_GENERATORS; ++g) maxb = std::max(maxb, state_bytes_per_stream(g));
     void *scratch = nullptr;

@@ -2,6 +2,7 @@
 // resident-stream server built on it (serve.cpp).
 #pragma once
 
+#include <memory>
 #include <vector>
 
 #include "prand_internal.h"
@@ -49,7 +50,19 @@ struct BatchParams {
     uint32_t row_bytes = 128;         // its staged row size (128 or 256 bytes: 32 or 64 u32 outputs per row store)
 };
 
-prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, DevTables **T);
+// One seed's base states of all generators, in device memory.  Kernels read them by the
+// raw pointers of a BatchCtx, so whoever keeps one (a plan, a server) keeps the bases too.
+struct SeedBases {
+    uint64_t seed = 0;
+    void *dev = nullptr;
+    size_t off[PRAND_NUM_GENERATORS] = {};
+    SeedBases() = default;
+    SeedBases(const SeedBases &) = delete;
+    ~SeedBases();
+};
+using BasesRef = std::shared_ptr<const SeedBases>;
+
+prand_status_t batch_ctx(uint64_t seed, cudaStream_t st, BatchCtx *ctx, BasesRef *bases, DevTables **T);
 BatchParams batch_params();
 // tc: GM/GQ requests may go to the tensor-core kernels (from the seeded base only).
 void plan_request(const prand_request_t &r, int32_t slot, int32_t wslot, bool from_slot, const BatchParams &P,

@@ -164,6 +164,7 @@ struct prand_server_s {
     int device = -1;
     uint64_t seed = 0;
     BatchCtx ctx;
+    BasesRef bases;  // ctx's base states
     BatchParams P;
     char *out_base = nullptr;
     uint64_t out_cap = 0;
@@ -467,7 +468,7 @@ prand_status_t prand_server_create(prand_server_t *out, uint64_t seed, uint64_t 
     };
     if (cudaGetDevice(&S->device) != cudaSuccess) return fail(PRAND_ERR_CUDA);
     S->seed = seed;
-    prand_status_t s = batch_ctx(seed, 0, &S->ctx, nullptr);
+    prand_status_t s = batch_ctx(seed, 0, &S->ctx, &S->bases, nullptr);
     if (s != PRAND_OK) return fail(s);
     // The tuned launch shape of this GPU, with the server's own section
     // lengths: requests are short and latency counts, so 2048 outputs per lane
