@@ -275,7 +275,9 @@ typedef struct {
  * from a shared counter, longest first.  Each request's output equals
  * prand_init_streams(stream, 1) then prand_generate_<dtype>(length) on a handle
  * created with the same seed.  The request array may be reused as soon as the
- * call returns; the library keeps its own copy of the work list.
+ * call returns; the library keeps its own copy of the work list.  Calls from any
+ * threads and on any streams are allowed; their batches run on a device one
+ * after another (plans on different streams run beside one another).
  * Errors: PRAND_ERR_ARG, PRAND_ERR_ALIGN, PRAND_ERR_NOMEM, PRAND_ERR_CUDA. */
 prand_status_t prand_batch_run(const prand_request_t *reqs, size_t n, uint64_t seed, prand_stream_t stream);
 

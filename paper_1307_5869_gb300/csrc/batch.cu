@@ -60,13 +60,14 @@ struct Engine {
     BatchTile *h_tiles = nullptr;  // pinned staging
     size_t h_cap = 0;
     cudaEvent_t staged = nullptr;  // the last copy out of h_tiles
+    cudaEvent_t done = nullptr;    // the last batch on d_tiles, d_counter and br
     uint32_t *d_counter = nullptr;
     BatchParams params;
     int sms = 1, blocks_per_sm[kModes] = { 1, 1, 1 };  // the wide build's (the others keep their own)
     int mt_team_bps = 1;                               // MT19937 build: a team of warps per tile
     int rest_bps[kRestVariants] = { 1, 1, 1, 1 };      // the rest build's variants
     Branches br;                                  // side branches of mixed launches
-    std::mutex aux_mu;
+    std::mutex run_mu;  // one call of prand_batch_run at a time uses the buffers, the events and br
     bool ready = false;
 };
 
@@ -84,7 +85,9 @@ prand_status_t engine_get(Engine **out)
         prand_status_t s = get_tables(PRAND_MT19937, &E.T);
         if (s != PRAND_OK) return s;
         if (!dev_alloc(&E.d_counter, 64)) return PRAND_ERR_NOMEM;
-        if (cudaEventCreateWithFlags(&E.staged, cudaEventDisableTiming) != cudaSuccess) return PRAND_ERR_CUDA;
+        if (cudaEventCreateWithFlags(&E.staged, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&E.done, cudaEventDisableTiming) != cudaSuccess)
+            return PRAND_ERR_CUDA;
         E.sms = device_sm_count();
         {
             int bps = 0;
@@ -420,12 +423,13 @@ prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, u
     return PRAND_OK;
 }
 
-prand_status_t upload_tiles(const std::vector<BatchTile> &tiles, cudaStream_t st, BatchTile **d_out, uint32_t **counter)
+// The tile list into the engine's buffer, on `st` behind the last batch that reads it
+// (which may be on another stream).  The engine's run_mu is held until that batch's
+// successor is launched and recorded.
+static prand_status_t upload_tiles(Engine *E, const std::vector<BatchTile> &tiles, cudaStream_t st)
 {
-    Engine *E;
-    prand_status_t s = engine_get(&E);
-    if (s != PRAND_OK) return s;
     const size_t n = tiles.size();
+    if (cudaStreamWaitEvent(st, E->done, 0) != cudaSuccess) return PRAND_ERR_CUDA;
     if (cudaEventSynchronize(E->staged) != cudaSuccess) return PRAND_ERR_CUDA;  // staging free again
     if (n > E->h_cap) {
         if (E->h_tiles) cudaFreeHost(E->h_tiles);
@@ -433,8 +437,7 @@ prand_status_t upload_tiles(const std::vector<BatchTile> &tiles, cudaStream_t st
         if (!host_alloc(&E->h_tiles, E->h_cap * sizeof(BatchTile))) { E->h_cap = 0; E->h_tiles = nullptr; return PRAND_ERR_NOMEM; }
     }
     if (n > E->d_cap) {
-        // the previous batch may still read the old buffer: free it in stream order
-        if (E->d_tiles) { cudaStreamSynchronize(st); cudaFree(E->d_tiles); }
+        if (E->d_tiles) { cudaEventSynchronize(E->done); cudaFree(E->d_tiles); }
         E->d_cap = std::max<size_t>(n, 2 * E->d_cap);
         if (!dev_alloc(&E->d_tiles, E->d_cap * sizeof(BatchTile))) { E->d_cap = 0; E->d_tiles = nullptr; return PRAND_ERR_NOMEM; }
     }
@@ -444,8 +447,6 @@ prand_status_t upload_tiles(const std::vector<BatchTile> &tiles, cudaStream_t st
             return PRAND_ERR_CUDA;
         if (cudaEventRecord(E->staged, st) != cudaSuccess) return PRAND_ERR_CUDA;
     }
-    *d_out = E->d_tiles;
-    *counter = E->d_counter;
     return PRAND_OK;
 }
 
@@ -482,13 +483,13 @@ prand_status_t prand_batch_run(const prand_request_t *reqs, size_t n, uint64_t s
     for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles, 0, true);
     order_tiles(tiles);
     if (tiles.size() > 0xFFFFFFFFull) return PRAND_ERR_ARG;
-    BatchTile *d_tiles;
-    uint32_t *counter;
-    if ((s = upload_tiles(tiles, st, &d_tiles, &counter)) != PRAND_OK) return s;
     Engine *E;
     if ((s = engine_get(&E)) != PRAND_OK) return s;
-    std::lock_guard<std::mutex> lk(E->aux_mu);  // one user of the branches at a time
-    return launch_batch(d_tiles, batch_parts(tiles), counter, ctx, st, &E->br);
+    std::lock_guard<std::mutex> lk(E->run_mu);
+    if ((s = upload_tiles(E, tiles, st)) != PRAND_OK) return s;
+    s = launch_batch(E->d_tiles, batch_parts(tiles), E->d_counter, ctx, st, &E->br);
+    if (cudaEventRecord(E->done, st) != cudaSuccess && s == PRAND_OK) s = PRAND_ERR_CUDA;
+    return s;
 }
 
 prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_request_t *reqs, size_t n, uint64_t seed)

@@ -70,7 +70,6 @@ void plan_request(const prand_request_t &r, int32_t slot, int32_t wslot, bool fr
 // Number of tiles plan_request() makes for r (without planning it).
 uint64_t plan_tile_count(const prand_request_t &r, const BatchParams &P, uint32_t max_tiles = 0);
 size_t slot_words(int gen);  // 32-bit words per state slot
-prand_status_t upload_tiles(const std::vector<BatchTile> &tiles, cudaStream_t st, BatchTile **d_out, uint32_t **counter);
 void order_tiles(std::vector<BatchTile> &tiles);
 prand_status_t validate_requests(const prand_request_t *reqs, size_t n);
 // A tile list runs in parts, each a persistent launch of its own kernel build, in
