@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -68,58 +69,68 @@ struct Engine {
     int rest_bps[kRestVariants] = { 1, 1, 1, 1 };      // the rest build's variants
     Branches br;                                  // side branches of mixed launches
     std::mutex run_mu;  // one call of prand_batch_run at a time uses the buffers, the events and br
-    bool ready = false;
+    std::atomic<bool> ready{ false };
 };
 
 constexpr int kMaxDev = 64;
 Engine *const g_eng = new Engine[kMaxDev];  // never destroyed: its device memory may outlive CUDA at exit
 std::mutex g_eng_mu;
 
+// A device's engine: set up by the first call, under the lock, for any number of threads.
+// What a failed set-up has made is kept for the next attempt.
+prand_status_t engine_set_up(Engine &E, int dev)
+{
+    std::lock_guard<std::mutex> lk(g_eng_mu);
+    if (E.ready.load(std::memory_order_relaxed)) return PRAND_OK;
+    E.device = dev;
+    prand_status_t s = get_tables(PRAND_MT19937, &E.T);
+    if (s != PRAND_OK) return s;
+    if (!E.d_counter && !dev_alloc(&E.d_counter, 64)) { E.d_counter = nullptr; return PRAND_ERR_NOMEM; }
+    for (cudaEvent_t *e : { &E.staged, &E.done })
+        if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) { *e = nullptr; return PRAND_ERR_CUDA; }
+    E.sms = device_sm_count();
+    {
+        int bps = 0;
+        const cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, batch_kernel<kModeWide, kBatchThreads, 128>, kBatchThreads, 0);
+        E.blocks_per_sm[kModeWide] = (e == cudaSuccess && bps >= 1) ? bps : 1;
+    }
+    for (int v = 0; v < kRestVariants; ++v) E.rest_bps[v] = rest_blocks_per_sm(v);
+    {
+        int bps = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &bps, batch_kernel<kModeMt, 32 * kMtTeam, 128>, 32 * kMtTeam, 0);
+        E.mt_team_bps = (e == cudaSuccess && bps >= 1) ? bps : 1;
+    }
+    if (E.br.create() != PRAND_OK) { E.br.destroy(); return PRAND_ERR_CUDA; }
+    const char *path = getenv("PRAND_TUNE_CACHE");
+    if (path) {
+        FILE *f = fopen(path, "r");
+        if (f) {
+            unsigned a = 0, b = 0, c = 0, d = 0;
+            if (fscanf(f, "{\"seclen_mrg_lfsr\": %u, \"seclen_gm\": %u, \"block\": %u, \"row_bytes\": %u", &a, &b,
+                       &c, &d) == 4 && a && b && a % 4 == 0 && b % 4 == 0 && (c == 64 || c == 128) &&
+                (d == 128 || d == 256)) {
+                E.params.seclen_mrg_lfsr = a;
+                E.params.seclen_gm = b;
+                E.params.block = c;
+                E.params.row_bytes = d;
+            }
+            fclose(f);
+        }
+    }
+    E.ready.store(true, std::memory_order_release);
+    return PRAND_OK;
+}
+
 prand_status_t engine_get(Engine **out)
 {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return PRAND_ERR_CUDA;
     Engine &E = g_eng[dev];
-    if (!E.ready) {
-        E.device = dev;
-        prand_status_t s = get_tables(PRAND_MT19937, &E.T);
+    if (!E.ready.load(std::memory_order_acquire)) {
+        const prand_status_t s = engine_set_up(E, dev);
         if (s != PRAND_OK) return s;
-        if (!dev_alloc(&E.d_counter, 64)) return PRAND_ERR_NOMEM;
-        if (cudaEventCreateWithFlags(&E.staged, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&E.done, cudaEventDisableTiming) != cudaSuccess)
-            return PRAND_ERR_CUDA;
-        E.sms = device_sm_count();
-        {
-            int bps = 0;
-            const cudaError_t e =
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, batch_kernel<kModeWide, kBatchThreads, 128>, kBatchThreads, 0);
-            E.blocks_per_sm[kModeWide] = (e == cudaSuccess && bps >= 1) ? bps : 1;
-        }
-        for (int v = 0; v < kRestVariants; ++v) E.rest_bps[v] = rest_blocks_per_sm(v);
-        {
-            int bps = 0;
-            const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &bps, batch_kernel<kModeMt, 32 * kMtTeam, 128>, 32 * kMtTeam, 0);
-            E.mt_team_bps = (e == cudaSuccess && bps >= 1) ? bps : 1;
-        }
-        if (E.br.create() != PRAND_OK) return PRAND_ERR_CUDA;
-        const char *path = getenv("PRAND_TUNE_CACHE");
-        if (path) {
-            FILE *f = fopen(path, "r");
-            if (f) {
-                unsigned a = 0, b = 0, c = 0, d = 0;
-                if (fscanf(f, "{\"seclen_mrg_lfsr\": %u, \"seclen_gm\": %u, \"block\": %u, \"row_bytes\": %u", &a, &b,
-                           &c, &d) == 4 && a && b && a % 4 == 0 && b % 4 == 0 && (c == 64 || c == 128) &&
-                    (d == 128 || d == 256)) {
-                    E.params.seclen_mrg_lfsr = a;
-                    E.params.seclen_gm = b;
-                    E.params.block = c;
-                    E.params.row_bytes = d;
-                }
-                fclose(f);
-            }
-        }
-        E.ready = true;
     }
     *out = &E;
     return PRAND_OK;
