@@ -378,60 +378,76 @@ void Branches::destroy()
     }
 }
 
-// d_counter: [0] MT19937, [1] the rest, [2] thread-per-stream tiles.
-prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter, const BatchCtx &ctx,
-                            cudaStream_t st, const Branches *br)
+// The parts' launches, MT19937's, the thread-per-stream and the tensor-core tiles on
+// their branches' streams (st where there is none).
+static prand_status_t launch_parts(const Engine &E, const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter,
+                                   const BatchCtx &ctx, cudaStream_t st, const cudaStream_t (&on)[kBranches])
 {
-    if (cudaMemsetAsync(d_counter, 0, 3 * sizeof(uint32_t), st) != cudaSuccess) return PRAND_ERR_CUDA;
-    if (!parts.all()) return PRAND_OK;
-    const uint32_t nmt = parts.mt, nwide = parts.wide, nrest = parts.rest, ntc = parts.tc_all();
-    // a part goes to its branch when a later part runs beside it
-    const bool on_branch[kBranches] = { br && nmt && (nwide || nrest || ntc), br && nwide && (nrest || ntc), br && ntc && nrest };
+    const uint32_t nmt = parts.mt, nwide = parts.wide, nrest = parts.rest;
     prand_status_t s = PRAND_OK;
-    for (int b = 0; b < kBranches; ++b)
-        if (on_branch[b] && (cudaEventRecord(br->fork[b], st) != cudaSuccess ||
-                             cudaStreamWaitEvent(br->st[b], br->fork[b], 0) != cudaSuccess))
-            return PRAND_ERR_CUDA;
-    Engine *E;
-    if ((s = engine_get(&E)) != PRAND_OK) return s;
     if (nmt) {
-        cudaStream_t ms = on_branch[0] ? br->st[0] : st;
         // few tiles: a cluster of blocks each, while every block has an SM to itself (a
         // stream of eight jumps and 1000 outputs: 175 us, by one block 669; 19 such 199)
-        if ((uint64_t)nmt * kMtCluster <= (uint64_t)E->sms) {
-            s = mt_cluster_launch(batch_kernel<kModeMt, 32 * kMtTeam, 128, kMtCluster>, nmt * kMtCluster, 32 * kMtTeam, kMtCluster, ms,
+        if ((uint64_t)nmt * kMtCluster <= (uint64_t)E.sms) {
+            s = mt_cluster_launch(batch_kernel<kModeMt, 32 * kMtTeam, 128, kMtCluster>, nmt * kMtCluster, 32 * kMtTeam, kMtCluster, on[0],
                                   d_tiles, nmt, d_counter, ctx);
             if (s != PRAND_OK) return s;
         } else {
-            const unsigned g = batch_grid(nmt, 32, E->mt_team_bps);  // one tile per block
-            batch_kernel<kModeMt, 32 * kMtTeam, 128><<<g, 32 * kMtTeam, 0, ms>>>(d_tiles, nmt, d_counter, ctx);
+            const unsigned g = batch_grid(nmt, 32, E.mt_team_bps);  // one tile per block
+            batch_kernel<kModeMt, 32 * kMtTeam, 128><<<g, 32 * kMtTeam, 0, on[0]>>>(d_tiles, nmt, d_counter, ctx);
             if ((s = launch_check()) != PRAND_OK) return s;
         }
     }
     if (nwide) {
-        const unsigned g = batch_grid(nwide, kBatchThreads, E->blocks_per_sm[kModeWide]);
-        batch_kernel<kModeWide, kBatchThreads, 128><<<g, kBatchThreads, 0, on_branch[1] ? br->st[1] : st>>>(
-            d_tiles + nmt, nwide, d_counter + 2, ctx);
+        const unsigned g = batch_grid(nwide, kBatchThreads, E.blocks_per_sm[kModeWide]);
+        batch_kernel<kModeWide, kBatchThreads, 128><<<g, kBatchThreads, 0, on[1]>>>(d_tiles + nmt, nwide, d_counter + 2, ctx);
         if ((s = launch_check()) != PRAND_OK) return s;
     }
     const BatchTile *tc_tiles = d_tiles + nmt + nwide + nrest;
     for (int g = 0; g < 8; ++g) {
         if (!parts.tc[g]) continue;
-        s = gm_batch(PRAND_GM19 + g, E->T, tc_tiles, parts.tc[g], ctx.base[PRAND_GM19 + g], on_branch[2] ? br->st[2] : st);
+        s = gm_batch(PRAND_GM19 + g, E.T, tc_tiles, parts.tc[g], ctx.base[PRAND_GM19 + g], on[2]);
         if (s != PRAND_OK) return s;
         tc_tiles += parts.tc[g];
     }
     if (nrest) {
-        const int v = rest_variant(E->params.block, E->params.row_bytes);
-        rest_launch(v, batch_grid(nrest, rest_block(v), E->rest_bps[v]), st, d_tiles + nmt + nwide, nrest,
+        const int v = rest_variant(E.params.block, E.params.row_bytes);
+        rest_launch(v, batch_grid(nrest, rest_block(v), E.rest_bps[v]), st, d_tiles + nmt + nwide, nrest,
                     d_counter + 1, ctx);
         if ((s = launch_check()) != PRAND_OK) return s;
     }
-    for (int b = 0; b < kBranches; ++b)
-        if (on_branch[b] && (cudaEventRecord(br->join[b], br->st[b]) != cudaSuccess ||
-                             cudaStreamWaitEvent(st, br->join[b], 0) != cudaSuccess))
-            return PRAND_ERR_CUDA;
     return PRAND_OK;
+}
+
+// d_counter: [0] MT19937, [1] the rest, [2] thread-per-stream tiles.  Whatever comes of
+// it, `st` goes on only behind every branch that was forked: the caller's buffers are
+// free when its work in `st` is done.
+prand_status_t launch_batch(const BatchTile *d_tiles, const BatchParts &parts, uint32_t *d_counter, const BatchCtx &ctx,
+                            cudaStream_t st, const Branches *br)
+{
+    Engine *E;
+    prand_status_t s = engine_get(&E);
+    if (s != PRAND_OK) return s;
+    if (cudaMemsetAsync(d_counter, 0, 3 * sizeof(uint32_t), st) != cudaSuccess) return PRAND_ERR_CUDA;
+    if (!parts.all()) return PRAND_OK;
+    const uint32_t nmt = parts.mt, nwide = parts.wide, nrest = parts.rest, ntc = parts.tc_all();
+    // a part goes to its branch when a later part runs beside it
+    const bool on_branch[kBranches] = { br && nmt && (nwide || nrest || ntc), br && nwide && (nrest || ntc), br && ntc && nrest };
+    bool forked[kBranches] = {};
+    cudaStream_t on[kBranches];
+    for (int b = 0; b < kBranches; ++b) {
+        on[b] = on_branch[b] ? br->st[b] : st;
+        if (!on_branch[b] || s != PRAND_OK) continue;
+        if (cudaEventRecord(br->fork[b], st) != cudaSuccess || cudaStreamWaitEvent(br->st[b], br->fork[b], 0) != cudaSuccess)
+            s = PRAND_ERR_CUDA;
+        else forked[b] = true;
+    }
+    if (s == PRAND_OK) s = launch_parts(*E, d_tiles, parts, d_counter, ctx, st, on);
+    for (int b = 0; b < kBranches; ++b)
+        if (forked[b] && (cudaEventRecord(br->join[b], br->st[b]) != cudaSuccess ||
+                          cudaStreamWaitEvent(st, br->join[b], 0) != cudaSuccess) && s == PRAND_OK)
+            s = PRAND_ERR_CUDA;
+    return s;
 }
 
 // The tile list into the engine's buffer, on `st` behind the last batch that reads it
