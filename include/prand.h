@@ -61,11 +61,21 @@ typedef enum {
     PRAND_ERR_CUDA = 4,            /* a CUDA runtime call or kernel launch failed         */
     PRAND_ERR_STATE = 5,           /* call out of order (e.g. generate before init) or a
                                       state blob of the wrong generator/size/version      */
-    PRAND_ERR_TIMEOUT = 6,         /* a bounded device wait gave up                       */
+    PRAND_ERR_TIMEOUT = 6,         /* a bounded device wait gave up (see below)           */
     PRAND_WARN_STREAM_OVERLAP = 7  /* success, but first_stream + n_streams exceeds the
                                       Table 4 capacity of the generator, so streams may
                                       overlap within the generator's period             */
 } prand_status_t;
+
+/* PRAND_ERR_TIMEOUT: the GM/GQ kernels (all but GQ58.3's) wait for their tensor-core
+ * products with a limit of about a second, so that they always end.  A wait that
+ * reaches it means that the device does not work as it should; it does not happen in
+ * ordinary use.  The outputs of that fill or batch, and the states it left, are wrong.
+ * A call that waits for its outputs (prand_generate_host_*, prand_batch_run_per_request)
+ * returns the error itself; after an asynchronous one the next call does that fills,
+ * runs a batch or launches a plan with these generators, or that waits for such a
+ * handle's work (skip-ahead, stream initialisation, state get and set).  The error
+ * stays for the life of the process. */
 
 /* Seed value meaning "the paper's default initial state" (rng_init_, Sec. 7.1):
  * MT19937 init_genrand(5489); MRG32K3A all six words 12345; LFSR113 all four
@@ -162,7 +172,7 @@ prand_status_t prand_generate_f64(prand_handle_t h, double *dev_out, uint64_t n_
  * (after work already queued there); the call returns once every output is in
  * host_out.
  * Errors: PRAND_ERR_ARG, PRAND_ERR_ALIGN, PRAND_ERR_STATE, PRAND_ERR_NOMEM
- * (staging), PRAND_ERR_CUDA. */
+ * (staging), PRAND_ERR_CUDA, PRAND_ERR_TIMEOUT. */
 prand_status_t prand_generate_host_u32(prand_handle_t h, uint32_t *host_out, uint64_t n_per_stream, prand_stream_t stream);
 prand_status_t prand_generate_host_f32(prand_handle_t h, float *host_out, uint64_t n_per_stream, prand_stream_t stream);
 prand_status_t prand_generate_host_f64(prand_handle_t h, double *host_out, uint64_t n_per_stream, prand_stream_t stream);

@@ -490,6 +490,7 @@ struct prand_batch_plan_s {
     uint32_t *d_counter = nullptr;
     BatchCtx ctx;
     BasesRef bases;  // ctx's base states
+    DevTables *T = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -539,7 +540,7 @@ prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_requ
         delete p;
         return e;
     };
-    if ((s = batch_ctx(seed, 0, &p->ctx, &p->bases, nullptr)) != PRAND_OK) return fail(s);
+    if ((s = batch_ctx(seed, 0, &p->ctx, &p->bases, &p->T)) != PRAND_OK) return fail(s);
     const BatchParams P = batch_params();
     std::vector<BatchTile> tiles;
     for (size_t i = 0; i < n; ++i) plan_request(reqs[i], -1, -1, false, P, tiles, 0, true);
@@ -562,7 +563,8 @@ prand_status_t prand_batch_plan_create(prand_batch_plan_t *out, const prand_requ
     cudaGraph_t g = nullptr;
     cudaError_t ce = cudaStreamEndCapture(cap, &g);
     p->graph = g;
-    if (ls != PRAND_OK || ce != cudaSuccess) return fail(PRAND_ERR_CUDA);
+    if (ls != PRAND_OK) return fail(ls);
+    if (ce != cudaSuccess) return fail(PRAND_ERR_CUDA);
     if (cudaGraphInstantiate(&p->exec, p->graph, 0) != cudaSuccess) return fail(PRAND_ERR_CUDA);
     cudaStreamDestroy(cap);
     cap = nullptr;
@@ -575,6 +577,7 @@ prand_status_t prand_batch_plan_launch(prand_batch_plan_t p, prand_stream_t stre
     if (!p || !p->exec) return PRAND_ERR_ARG;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) return PRAND_ERR_STATE;
+    if (p->parts.tc_all() && *p->T->wait_failed) return PRAND_ERR_TIMEOUT;  // (the graph launches without a look)
     g_launches.fetch_add(p->parts.all() ? 1 : 0, std::memory_order_relaxed);
     return cudaGraphLaunch(p->exec, (cudaStream_t)stream) == cudaSuccess ? PRAND_OK : PRAND_ERR_CUDA;
 }
@@ -724,6 +727,8 @@ prand_status_t prand_batch_run_per_request(const prand_request_t *reqs, size_t n
     // scratch is freed in stream order (the runtime defers it until the work is done)
     cudaStreamSynchronize(st);
     if (scratch) cudaFree(scratch);
+    for (size_t i = 0; i < n && s == PRAND_OK; ++i)
+        if (is_gm(reqs[i].gen) && T->gm_tc[reqs[i].gen - PRAND_GM19] && *T->wait_failed) s = PRAND_ERR_TIMEOUT;
     return s;
 }
 

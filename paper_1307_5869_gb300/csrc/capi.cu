@@ -217,9 +217,16 @@ prand_status_t check_device(prand_handle_t h)
     return dev == h->device ? PRAND_OK : PRAND_ERR_STATE;
 }
 
+// After a wait for the handle's work: whether a kernel of the kind its generator's fills
+// use has given up a wait.
+prand_status_t waits_held(prand_handle_t h)
+{
+    return is_gm(h->gen) && h->T->gm_tc[h->gen - PRAND_GM19] && *h->T->wait_failed ? PRAND_ERR_TIMEOUT : PRAND_OK;
+}
+
 prand_status_t sync_last(prand_handle_t h)
 {
-    return cudaStreamSynchronize(h->last_stream) == cudaSuccess ? PRAND_OK : PRAND_ERR_CUDA;
+    return cudaStreamSynchronize(h->last_stream) == cudaSuccess ? waits_held(h) : PRAND_ERR_CUDA;
 }
 
 void free_states(prand_handle_t h)
@@ -336,7 +343,7 @@ prand_status_t generate_host(prand_handle_t h, void *host_out, int dtype, uint64
     if (void *mapped = mapped_host_address(host_out)) {
         s = generate_any(h, mapped, dtype, nper, stream, true);
         if (s == PRAND_OK && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) s = PRAND_ERR_CUDA;
-        return s;
+        return s == PRAND_OK ? waits_held(h) : s;
     }
     if ((s = ensure_staging(h)) != PRAND_OK) return s;
     const uint64_t n = h->n, stage = h->stage_bytes;
@@ -396,7 +403,7 @@ prand_status_t generate_host(prand_handle_t h, void *host_out, int dtype, uint64
     // the copies into host_out are complete (or abandoned) before returning
     if (cudaStreamSynchronize(h->copy_st) != cudaSuccess && s == PRAND_OK) s = PRAND_ERR_CUDA;
     h->last_stream = st;
-    return s;
+    return s == PRAND_OK ? waits_held(h) : s;
 }
 
 }  // namespace

@@ -518,8 +518,8 @@ struct TcBatch {
 // tensor cores run on from tile to tile.  The strips are transposed across the
 // lanes, so lane l ends with words 2 l and 2 l + 1 (v = 1) or words 4 i .. 4 i + 3 of
 // either half of its stream's block (v = 4), and rows leave 256 or 128 bytes at a time.
-// err: a word in host memory, set if a wait ran out (the caller's next call
-// reports it).
+// err: a word in host memory, set if a wait ran out (DevTables::wait_failed: the call
+// reports it if it waits for the outputs, else the next one does).
 template <int GEN, typename Src>
 __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, const uint64_t *__restrict__ jump, const Src &src,
                                           volatile uint32_t *err)

@@ -118,7 +118,11 @@ struct DevTables {
     uint32_t *lfsr = nullptr;     // [4][kJumpBits][32]: column images of T_c^(2^b)
     uint64_t *gm[8] = {};         // per GM/GQ generator: powers of its step, by bits and by bytes (gm_impl.cuh)
     struct GmTcTable *gm_tc[8] = {};      // the tensor-core generation's constants (null: not used by the generator)
-    volatile uint32_t *wait_failed = nullptr;  // mapped host memory: set by a kernel whose bounded wait ran out
+    // Mapped host memory: set by a tensor-core kernel whose bounded wait ran out, and never
+    // cleared (the device does not work as it should, and what such a kernel wrote, states
+    // among it, is wrong).  Every call that uses those kernels looks before it launches, and
+    // after its wait if it waits.
+    volatile uint32_t *wait_failed = nullptr;
     uint32_t *mt = nullptr;       // [kMtPolyCount][kMtPolyWords]: x^(2^b) mod phi
     uint32_t *mt_win = nullptr;   // [kMtWinPositions][kMtWinDigits][kMtPolyWords]: x^(d 2^(432 + 8 i)) mod phi
     bool ready_basic = false;

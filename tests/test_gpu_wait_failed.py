@@ -21,17 +21,23 @@ class DevTables(ctypes.Structure):  # the head of the library's per-device table
 
 
 @contextmanager
-def failed_wait():
+def wait_word():
     get = P.load()._ZN5prand10get_tablesEiPPNS_9DevTablesE
     t = ctypes.POINTER(DevTables)()
     assert get(P.GEN_ID["GM31"], ctypes.byref(t)) == 0
     word = t.contents.wait_failed
     assert word[0] == 0
-    word[0] = 1
     try:
-        yield
+        yield word
     finally:
         word[0] = 0
+
+
+@contextmanager
+def failed_wait():
+    with wait_word() as word:
+        word[0] = 1
+        yield
 
 
 def _status(fn):
@@ -66,3 +72,58 @@ def test_a_batch_that_fails_half_way_is_joined():
     P.prand_batch_run(reqs, 61, st.cuda_stream)
     torch.cuda.synchronize()
     assert torch.equal(buf, want)
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+def test_a_host_fill_reports_its_own_wait(pinned):
+    # the word is set after the fill is launched: it waits behind some 0.15 s of MT19937
+    import threading
+    import time
+
+    import torch
+    st = torch.cuda.Stream()
+    g, before = P.Generator("GM31", 5, 0, 3000), P.Generator("MT19937", 5)
+    out = torch.zeros(3000, 500, dtype=torch.int32, pin_memory=pinned)
+    fill = lambda: P.prand_generate_host_u32(g.h, out.data_ptr(), 500, st.cuda_stream)
+    fill()
+    assert np.array_equal(out.numpy().view(np.uint32), O.Streams("GM31", 5, 0, 3000).generate("u32", 500))
+    buf = torch.empty(400_000_000, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    with wait_word() as word:
+        t = threading.Thread(target=lambda: (time.sleep(0.04), word.__setitem__(0, 1)))
+        P.prand_generate_u32(before.h, buf.data_ptr(), buf.numel(), st.cuda_stream)
+        t.start()
+        assert _status(fill) == TIMEOUT
+        t.join()
+    fill()
+
+
+def test_calls_after_a_failed_wait():
+    import torch
+    buf = torch.zeros(4000, dtype=torch.int32, device="cuda")
+    reqs = [("GM61", 0, 3, 1000, buf.data_ptr()), ("MRG32K3A", 0, 3, 1000, buf.data_ptr() + 4000)]
+    other = reqs[1:] + [("GQ58_3", 0, 3, 1000, buf.data_ptr() + 8000)]
+    g, mrg = P.Generator("GM61", 5, 0, 200), P.Generator("MRG32K3A", 5, 0, 200)
+    blob = g.get_state()
+    plan, plain = P.prand_batch_plan_create(reqs, 62), P.prand_batch_plan_create(other, 62)
+    host = np.zeros((200, 300), dtype=np.uint32)
+    with failed_wait():
+        for call in (lambda: g.generate(300), lambda: P.prand_generate_host_u32(g.h, host.ctypes.data, 300, 0),
+                     lambda: P.prand_batch_run(reqs, 62), lambda: P.prand_batch_plan_create(reqs, 62),
+                     lambda: P.prand_batch_plan_launch(plan), lambda: P.prand_batch_run_per_request(reqs, 62),
+                     g.get_state, lambda: g.set_state(blob), lambda: g.skipahead(5), lambda: P.prand_init_streams(g.h, 0, 200)):
+            assert _status(call) == TIMEOUT
+        # what does not use those kernels goes on
+        mrg.generate(300)
+        P.prand_batch_run(other, 62)
+        P.prand_batch_plan_launch(plain)
+        torch.cuda.synchronize()
+    for _ in range(2):
+        buf.zero_()
+        P.prand_batch_plan_launch(plan)
+        torch.cuda.synchronize()
+        assert np.array_equal(buf[:1000].cpu().numpy().view(np.uint32), O.State.stream("GM61", 62, 3).u32(1000))
+    g.set_state(blob)
+    assert np.array_equal(g.generate(300).cpu().numpy().view(np.uint32).reshape(200, 300), O.Streams("GM61", 5, 0, 200).generate("u32", 300))
+    P.prand_batch_plan_destroy(plan)
+    P.prand_batch_plan_destroy(plain)
