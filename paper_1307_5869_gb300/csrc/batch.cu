@@ -585,11 +585,12 @@ prand_status_t prand_batch_plan_launch(prand_batch_plan_t p, prand_stream_t stre
 prand_status_t prand_batch_plan_destroy(prand_batch_plan_t p)
 {
     if (!p) return PRAND_OK;
-    cudaDeviceSynchronize();
+    // the first cudaFree waits for the device (cudaDeviceSynchronize would end a capture
+    // under way in another thread)
+    if (p->d_counter) cudaFree(p->d_counter);
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     if (p->d_tiles) cudaFree(p->d_tiles);
-    if (p->d_counter) cudaFree(p->d_counter);
     p->br.destroy();
     delete p;
     return PRAND_OK;

@@ -155,7 +155,7 @@ prand_status_t get_tables(int gen, DevTables **out)
         prand_status_t s = mrg_build_table(T.mrg, 0);
         if (s == PRAND_OK) s = lfsr_build_table(T.lfsr, 0);
         for (int g = 0; g < 8 && s == PRAND_OK; ++g) s = gm_build_table(PRAND_GM19 + g, T.gm[g], 0);
-        if (s == PRAND_OK && cudaDeviceSynchronize() != cudaSuccess) s = PRAND_ERR_CUDA;
+        if (s == PRAND_OK && cudaStreamSynchronize(0) != cudaSuccess) s = PRAND_ERR_CUDA;
         if (s != PRAND_OK) return s;
         T.ready_basic = true;
     }
@@ -235,6 +235,15 @@ void free_states(prand_handle_t h)
     if (h->d_spare) cudaFree(h->d_spare);
     h->d_state = h->d_spare = nullptr;
     h->n = 0;
+}
+
+// Wait for everything on the device, as freeing a buffer does: cudaFree waits for every
+// stream whatever the size (2 us when there is nothing to wait for), and while another
+// thread captures a graph, where cudaDeviceSynchronize would fail and end that capture.
+bool wait_device()
+{
+    void *p;
+    return dev_alloc(&p, 256) && cudaFree(p) == cudaSuccess;
 }
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t *r)
@@ -455,13 +464,8 @@ static prand_status_t init_layout(prand_handle_t h, int32_t layout, uint64_t fir
     // as many streams as the handle has: its buffers serve again, after the wait for the
     // device that freeing them would be (2^22 streams of GQ58.3, 1.6 GB: freeing and
     // allocating 1.4 ms of an opening of 1.7)
-    const bool keep = h->d_state && h->n == n_streams;
-    if (keep) {
-        if (cudaDeviceSynchronize() != cudaSuccess) { free_states(h); return PRAND_ERR_CUDA; }
-        h->n = 0;
-    } else {
-        free_states(h);
-    }
+    if (h->d_state && h->n == n_streams && wait_device()) h->n = 0;
+    else free_states(h);
     uint64_t bytes;
     if (mul_overflows(n_streams, state_bytes_per_stream(h->gen), &bytes)) return PRAND_ERR_ARG;
     if (!h->d_state && !dev_alloc(&h->d_state, bytes)) { h->d_state = nullptr; return PRAND_ERR_NOMEM; }
