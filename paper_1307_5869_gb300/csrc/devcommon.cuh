@@ -342,19 +342,22 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 // fits there.  Rows on 16-byte boundaries: staged from 96 MiB on, and below if sections
 // are own_len or longer (32 for the lighter steps; never for MRG32K3A, whose stores then
 // hide behind its steps), but not for less than a warp of sections.  Others: staged when
-// long and beyond L2.  Measured, us, staged / own:
+// long and beyond L2.  host: the rows are in host memory, where no cache puts a thread's
+// stores together on the way over the link (MRG32K3A u32 65536 x 256 366 staged, 1610 own;
+// 3 x 100000 23 / 36): staged whenever they are on 16-byte boundaries.  Measured on the
+// device, us, staged / own:
 //   on 16 bytes: MRG32K3A one stream of 10^6 f64 10.3 / 8.2, 65536 x 300 u32 32.7 / 30.8,
 //     x 500 f32 51 / 71; LFSR113 f32 2^20 x 16 30.8 / 22.6, 2^18 x 32 12.6 / 13.3, 65536 x
 //     320 26.7 / 32.8; one stream of 64: LFSR113 u32 8.2 / 4.2, GQ58.3 18.5 / 12.3
 //   others: MRG32K3A u32 2^20 x 47 162 / 152, x 63 180 / 212, x 777 920 / 3385, 65536 x
 //     777 88 / 187, x 301 47 / 32
 template <typename OutT>
-inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len)
+inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len, bool host = false)
 {
     constexpr uint64_t E = RowFill<OutT>::E;
     const uint64_t mib = n * nper / ((1ull << 20) / sizeof(OutT));
     if ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0)
-        return mib >= 96 || (seclen >= own_len && n * nsec >= 32);
+        return host || mib >= 96 || (seclen >= own_len && n * nsec >= 32);
     return nper >= 64 && mib >= 144;
 }
 

@@ -495,7 +495,7 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
     const unsigned B = 256;
     uint64_t threads = nstreams * nsec;
     uint32_t *sin = (uint32_t *)d_state + R.j0, *sout = (nsec > 1 ? (uint32_t *)d_spare : (uint32_t *)d_state) + R.j0;
-    const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, gen == PRAND_MRG32K3A ? UINT64_MAX : 32);
+    const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, gen == PRAND_MRG32K3A ? UINT64_MAX : 32, R.host);
     // section jumps as one matrix per section when there are few sections
     const bool sj = nsec > 1 && nsec <= (uint32_t)kSecJumps + 1;
     if (gen == PRAND_MRG32K3A) {

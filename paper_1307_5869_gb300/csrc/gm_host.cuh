@@ -140,7 +140,7 @@ struct GmHost {
             const uint32_t nsec = R.nsec;
             const uint64_t seclen = R.seclen, nstreams = R.count;
             uint64_t *sout = (nsec > 1 ? spare : state) + off;
-            const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, 32);
+            const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, 32, R.host);
             const unsigned grid = gm_grid_for(nstreams * nsec, B);
             if (rows) gmt_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
             else gmt_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
