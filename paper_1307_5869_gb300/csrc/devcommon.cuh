@@ -210,6 +210,15 @@ __device__ __forceinline__ void store4<double>(double *p, double a, double b, do
     reinterpret_cast<double2 *>(p)[1] = make_double2(c, d);
 }
 
+// Store four consecutive elements at p, aligned to all of them: doubles as one 32-byte
+// store, so that a sector leaves whole.
+template <typename OutT>
+__device__ __forceinline__ void store4_whole(OutT *p, OutT a, OutT b, OutT c, OutT d)
+{
+    if constexpr (sizeof(OutT) == 8) asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" :: "l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+    else store4<OutT>(p, a, b, c, d);
+}
+
 // ---------------------------------------------------------------- row staging
 // Thread-per-stream generators produce one row of outputs per lane; written
 // directly, a warp store would scatter 32 small pieces over 32 rows.  Instead

@@ -35,3 +35,13 @@ def test_rows_staged_into_host_memory(gen, dt):
         check(gen, n, per, dt)
     check(gen, 65, 33, dt)
     check(gen, 33, 64, dt, offset=1)
+
+
+@pytest.mark.parametrize("dt", ["f64", "u32"])
+@pytest.mark.parametrize("gen", ["GM55", "GQ58_4"])
+def test_rows_of_the_tensor_core_kernel_in_host_memory(gen, dt):
+    # doubles leave four to a store where rows allow it, also in a block that ends early
+    for n, per in ((5, 100), (17, 260), (33, 64), (700, 132)):
+        check(gen, n, per, dt)
+    check(gen, 17, 260, dt, offset=2)
+    check(gen, 9, 131, dt)
