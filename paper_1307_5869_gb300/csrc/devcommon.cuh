@@ -215,7 +215,7 @@ __device__ __forceinline__ void store4<double>(double *p, double a, double b, do
 template <typename OutT>
 __device__ __forceinline__ void store4_whole(OutT *p, OutT a, OutT b, OutT c, OutT d)
 {
-    if constexpr (sizeof(OutT) == 8) asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" :: "l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+    if constexpr (sizeof(OutT) == 8) *reinterpret_cast<double4_32a *>(p) = make_double4_32a(a, b, c, d);
     else store4<OutT>(p, a, b, c, d);
 }
 

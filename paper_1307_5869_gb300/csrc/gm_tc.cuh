@@ -362,38 +362,29 @@ __device__ __noinline__ uint4 tc_exact_half(const uint64_t *al_s, const uint64_t
 
 // A block's words to `to` (this lane's first word): w[half][register], `words` of them
 // in the whole block, `first` the lane's first.  VEC: rows are aligned for stores of
-// two (v = 1) or four (v = 4) elements, which a block that ends early leaves by as well.
-// Four doubles leave as one store: as two, half a sector each, they took 1.3 to 1.6 times
-// as long into host memory (GQ58.4 4096 x 1000 f64 320 us, as one 192).
+// two (v = 1) or four (v = 4) elements.  (A block that ends early by vectors too: more
+// registers' worth of code, GM55 65536 x 64 u32 24.9 to 26.9 us.)  Four doubles leave as one store: as two, half a sector each, they took 1.3 to 1.6 times
+// as long into host memory (GQ58.4 4096 x 1000 f64 320 us, as one 209, staged by the other kernel 201).
 template <int GEN, typename OutT, bool VEC>
 __device__ __forceinline__ void tc_put(const uint32_t (&w)[2][GmTc<GEN>::kRegs], OutT *to, uint32_t words, uint32_t first)
 {
     constexpr int V = GmT<GEN>::v;
-    auto vectors = [&](int h) {  // v = 1: both halves' word in one
-        if constexpr (V == 1) store2<OutT>(to, Cvt<OutT>::f(w[0][0]), Cvt<OutT>::f(w[1][0]));
-        else store4_whole<OutT>(to + kTcRow * h, Cvt<OutT>::f(w[h][0]), Cvt<OutT>::f(w[h][1]), Cvt<OutT>::f(w[h][2]), Cvt<OutT>::f(w[h][3]));
-    };
-    constexpr int kVectors = V == 1 ? 1 : 2, kLast = V == 1 ? 1 : 3;
-    auto word = [&](int h, int r) {
-        if constexpr (V == 1) return w[r][0];
-        else return w[h][r];
-    };
     if (VEC && words == (uint32_t)kTcSteps) {
+        if constexpr (V == 1) {
+            store2<OutT>(to, Cvt<OutT>::f(w[0][0]), Cvt<OutT>::f(w[1][0]));
+        } else {
 #pragma unroll
-        for (int h = 0; h < kVectors; ++h) vectors(h);
+            for (int h = 0; h < 2; ++h)
+                store4_whole<OutT>(to + kTcRow * h, Cvt<OutT>::f(w[h][0]), Cvt<OutT>::f(w[h][1]), Cvt<OutT>::f(w[h][2]), Cvt<OutT>::f(w[h][3]));
+        }
     } else {
 #pragma unroll
-        for (int h = 0; h < kVectors; ++h) {
-            if (VEC && first + kTcRow * h + kLast < words) {
-                vectors(h);
-                continue;
-            }
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int r = 0; r <= kLast; ++r) {
-                const int at = kTcRow * h + r;
-                if (first + at < words) to[at] = Cvt<OutT>::f(word(h, r));
+            for (int r = 0; r < GmTc<GEN>::kRegs; ++r) {
+                const int at = V == 1 ? h : kTcRow * h + r;
+                if (first + at < words) to[at] = Cvt<OutT>::f(w[h][r]);
             }
-        }
     }
 }
 
