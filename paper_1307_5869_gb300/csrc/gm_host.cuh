@@ -49,28 +49,55 @@ struct GmHost {
         if (*nsec == 0) *nsec = 1;
     }
     // Whether a fill goes to the tensor-core kernel (cap: its resident sections) or to
-    // this file's other one.  With streams for more than one wave, by the work of a
-    // row: the tensor-core kernel makes whole blocks of 64 outputs and spends 0.9
-    // block's time per row besides, the other one 14 outputs' time, and an output
-    // takes kRatio / 100 times as long there (2^20 streams, u32, ns per output of a
-    // stream, other / this: GM31 11.6 / 7.1, GM61 20.3 / 8.2, GM55 7.1 / 2.7, GQ58.4
-    // 3.8 / 2.3, GM29 8.0 / 7.0).  With fewer the launch and the chain of steps count:
-    // 7 us whatever the row up to 200 outputs here, 16 (GM31) to 300 ns (GM55) a step
-    // there (64 streams x 100: GM31 6.6 / 7.0, GM61 7.6 / 7.0, GQ58.4 16.4 / 6.9 us).
+    // this file's other one.  By the work of a row: the tensor-core kernel
+    // makes whole blocks of 64 outputs and spends 0.9 block's time per row besides, the
+    // other one 14 outputs' time, and an output takes r / 100 times as long there, r from
+    // both kernels over 1 to 10^6 rows of 8 to 400 outputs (us, other / this):
+    //   8 points: r falls with the bytes of an output; with fewer streams than the other
+    //     kernel has threads its time stays and this one's falls (`few`).  GM55 u32
+    //     300000 x 48, x 40, 20000 x 32: 0.87, 1.02, 0.87; f64 300000 x 96, x 80, 20000 x
+    //     40: 0.96, 1.17, 0.79; GQ58.4 f32 300000 x 128, x 100, 20000 x 48: 0.87, 1.11, 0.99
+    //     (this / other).  In one wave the chain of steps counts, 300 ns each there.
+    //   32 points: up to four waves the last, partly empty one counts and the lines are
+    //     measured ones: GM61 2500 x 36 u32 10.4 us here, 7.3 there, 2432 x 80 10.5 / 8.5,
+    //     3500 x 96 1.0, 5000 x 64 0.86; GM31 2432 x 128 9.6 / 8.5, 3500 x 112 1.0; GM29
+    //     3500 x 700 30.7 / 25.0.  Beyond: GM61 65536 x 40 0.94, x 36 1.03; GM31 12345 x
+    //     60, x 80 1.0, 1.02.
     // A fill of more than a wave into host memory is bound by the link, which takes the
     // lane-per-point kernel's rows (9728 at once, out of step) 1 to 2 % faster than this
     // one's 2432 (65536 x 1024 f32: GM61 1439 / 1459 us, GM31 1413 / 1442; stores of 4, 8
     // or 16 bytes per lane alike).
+    template <typename OutT>
     static bool use_tc(uint64_t nstreams, uint64_t nper, uint64_t cap, bool host)
     {
-        constexpr uint64_t ratio = GEN == PRAND_GM61 ? 249 : GEN == PRAND_GM55 ? 260 : GEN == PRAND_GQ58_4 ? 167
-                                 : GEN == PRAND_GM31 || GEN == PRAND_GQ58_1 ? 164 : 114;
-        constexpr uint64_t one_wave = GEN == PRAND_GM61 ? 80 : GmT<GEN>::v == 4 ? 24
-                                    : GEN == PRAND_GM31 || GEN == PRAND_GQ58_1 ? 128 : UINT64_MAX;
-        if (nstreams <= cap) return nper >= one_wave;
-        if (host && GmT<GEN>::v == 1) return false;
+        constexpr bool kF64 = std::is_same<OutT, double>::value, kF32 = std::is_same<OutT, float>::value;
+        constexpr bool kGm61 = GEN == PRAND_GM61, kGm31 = GEN == PRAND_GM31 || GEN == PRAND_GQ58_1;
+        const uint64_t row = (nper + kTcSteps - 1) / kTcSteps * kTcSteps + 56, other = nper + 14;
+        const uint64_t waves = (nstreams + cap - 1) / cap;
+        const bool nearly_full = 8 * nstreams > 7 * cap;  // (one wave)
+        if constexpr (GmT<GEN>::v == 4) {
+            if (waves == 1) return nper >= (GEN == PRAND_GQ58_4 && nearly_full ? 32 : 24);
+            if (nper > 65536) return true;
+            constexpr bool kGm55 = GEN == PRAND_GM55;
+            constexpr uint64_t few = kF64 ? 11000 : 7300;
+            // doubles: a block that ends early leaves by single ones
+            const uint64_t cost = row + (kF64 && nper % kTcSteps ? 16 : 0);
+            uint64_t r = kGm55 ? (kF64 ? 188 : kF32 ? 188 : 217) : (kF64 ? 150 : kF32 ? 146 : 162);
+            if (nper % 4 && nper > 64) r += !kF64 ? r / 8 : kGm55 ? r * 2 / 7 : 0;  // the other kernel's rows by its threads' own stores
+            return 100 * cost * nstreams < r * other * (nstreams + few);
+        }
+        if (waves == 1) {
+            if (kGm61) return nper >= 88;
+            return kGm31 && (nstreams < 8 ? nper >= 192 : nearly_full ? nper >= 256 || 100 * row < 125 * other : nper >= 120);
+        }
+        if (host) return false;
         if (nper > 65536) return true;
-        return 100 * ((nper + kTcSteps - 1) / kTcSteps * kTcSteps + 56) < ratio * (nper + 14);
+        if (kGm61) {
+            if (waves == 2) return nper >= (4 * nstreams > 5 * cap ? 88 : 80);
+            return nper >= (waves <= 4 ? 56 : 0) && 100 * row < (waves <= 4 ? 215 : waves <= 16 ? 222 : 240) * other;
+        }
+        if (kGm31) return nper >= (waves == 2 ? 112 : waves <= 4 ? 96 : 0) && 100 * row < 164 * other;
+        return waves == 2 && 4 * nstreams > 5 * cap ? nper >= 2048 : 100 * row < 109 * other;
     }
     // A batch's tiles (plan_request) from the seeded base.
     static prand_status_t batch(const uint64_t *tab, const GmTcTable *tc, volatile uint32_t *failed, const BatchTile *tiles,
@@ -94,7 +121,7 @@ struct GmHost {
         const uint64_t *sin = state + off;
         if constexpr (GmTc<GEN>::kUse) {
             const uint64_t ctas = (uint64_t)device_sm_count() * kTcCtas;
-            if (use_tc(R.count, nper, ctas * GmTc<GEN>::kStreams, R.host)) {
+            if (use_tc<OutT>(R.count, nper, ctas * GmTc<GEN>::kStreams, R.host)) {
                 if (*failed) return PRAND_ERR_TIMEOUT;
                 if (R.nsec == 0) pick(R.count, nper, ctas * GmTc<GEN>::kStreams, kTcSteps, 256, 256, &R.nsec, &R.seclen);
                 const uint32_t nsec = R.nsec;
