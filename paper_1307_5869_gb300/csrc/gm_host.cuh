@@ -15,6 +15,9 @@ inline prand_status_t gm_build_table_t(uint64_t *tab, cudaStream_t st)
 
 inline unsigned gm_grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1) / block); }
 
+// Streams from which a thread-per-stream fill takes its states through shared memory.
+constexpr uint64_t kWholeStates = 64;
+
 template <int GEN>
 struct GmHost {
     static prand_status_t seed(const uint64_t *tab, uint64_t *base, uint64_t seed, const Variant &V, cudaStream_t st)
@@ -40,7 +43,11 @@ struct GmHost {
     static void pick(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t align, uint64_t min_len, uint64_t fixed,
                      uint32_t *nsec, uint64_t *seclen)
     {
-        const uint32_t s = pick_nsec(nstreams, cap, nper / min_len, nper, fixed);
+        split(nper, pick_nsec(nstreams, cap, nper / min_len, nper, fixed), align, nsec, seclen);
+    }
+    // About s sections, on multiples of `align`.
+    static void split(uint64_t nper, uint64_t s, uint64_t align, uint32_t *nsec, uint64_t *seclen)
+    {
         uint64_t len = (nper + s - 1) / s;
         len = (len + align - 1) / align * align;
         if (len == 0) len = align;
@@ -163,14 +170,26 @@ struct GmHost {
             if (gm_blocks_per_sm<GEN>() > 6 && grid <= 3 * (unsigned)device_sm_count()) by_vec(std::integral_constant<bool, (gm_blocks_per_sm<GEN>() > 6)>{});
             else by_vec(std::false_type{});
         } else {
-            if (R.nsec == 0) pick(R.count, nper, resident_threads<200 + GEN>(gmt_gen_kernel<GEN, OutT, true>), 32, 256, 128, &R.nsec, &R.seclen);
+            const uint64_t wave = (uint64_t)B * device_sm_count();  // threads of one block per SM
+            if (R.nsec == 0) {
+                pick(R.count, nper, 3 * wave, 32, 256, 128, &R.nsec, &R.seclen);
+                // A third block on some of the SMs costs as on all: a step of a thread takes
+                // 1.37 times as long as with two (GQ58.3 2 x 11348014 f32: 88656 sections of
+                // 256 outputs 181 us, 77824 of 292 146).
+                const uint64_t units = R.count * R.nsec, s2 = 2 * wave / R.count;
+                if (units > 2 * wave && units < 3 * wave && s2 >= 1 && 100 * (nper / s2 + 128) < 137 * (R.seclen + 128))
+                    split(nper, s2, 32, &R.nsec, &R.seclen);
+            }
             const uint32_t nsec = R.nsec;
             const uint64_t seclen = R.seclen, nstreams = R.count;
             uint64_t *sout = (nsec > 1 ? spare : state) + off;
             const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, 32, R.host);
             const unsigned grid = gm_grid_for(nstreams * nsec, B);
-            if (rows) gmt_gen_kernel<GEN, OutT, true><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
-            else gmt_gen_kernel<GEN, OutT, false><<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out);
+            const bool whole = nsec == 1 && nstreams >= kWholeStates;
+            auto launch = [&](auto kernel) { kernel<<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, whole); };
+            if (rows) launch(gmt_gen_kernel<GEN, OutT, true>);
+            else if (GEN == PRAND_GQ58_3 || nper < 32) launch(gmt_gen_kernel<GEN, OutT, false>);
+            else launch(gmt_gen_kernel<GEN, OutT, false, 2>);
         }
         return launch_check();
     }

@@ -703,11 +703,15 @@ __device__ __forceinline__ void gmt_stage_out(const GmZ<GEN> *z, int rows, uint6
 // ROWS: every row start is 16-byte aligned, so rows leave through the staged
 // 128-byte row stores (every lane of a warp takes part); else one store per
 // output.  The thread of the last section writes the next state to state_out.
-template <int GEN, typename OutT, bool ROWS>
-__global__ void __launch_bounds__(256, 3) gmt_gen_kernel(const uint64_t *__restrict__ tab, const uint64_t *state_in,
+// BPS: blocks per SM, three, but two for GM55's and GQ58.4's long rows by own stores (88 to
+// 98 registers; at three, 80 with spills, GQ58.4 300000 x 90 u32 184 us, so 165).  Short
+// rows are mostly states in and out (at two, GQ58.3 424173 x 7 f64 54 us for 43), and
+// GQ58.3's own form has the rate of its points (3 x 11348014 u32 254 us at two, 214).
+template <int GEN, typename OutT, bool ROWS, int BPS = 3>
+__global__ void __launch_bounds__(256, BPS) gmt_gen_kernel(const uint64_t *__restrict__ tab, const uint64_t *state_in,
                                                       uint64_t *state_out, uint64_t nstreams, uint64_t stride,
                                                       uint64_t nper, uint32_t nsec, uint64_t seclen,
-                                                      OutT *__restrict__ out)
+                                                      OutT *__restrict__ out, bool whole)
 {
     using P = GmT<GEN>;
     using Z = GmZ<GEN>;
@@ -720,13 +724,13 @@ __global__ void __launch_bounds__(256, 3) gmt_gen_kernel(const uint64_t *__restr
     static_assert(32 * (P::s | 1) * 8 <= kTileBytes, "a warp's states fit its tile");
     const int lane = threadIdx.x & 31;
     uint64_t *const tile = reinterpret_cast<uint64_t *>(tiles[threadIdx.x >> 5]);
-    // whole streams: the warp's states are one run of memory (2^22 streams of GQ58.3, one
+    // whole (streams, each a section): the warp's states are one run of memory (2^22 streams of GQ58.3, one
     // output each: 482 us for a thread's own loads and stores, 305 through the tile, of
     // which 240 for the bytes; 2^16 streams of 4096: 1637 and 1474 us)
     const uint64_t j0 = tid - lane;
-    const int rows = nsec == 1 ? (int)min((uint64_t)32, nstreams > j0 ? nstreams - j0 : 0) : 0;
+    const int rows = whole ? (int)min((uint64_t)32, nstreams > j0 ? nstreams - j0 : 0) : 0;
     Z zc[P::s], zp[P::s];
-    if (nsec == 1) {
+    if (whole) {
         if (!rows) return;  // whole warp
         gmt_stage_in<GEN>(state_in + j0 * P::s, rows, tile, lane, zp);
         gmt_stage_in<GEN>(state_in + (stride + j0) * P::s, rows, tile, lane, zc);
@@ -744,7 +748,7 @@ __global__ void __launch_bounds__(256, 3) gmt_gen_kernel(const uint64_t *__restr
     } else {
         for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(gmt_next_word<GEN>(zc, zp));
     }
-    if (nsec == 1) {
+    if (whole) {
         __syncwarp();
         gmt_stage_out<GEN>(zp, rows, tile, lane, state_out + j0 * P::s);
         gmt_stage_out<GEN>(zc, rows, tile, lane, state_out + (stride + j0) * P::s);

@@ -34,3 +34,14 @@ def test_rows_and_waves_around_the_lines(gen):
             (121, "u32"), (128, "f64"), (191, "u32"), (256, "f32")]
     for n in (1, 8, 64, w * 7 // 8 + 1, w, w + 1, w * 5 // 4 + 1, 3 * w - 5):
         _fill(gen, n, rows if n < 3000 else rows[::3])
+
+
+@pytest.mark.parametrize("gen", ["GM55", "GQ58_3", "GQ58_4"])
+def test_states_by_threads_and_by_tiles(gen):
+    for n in (1, 31, 63, 64, 65, 100, 4097):
+        _fill(gen, n, [(1, "u32"), (7, "f64"), (17, "f32"), (22, "u32"), (33, "u32")])
+
+
+def test_a_split_stream_fills_no_part_of_a_third_block():
+    # two streams of rows off the vectors: 77824 sections on two blocks per SM
+    _fill("GQ58_3", 2, [(10_000_002, "u32"), (5, "u32"), (3_000_000, "f64")])
