@@ -41,7 +41,7 @@ __device__ __forceinline__ void batch_mrg(const BatchTile &T, const BatchCtx &C,
     uint32_t x0 = x[0], x1 = x[1], x2 = x[2], y0 = y[0], y1 = y[1], y2 = y[2];
     OutT *o = (OutT *)T.out + off;
     if (T.flags & kTileVec) {
-        fill_rows<OutT, ROWB>([&]() { return mrg_next(x0, x1, x2, y0, y1, y2); },
+        fill_rows<OutT, ROWB, false, true>([&]() { return mrg_next(x0, x1, x2, y0, y1, y2); },
                         [](uint32_t u) { return Cvt<OutT, true>::f(u); }, o, len, wsm, lane);
     } else {
         for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT, true>::f(mrg_next(x0, x1, x2, y0, y1, y2));
@@ -79,7 +79,7 @@ __device__ __forceinline__ void batch_lfsr(const BatchTile &T, const BatchCtx &C
     LfsrRun run(z[0], z[1], z[2], z[3]);
     OutT *o = (OutT *)T.out + off;
     if (T.flags & kTileVec) {
-        fill_rows<OutT, ROWB>(run, [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len,
+        fill_rows<OutT, ROWB, false, true>(run, [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len,
                         wsm, lane);
     } else {
         for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(run());
@@ -144,7 +144,7 @@ __device__ __forceinline__ void batch_gm(const BatchTile &T, const BatchCtx &C, 
         }
         OutT *o = (OutT *)T.out + off;
         if (T.flags & kTileVec) {
-            fill_rows<OutT, 128, true>([&]() { return gmt_next_word<GEN>(zc, zp); },
+            fill_rows<OutT, 128, true, true>([&]() { return gmt_next_word<GEN>(zc, zp); },
                                        [](uint32_t u) { return Cvt<OutT>::f(u); }, o, len, wsm, lane);
         } else {
             for (uint64_t i = 0; i < len; ++i) o[i] = Cvt<OutT>::f(gmt_next_word<GEN>(zc, zp));

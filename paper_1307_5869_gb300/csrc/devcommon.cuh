@@ -247,11 +247,15 @@ constexpr int kTileBytes = RowFill<uint32_t, 128>::TILE;  // per warp, 128-byte 
 // and last leaves as whole lines in 16-byte stores (2^20 rows of 777: LFSR113 f32 742 us,
 // MRG32K3A u32 920, by each thread's own stores 3436 and 3385).  The chunks that every
 // lane has whole are a loop of their own; tests in it cost MRG32K3A 2 % of its bulk fill.
+// ENDS: lanes may be idle or their rows end apart by whole chunks (a batch's request of
+// fewer than 32 sections); the chunks between two ends go through that loop too, by the lanes
+// that have them (3000 requests of 3000 LFSR113 u32 317 us without, 172).  Fills do without: it
+// costs rows of 32 to 100 outputs 4 to 6 %, and their idle lanes repeat the last section.
 // ROLL: keep the loop over a chunk's 16-byte pieces rolled (for generators
 // whose next() is long, where unrolling a whole chunk would outgrow the
 // instruction cache).  A generator may offer next(k) as well, for output k of a
 // whole chunk (k a constant, in order from 0).
-template <typename OutT, int ROWB = 128, bool ROLL = false, typename Next, typename Conv>
+template <typename OutT, int ROWB = 128, bool ROLL = false, bool ENDS = false, typename Next, typename Conv>
 __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, uint64_t len, unsigned char *tile, int lane)
 {
     using RF = RowFill<OutT, ROWB>;
@@ -263,32 +267,42 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
     // (a row in memory is fewer than 2^32 chunks; 64-bit lengths by shuffles took 1 to 2 % of
     // the bulk fills)
     const uint32_t nch = __reduce_max_sync(kFull, (uint32_t)((end + K - 1) / K));
-    const uint32_t whole0 = on_vectors ? 0 : 1, whole1 = __reduce_min_sync(kFull, (uint32_t)(end / K));  // the chunks every lane has whole
+    const uint32_t whole = (uint32_t)(end / K);  // up to where this lane's chunks are whole
+    const uint32_t whole0 = on_vectors ? 0 : 1, whole1 = ENDS ? 0u : __reduce_min_sync(kFull, whole);  // those every lane has whole
     unsigned char *myrow = tile + lane * PITCH;
     const int piece = lane % PIECES;
+    // a whole chunk's outputs of this lane into the tile
+    auto make = [&]() {
+#pragma unroll (ROLL ? 1 : PIECES)
+        for (int v = 0; v < PIECES; ++v) {
+            OutT vals[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if constexpr (std::is_invocable<Next, int>::value) vals[e] = cvt(next(v * E + e));
+                else vals[e] = cvt(next());
+            }
+            *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
+        }
+    };
+    // (by the whole warp) the tile's rows out, from their places in a chunk (mydst): `cols` outputs of those in `rows`
+    auto leave = [&](unsigned long long mydst, auto all, uint32_t rows, int cols) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < PIECES; ++i) {
+            const int r = ROWS * i + lane / PIECES;
+            OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
+            if (decltype(all)::value || (piece * E < cols && ((rows >> r) & 1u)))
+                *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
+        }
+        __syncwarp();
+    };
     for (uint32_t ch = 0; ch < nch; ++ch) {
-        if (ch >= whole0 && ch < whole1) {
+        if (!ENDS && ch >= whole0 && ch < whole1) {
             // no per-output tests, and every row segment of the tile is stored whole
             do {
                 const unsigned long long mydst = (unsigned long long)(base + (uint64_t)ch * K);
-#pragma unroll (ROLL ? 1 : PIECES)
-                for (int v = 0; v < PIECES; ++v) {
-                    OutT vals[E];
-#pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        if constexpr (std::is_invocable<Next, int>::value) vals[e] = cvt(next(v * E + e));
-                        else vals[e] = cvt(next());
-                    }
-                    *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < PIECES; ++i) {
-                    const int r = ROWS * i + lane / PIECES;
-                    OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
-                    *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
-                }
-                __syncwarp();
+                make();
+                leave(mydst, std::true_type{}, kFull, K);
             } while (++ch < whole1);
             if (ch >= nch) return;
         }
@@ -296,25 +310,34 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
         const uint32_t lo = ch ? 0u : phase;
         const uint32_t hi = end > (uint64_t)ch * K ? (uint32_t)min((uint64_t)K, end - (uint64_t)ch * K) : 0u;
         const unsigned long long mydst = (unsigned long long)(base + (uint64_t)ch * K);
-        const uint32_t hi0 = __shfl_sync(kFull, hi, 0);
-        if (hi0 % E == 0 && __all_sync(kFull, lo == 0 && hi == hi0)) {
-            // every lane has the same whole pieces: short rows, or the end of rows
+        if constexpr (ENDS) {
+            if (__all_sync(kFull, hi == 0 || (lo == 0 && hi == (uint32_t)K))) {
+                const uint32_t rows = __ballot_sync(kFull, hi != 0), stop = __reduce_min_sync(kFull, hi ? whole : nch);
+                for (;;) {
+                    if (hi) make();
+                    const unsigned long long to = (unsigned long long)(base + (uint64_t)ch * K);
+                    if (rows == kFull) leave(to, std::true_type{}, kFull, K);
+                    else leave(to, std::false_type{}, rows, K);
+                    if (ch + 1 >= stop) break;
+                    ++ch;
+                }
+                continue;
+            }
+        }
+        const uint32_t hi0 = ENDS ? __reduce_max_sync(kFull, hi) : __shfl_sync(kFull, hi, 0);
+        if (hi0 % E == 0 && __all_sync(kFull, (ENDS && hi == 0) || (lo == 0 && hi == hi0))) {
+            // every lane has the same whole pieces (or none): short rows, or the end of rows
+            const uint32_t rows = ENDS ? __ballot_sync(kFull, hi != 0) : kFull;
+            if (!ENDS || hi) {
 #pragma unroll 4
-            for (int v = 0; v < (int)(hi0 / E); ++v) {
-                OutT vals[E];
+                for (int v = 0; v < (int)(hi0 / E); ++v) {
+                    OutT vals[E];
 #pragma unroll
-                for (int e = 0; e < E; ++e) vals[e] = cvt(next());
-                *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
+                    for (int e = 0; e < E; ++e) vals[e] = cvt(next());
+                    *reinterpret_cast<uint4 *>(myrow + 16 * v) = *reinterpret_cast<const uint4 *>(vals);
+                }
             }
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < PIECES; ++i) {
-                const int r = ROWS * i + lane / PIECES;
-                OutT *rd = (OutT *)__shfl_sync(kFull, mydst, r);
-                if (piece * E < (int)hi0)
-                    *reinterpret_cast<uint4 *>(rd + piece * E) = *reinterpret_cast<const uint4 *>(tile + r * PITCH + 16 * piece);
-            }
-            __syncwarp();
+            leave(mydst, std::false_type{}, rows, (int)hi0);
             continue;
         }
         // a row's first or last chunk, or rows of several lengths: rolled (a warp comes here

@@ -681,7 +681,7 @@ __device__ __forceinline__ void gmt_stage_in(const uint64_t *from, int rows, uin
     }
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < S; ++i) z[i] = lane < rows ? (GmZ<GEN>)(tile[lane * PITCH + i] >> GmT<GEN>::t) : 0;
+    for (int i = 0; i < S; ++i) z[i] = (GmZ<GEN>)(tile[min(lane, rows - 1) * PITCH + i] >> GmT<GEN>::t);
     __syncwarp();
 }
 template <int GEN>
@@ -716,10 +716,12 @@ __global__ void __launch_bounds__(256, BPS) gmt_gen_kernel(const uint64_t *__res
     using P = GmT<GEN>;
     using Z = GmZ<GEN>;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = tid < nstreams * nsec;
-    const uint64_t j = live ? tid % nstreams : 0;
-    const uint64_t start = live ? (tid / nstreams) * seclen : 0;
-    const uint64_t len = (live && start < nper) ? min(seclen, nper - start) : 0;
+    const uint64_t units = nstreams * nsec;
+    if (tid - (threadIdx.x & 31) >= units) return;  // whole warp
+    // (ROWS: lanes past the last section make it once more, so that no lane is without)
+    const bool live = ROWS || tid < units;
+    const uint64_t unit = min(tid, units - 1), j = unit % nstreams, start = unit / nstreams * seclen;
+    const uint64_t len = live && start < nper ? min(seclen, nper - start) : 0;
     __shared__ __align__(16) unsigned char tiles[256 / 32][kTileBytes];
     static_assert(32 * (P::s | 1) * 8 <= kTileBytes, "a warp's states fit its tile");
     const int lane = threadIdx.x & 31;
@@ -731,7 +733,6 @@ __global__ void __launch_bounds__(256, BPS) gmt_gen_kernel(const uint64_t *__res
     const int rows = whole ? (int)min((uint64_t)32, nstreams > j0 ? nstreams - j0 : 0) : 0;
     Z zc[P::s], zp[P::s];
     if (whole) {
-        if (!rows) return;  // whole warp
         gmt_stage_in<GEN>(state_in + j0 * P::s, rows, tile, lane, zp);
         gmt_stage_in<GEN>(state_in + (stride + j0) * P::s, rows, tile, lane, zc);
     } else if (len) {
@@ -752,7 +753,7 @@ __global__ void __launch_bounds__(256, BPS) gmt_gen_kernel(const uint64_t *__res
         __syncwarp();
         gmt_stage_out<GEN>(zp, rows, tile, lane, state_out + j0 * P::s);
         gmt_stage_out<GEN>(zc, rows, tile, lane, state_out + (stride + j0) * P::s);
-    } else if (len && start + len == nper) {
+    } else if (tid < units && len && start + len == nper) {
         gmt_store<GEN>(zc, zp, state_out + j * P::s, state_out + (stride + j) * P::s);
     }
 }
