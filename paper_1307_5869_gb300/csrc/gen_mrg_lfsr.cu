@@ -7,6 +7,7 @@
 // GF(2) powers of the LFSR word step), exactly as the paper's array fill
 // splits an array into sections (Sec. 6).  State is stored structure-of-arrays
 // (word c of stream j at state[c * nstreams + j]) so a warp loads it coalesced.
+#include <algorithm>
 #include <array>
 #include <atomic>
 #include <cstring>
@@ -460,18 +461,13 @@ void sec_jumps(std::map<std::tuple<int, uint64_t, uint32_t>, SJ> &cache, int gen
 
 }  // namespace
 
-// Sections per stream: whole waves of the kernel's resident threads (cap),
-// sections no shorter than min_len outputs (64 for LFSR113, whose section
-// jumps beyond the 15 tabulated ones take one table entry per set bit of the
-// offset: one stream of 10^6 u32 16.4 us, by sections of 128 27.1, of 256 36.9;
-// 32 for MRG32K3A, whose take one product per byte: one stream of 10^6 doubles
-// 10.3 us staged, by sections of 64 and matrices passed with the launch 16.4) and starting on
-// multiples of 32 outputs, so the staged 128-byte row stores of every section
-// fill whole cache lines.
-static void pick_sections(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t min_len, uint32_t *nsec,
+// Sections per stream: whole waves of the kernel's resident threads (cap), at most
+// max_s, starting on multiples of 32 outputs, so the staged 128-byte row stores of every
+// section fill whole cache lines.
+static void pick_sections(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64_t max_s, uint32_t *nsec,
                           uint64_t *seclen)
 {
-    const uint32_t s = pick_nsec(nstreams, cap, nper / min_len, nper);
+    const uint32_t s = pick_nsec(nstreams, cap, max_s, nper);
     uint64_t len = (nper + s - 1) / s;
     len = (len + 31) & ~31ull;
     if (len == 0) len = 32;
@@ -480,6 +476,24 @@ static void pick_sections(uint64_t nstreams, uint64_t nper, uint64_t cap, uint64
     if (*nsec == 0) *nsec = 1;
 }
 
+// The most sections for a stream.  MRG32K3A's are reached by a product per byte of the
+// offset: sections of 32 outputs (one stream of 10^6 doubles 10.3 us staged, by sections of 64
+// and matrices passed with the launch 16.4).  LFSR113's first 16 are reached by a matrix
+// passed with the launch, further ones by a table entry per set bit of the offset, some 250
+// outputs' time (u32, us, sections of 64 / at most 16: 900 x 4097 16.7 / 12.1, 33 x 1821 14.5 / 8.5,
+// 10 x 3120 12.5 / 14.9; f64 100 x 1821 16.7 / 12.6, 100 x 3120 16.6 / 20.8): 16 while they are short,
+// else sections of 64 (1 x 10^6 16.4; of 128 20.7, of 256 22.9).  Below 8 streams the matrices
+// of a warp's lanes differ and are read one after another (1 x 777 by 13 12.7, by 5 8.5).
+// Outputs off the vectors leave a word at a time, in sections of 64 (64 x 4097 u32 17.3, by 16
+// 26.9).
+template <typename OutT>
+static uint64_t most_sections(int gen, const OutT *out, uint64_t nstreams, uint64_t nper)
+{
+    if (gen == PRAND_MRG32K3A) return nper / 32;
+    if (nstreams < 8) return nper <= 1024 ? std::min<uint64_t>(nper / 64, 5) : nper / 64;
+    if ((uintptr_t)out % (sizeof(OutT) == 8 ? 32 : 16)) return nper / 64;
+    return nper <= (nstreams < 32 || sizeof(OutT) == 8 ? 2560 : 5120) ? std::min<uint64_t>(nper / 64, kSecJumps + 1) : nper / 64;
+}
 
 template <typename OutT>
 static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state, void *d_spare, StreamRange &R,
@@ -489,7 +503,7 @@ static prand_status_t mrg_lfsr_gen_t(int gen, const DevTables *T, void *d_state,
         // size by the rows form (the other form has the same footprint or less)
         const uint64_t cap = gen == PRAND_MRG32K3A ? resident_threads<1>(mrg_gen_kernel<OutT, true>)
                                                    : resident_threads<2, kLfsrBlock>(lfsr_gen_kernel<OutT, true>);
-        pick_sections(R.count, nper, cap, gen == PRAND_MRG32K3A ? 32 : 64, &R.nsec, &R.seclen);
+        pick_sections(R.count, nper, cap, most_sections(gen, out, R.count, nper), &R.nsec, &R.seclen);
     }
     const uint32_t nsec = R.nsec;
     const uint64_t seclen = R.seclen, nstreams = R.count;
@@ -645,7 +659,7 @@ extern "C" prand_status_t prand_mrg32k3a_generate_u32_noalloc(uint32_t *dev_stat
     // the store form of prand_generate_u32 on a handle; sections of at least
     // 256 outputs, since this path builds no section matrices (that would
     // allocate host memory) and jumps by one table entry per set bit
-    pick_sections(n_streams, n_per_stream, resident_threads<1>(mrg_gen_kernel<uint32_t, true>), 256, &nsec, &seclen);
+    pick_sections(n_streams, n_per_stream, resident_threads<1>(mrg_gen_kernel<uint32_t, true>), n_per_stream / 256, &nsec, &seclen);
     int vec = ((uintptr_t)dev_out % 16) == 0;
     const bool rows = staged_rows(dev_out, n_streams, n_per_stream, nsec, seclen, UINT64_MAX);
     const unsigned B = 256;
