@@ -373,8 +373,10 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 // fill_rows or by each thread's own stores, whose lines L2 puts together while the fill
 // fits there.  Rows on 16-byte boundaries: staged from 96 MiB on, and below if sections
 // are own_len or longer (32 for the lighter steps; never for MRG32K3A, whose stores then
-// hide behind its steps), but not for less than a warp of sections.  Others: staged when
-// long and beyond L2.  host: the rows are in host memory, where no cache puts a thread's
+// hide behind its steps), but not for less than a warp of sections.  Others: staged beyond
+// L2 when long: from off_len outputs (64; 512 for the thread-per-stream ensembles, whose
+// first and last chunks, made for all lanes, are half a chunk's long steps lost each: GQ58.3
+// u32 2^20 x 98 820 us, by own stores 636; 65536 x 777, x 1821 384 and 389, 797 and 909).  host: the rows are in host memory, where no cache puts a thread's
 // stores together on the way over the link (MRG32K3A u32 65536 x 256 366 staged, 1610 own;
 // 3 x 100000 23 / 36): staged whenever they are on 16-byte boundaries.  Measured on the
 // device, us, staged / own:
@@ -384,13 +386,14 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 //   others: MRG32K3A u32 2^20 x 47 162 / 152, x 63 180 / 212, x 777 920 / 3385, 65536 x
 //     777 88 / 187, x 301 47 / 32
 template <typename OutT>
-inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len, bool host = false)
+inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nsec, uint64_t seclen, uint64_t own_len, bool host = false,
+                        uint64_t off_len = 64)
 {
     constexpr uint64_t E = RowFill<OutT>::E;
     const uint64_t mib = n * nper / ((1ull << 20) / sizeof(OutT));
     if ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0)
         return host || mib >= 96 || (seclen >= own_len && n * nsec >= 32);
-    return nper >= 64 && mib >= 144;
+    return nper >= off_len && mib >= 144;
 }
 
 // Resident threads of a kernel launched with BS-thread blocks on the current

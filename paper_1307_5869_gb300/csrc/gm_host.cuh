@@ -1,6 +1,8 @@
 // Host side of the GM/GQ ensembles: launches of the kernels of gm_impl.cuh and
 // gm_tc.cuh, instantiated one translation unit per generator.
 #pragma once
+#include <algorithm>
+
 #include "gm_tc.cuh"
 
 namespace prand {
@@ -54,6 +56,30 @@ struct GmHost {
         *seclen = len;
         *nsec = (uint32_t)((nper + len - 1) / len);
         if (*nsec == 0) *nsec = 1;
+    }
+    // Sections per stream of a thread-per-stream fill, of at least 256 outputs; wave: the
+    // threads of one block per SM.  An SM's blocks share its pipes, so a fill takes as long as
+    // the SM with the most of them, whatever is resident: blocks per SM that come out whole,
+    // and three of them where there is a choice (a step takes 1.37 times as long with three
+    // as with two, 0.6 times with one).  A section's start is worth some 30 outputs.  GQ58.3,
+    // u32, us: 86625 x 1000 by one section 608, by three 484; 2 x 11348014 (f32) by 44328 181, by
+    // 38912 146.
+    static uint64_t thread_sections(uint64_t nstreams, uint64_t nper, uint64_t wave)
+    {
+        const uint64_t max_s = std::min<uint64_t>(std::max<uint64_t>(nper / 256, 1), kMaxSections);
+        uint64_t best = 1;
+        double best_score = 0;
+        auto consider = [&](uint64_t s) {
+            if (s < 1 || s > max_s) return;
+            const uint64_t units = nstreams * s, blocks = (units + wave - 1) / wave;
+            const double shared = blocks == 1 ? 0.76 : blocks == 2 ? 0.91 : 1.0;
+            const double score = shared * (double)units / (double)(blocks * wave) / (1.0 + 32.0 * (double)s / (double)nper);
+            if (score > best_score) { best_score = score; best = s; }
+        };
+        for (uint64_t s = 1; s <= 16; ++s) consider(s);
+        for (uint64_t k = 1; k <= 6; ++k) consider(k * wave / nstreams);
+        consider(max_s);
+        return best;
     }
     // Whether a fill goes to the tensor-core kernel (cap: its resident sections) or to
     // this file's other one.  By the work of a row: the tensor-core kernel
@@ -170,25 +196,17 @@ struct GmHost {
             if (gm_blocks_per_sm<GEN>() > 6 && grid <= 3 * (unsigned)device_sm_count()) by_vec(std::integral_constant<bool, (gm_blocks_per_sm<GEN>() > 6)>{});
             else by_vec(std::false_type{});
         } else {
-            const uint64_t wave = (uint64_t)B * device_sm_count();  // threads of one block per SM
-            if (R.nsec == 0) {
-                pick(R.count, nper, 3 * wave, 32, 256, 128, &R.nsec, &R.seclen);
-                // A third block on some of the SMs costs as on all: a step of a thread takes
-                // 1.37 times as long as with two (GQ58.3 2 x 11348014 f32: 88656 sections of
-                // 256 outputs 181 us, 77824 of 292 146).
-                const uint64_t units = R.count * R.nsec, s2 = 2 * wave / R.count;
-                if (units > 2 * wave && units < 3 * wave && s2 >= 1 && 100 * (nper / s2 + 128) < 137 * (R.seclen + 128))
-                    split(nper, s2, 32, &R.nsec, &R.seclen);
-            }
+            if (R.nsec == 0) split(nper, thread_sections(R.count, nper, (uint64_t)B * device_sm_count()), 32, &R.nsec, &R.seclen);
             const uint32_t nsec = R.nsec;
             const uint64_t seclen = R.seclen, nstreams = R.count;
             uint64_t *sout = (nsec > 1 ? spare : state) + off;
-            const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, 32, R.host);
+            const bool rows = staged_rows(out, nstreams, nper, nsec, seclen, 32, R.host, 512);
             const unsigned grid = gm_grid_for(nstreams * nsec, B);
             const bool whole = nsec == 1 && nstreams >= kWholeStates;
             auto launch = [&](auto kernel) { kernel<<<grid, B, 0, st>>>(tab, sin, sout, nstreams, R.stride, nper, nsec, seclen, out, whole); };
+            // blocks per SM: two for long rows by own stores (GQ58.3's only where streams are whole)
             if (rows) launch(gmt_gen_kernel<GEN, OutT, true>);
-            else if (GEN == PRAND_GQ58_3 || nper < 32) launch(gmt_gen_kernel<GEN, OutT, false>);
+            else if (nper < 32 || (GEN == PRAND_GQ58_3 && nsec > 1)) launch(gmt_gen_kernel<GEN, OutT, false>);
             else launch(gmt_gen_kernel<GEN, OutT, false, 2>);
         }
         return launch_check();

@@ -31,3 +31,9 @@ def _fill(gen, n, calls, offset):
 def test_lfsr113_sections(n, offset):
     _fill("LFSR113", n, [(64, "u32"), (320, "f64"), (777, "u32"), (1024, "f32"), (1025, "u32"), (1821, "f64"), (2560, "f64"),
                          (2561, "u32"), (5120, "u32"), (5121, "f32")], offset)
+
+
+@pytest.mark.parametrize("n,per", [(1, 255), (1, 512), (1, 100001), (50, 30000), (2500, 513)])
+def test_gq58_3_sections(n, per):
+    _fill("GQ58_3", n, [(per, "u32"), (per, "f64")], 0)
+    _fill("GQ58_3", n, [(per, "f32")], 1)
