@@ -376,10 +376,11 @@ __device__ __forceinline__ void fill_rows(Next &&next, Conv &&cvt, OutT *dst, ui
 // hide behind its steps), but not for less than a warp of sections.  Others: staged beyond
 // L2 when long: from off_len outputs (64; 512 for the thread-per-stream ensembles, whose
 // first and last chunks, made for all lanes, are half a chunk's long steps lost each: GQ58.3
-// u32 2^20 x 98 820 us, by own stores 636; 65536 x 777, x 1821 384 and 389, 797 and 909).  host: the rows are in host memory, where no cache puts a thread's
-// stores together on the way over the link (MRG32K3A u32 65536 x 256 366 staged, 1610 own;
-// 3 x 100000 23 / 36): staged whenever they are on 16-byte boundaries.  Measured on the
-// device, us, staged / own:
+// u32 2^20 x 98 820 us, by own stores 636; 65536 x 777, x 1821 384 and 389, 797 and 909).
+// host: the rows are in host memory, where no cache puts a thread's stores together on the
+// way over the link (MRG32K3A u32 65536 x 256 366 staged, 1610 own; 3 x 100000 23 / 36): staged
+// from 192 KiB on at the latest when they are on 16-byte boundaries (MRG32K3A 63 x 80 f64 20 / 15).
+// Measured on the device, us, staged / own:
 //   on 16 bytes: MRG32K3A one stream of 10^6 f64 10.3 / 8.2, 65536 x 300 u32 32.7 / 30.8,
 //     x 500 f32 51 / 71; LFSR113 f32 2^20 x 16 30.8 / 22.6, 2^18 x 32 12.6 / 13.3, 65536 x
 //     320 26.7 / 32.8; one stream of 64: LFSR113 u32 8.2 / 4.2, GQ58.3 18.5 / 12.3
@@ -392,7 +393,7 @@ inline bool staged_rows(const OutT *out, uint64_t n, uint64_t nper, uint32_t nse
     constexpr uint64_t E = RowFill<OutT>::E;
     const uint64_t mib = n * nper / ((1ull << 20) / sizeof(OutT));
     if ((uintptr_t)out % 16 == 0 && nper % E == 0 && seclen % E == 0)
-        return host || mib >= 96 || (seclen >= own_len && n * nsec >= 32);
+        return mib >= 96 || (n * nsec >= 32 && (seclen >= own_len || (host && n * nper * sizeof(OutT) >= 192u << 10)));
     return nper >= off_len && mib >= 144;
 }
 

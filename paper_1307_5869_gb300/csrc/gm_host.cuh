@@ -154,7 +154,14 @@ struct GmHost {
         const uint64_t *sin = state + off;
         if constexpr (GmTc<GEN>::kUse) {
             const uint64_t ctas = (uint64_t)device_sm_count() * kTcCtas;
-            if (use_tc<OutT>(R.count, nper, ctas * GmTc<GEN>::kStreams, R.host)) {
+            // Into host memory the 8-point rows' single elements (outputs off its vectors of four,
+            // ends of rows) are a third of the link's rate and less; where they are many, the
+            // other kernel's staged rows (GM55 f64 68929 x 60 818 us, 236; 105 x 34250 690, 260),
+            // which take its chain of up to 256 steps, 70 us.
+            const bool single = R.host && GmT<GEN>::v == 4 && (uintptr_t)out % 16 == 0 && nper % RowFill<OutT>::E == 0 &&
+                                (nper % 4 || nper % kTcSteps > nper / 4) &&
+                                R.count * nper * sizeof(OutT) >= (16u << 10) * std::min<uint64_t>(nper, 256);
+            if (!single && use_tc<OutT>(R.count, nper, ctas * GmTc<GEN>::kStreams, R.host)) {
                 if (*failed) return PRAND_ERR_TIMEOUT;
                 if (R.nsec == 0) pick(R.count, nper, ctas * GmTc<GEN>::kStreams, kTcSteps, 256, 256, &R.nsec, &R.seclen);
                 const uint32_t nsec = R.nsec;

@@ -45,3 +45,5 @@ def test_rows_of_the_tensor_core_kernel_in_host_memory(gen, dt):
         check(gen, n, per, dt)
     check(gen, 17, 260, dt, offset=2)
     check(gen, 9, 131, dt)
+    for per in (60, 130, 1026):   # many single elements: from 4 MiB on by the other kernel
+        check(gen, 4 * 2**20 // per // (8 if dt == "f64" else 4) + 2, per, dt)
