@@ -314,12 +314,13 @@ prand_status_t prand_batch_plan_destroy(prand_batch_plan_t plan);
 /* Tile tuner (no counterpart in the paper): times the batch (as a graph
  * plan, mean of three launches) over the launch parameters and keeps the
  * fastest for later batches on this device: first the two section lengths
- * (outputs per lane of the thread-per-section tiles -- MRG32K3A, LFSR113 and
- * the thread-per-stream GM/GQ ensembles -- and outputs per warp of the
- * lane-per-point GM/GQ tiles: 2048, 8192 or 32768 each), then, at the best
+ * (outputs per lane of the thread-per-section tiles -- MRG32K3A, LFSR113 and,
+ * up to 512, GQ58.3 -- and outputs per section of the other GM/GQ generators'
+ * tensor-core tiles: 2048, 8192 or 32768 each), then, at the best
  * lengths, the threads per block (64 or 128) and the staged row size (128 or
  * 256 bytes, i.e. 32 or 64 u32 outputs per row store) of the kernel build
- * that runs MRG32K3A, LFSR113 and the lane-per-point GM/GQ tiles.  Reports the
+ * that runs MRG32K3A, LFSR113 and the lane-per-point GM/GQ tiles (requests of
+ * fewer than 96 to 192 outputs; in the request server all).  Reports the
  * choice (any output pointer may be NULL).  If the environment variable
  * PRAND_TUNE_CACHE names a file, the result is written there and read back by
  * later processes.  The requests' outputs are written (several times).

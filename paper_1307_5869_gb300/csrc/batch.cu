@@ -239,20 +239,26 @@ uint64_t plan_tile_count(const prand_request_t &r, const BatchParams &P, uint32_
 
 // Tensor-core tiles: the 4 (v = 1) or 16 (v = 4) sections of a tile are made in step by
 // one block, each from its own jump, so a tile's sections are of one length, whole
-// blocks of 64 outputs, at most kTcSection: long enough that a jump is a small part of
-// a section, short enough that the longest requests still spread over tens of blocks
-// (10^4 mixed requests, the part's five larger generators alone: 2.33 ms at 512, 2.11 at
-// 1024, 1.99 at 2048, 1.93 at 4096; 100 requests without MT19937: 0.56, 0.56, 0.59,
-// 0.58 ms).
-constexpr uint64_t kTcSection = 4096;
+// blocks of 64 outputs, at most seclen_gm (4096 before the tuner has run): long enough that
+// a jump is a small part of a section, short enough that the longest requests still
+// spread over tens of blocks (10^4 mixed requests, the part's five larger generators alone:
+// 2.33 ms at 512, 2.11 at 1024, 1.99 at 2048, 1.93 at 4096; 100 requests without MT19937:
+// 0.56, 0.56, 0.59, 0.58 ms).  Requests of a fraction of a tile's four sections stay with
+// the lane-per-point tiles, a warp each (10^4 requests of one length, u32, us, these / those:
+// GM61 10 outputs 79 / 54, 64 79 / 66, 128 79 / 79; GM31 10 56 / 44, 64 56 / 52; GM29 10 60 / 46, 160 60 / 57).
+static bool tc_request(const prand_request_t &r)
+{
+    if (!is_gm(r.gen) || r.gen == PRAND_GQ58_3) return false;
+    if (gm_params(r.gen).v != 1) return true;
+    return r.length >= (r.gen == PRAND_GM29 ? 192u : r.gen == PRAND_GM19 ? 160u : r.gen == PRAND_GM61 ? 120u : 96u);
+}
 
-bool tc_tile_gen(int gen) { return is_gm(gen) && gen != PRAND_GQ58_3; }
-
-static void plan_tc(const prand_request_t &r, std::vector<BatchTile> &out)
+static void plan_tc(const prand_request_t &r, const BatchParams &P, std::vector<BatchTile> &out)
 {
     const GmParams &G = gm_params(r.gen);
     const uint64_t n = G.s == 32 ? 4 : 16, es = esize(r.dtype);
-    const uint64_t tiles = (r.length + n * kTcSection - 1) / (n * kTcSection);
+    const uint64_t most = std::min<uint64_t>((P.seclen_gm + 63ull) & ~63ull, 1u << 20);
+    const uint64_t tiles = (r.length + n * most - 1) / (n * most);
     const uint64_t sec = ((r.length + n * tiles - 1) / (n * tiles) + 63) & ~63ull, per_tile = sec * n;
     for (uint64_t off = 0; off < r.length; off += per_tile) {
         BatchTile t = {};
@@ -271,7 +277,7 @@ void plan_request(const prand_request_t &r, int32_t slot, int32_t wslot, bool fr
     const int gen = r.gen;
     const size_t es = esize(r.dtype);
     const uintptr_t base = (uintptr_t)r.dev_out;
-    if (tc && tc_tile_gen(gen)) return plan_tc(r, out);
+    if (tc && tc_request(r)) return plan_tc(r, P, out);
     auto vec_ok = [&](uint64_t seclen) { return base % 16 == 0 && (seclen * es) % 16 == 0 && seclen % 4 == 0; };
     const uint16_t fs = from_slot ? (uint16_t)kTileFromSlot : (uint16_t)0;
     if (gen == PRAND_MT19937) {
@@ -629,7 +635,7 @@ prand_status_t prand_batch_autotune(const prand_request_t *reqs, size_t n, uint6
         if (ms < best_t) { best_t = ms; best = c; }
     };
     // coordinate search: the two section lengths (outputs per lane and per
-    // warp section), then the rest build's threads per block and staged row
+    // tensor-core section), then the rest build's threads per block and staged row
     // size (outputs per row store) at the best lengths
     const uint32_t cand[] = { 2048, 8192, 32768 };
     for (uint32_t a : cand)

@@ -45,7 +45,7 @@ struct BatchParams {
     // outputs per lane section (thread-per-section tiles), chosen by the tuner; before it
     // has run, its choice for 10^4 mixed requests (11.3 ms at 8192, 10.1 at 2048)
     uint32_t seclen_mrg_lfsr = 2048;
-    uint32_t seclen_gm = 8192;        // outputs per warp section (lane-per-point GM/GQ tiles)
+    uint32_t seclen_gm = 4096;        // outputs per section of the tensor-core tiles, and per warp of the lane-per-point ones
     uint32_t block = 64;              // threads per block of the rest-of-generators build (64 or 128)
     uint32_t row_bytes = 128;         // its staged row size (128 or 256 bytes: 32 or 64 u32 outputs per row store)
 };

@@ -26,12 +26,12 @@ def test_requests_of_few_sections(block, row_bytes):
                 skew = i % 3 == 2   # off the vectors
                 outs.append((g, d, 5 + i, n, buf, skew))
                 reqs.append((g, d, 5 + i, n, buf[skew:].data_ptr()))
-    P.prand_batch_set_params(2048, 8192, block, row_bytes)
+    P.prand_batch_set_params(2048, 4096, block, row_bytes)
     try:
         P.prand_batch_run(reqs, 91)
         torch.cuda.synchronize()
     finally:
-        P.prand_batch_set_params(2048, 8192)
+        P.prand_batch_set_params(2048, 4096)
     for g, d, k, n, buf, skew in outs:
         got = buf.cpu().numpy().view(BITS[d])
         want = getattr(O.State.stream(g, 91, k), DT[d])(n).view(BITS[d])
