@@ -47,11 +47,17 @@ STATE_BYTES = {"MT19937": 624 * 4, "MRG32K3A": 24, "LFSR113": 16, "GM19": 32 * 1
 # 7-operation step and a 32-bit strip of 5; point 11 steps without a strip);
 # MRG32K3A = its two component steps and the combination.
 OPS_PER_WORD = {"GQ58_3": 11 * 12 + 7, "MRG32K3A": 28}
-# Tensor-core operations per output word of the other GM/GQ generators: a block of 64
-# steps of 128 points is a product 128 x K x 128 (K = 16 slots for the 32-bit primes'
-# bytes, 32 for nibbles) and makes 64 words of 4 (v = 1) or 16 (v = 4) streams.
-TENSOR_FLOP_PER_WORD = {"GM19": 2048, "GM29": 2048, "GM31": 2048, "GQ58_1": 2048, "GM61": 4096, "GM55": 1024,
-                        "GQ58_4": 1024}
+# The other GM/GQ generators' fills are bound by instruction issue beside their tensor-core
+# products: warp instructions per output word (u32, f32), from ncu captures of the current
+# kernel (smsp__inst_executed.sum, 2^16 streams x 2^10 outputs; profiles/gm_tc_mt_jump_lfsr.md).
+WARP_INST_PER_WORD = {"GM19": (5.78, 5.88), "GM29": (5.89, 5.99), "GM31": (5.88, 5.97), "GM55": (2.17, 2.29),
+                      "GM61": (6.65, 6.75), "GQ58_1": (5.90, 5.99), "GQ58_4": (1.90, 2.00)}
+# Their tensor-core operations per output word, the empty slots of the operands not counted:
+# a block of 64 steps of 128 points is a product 128 x K x 128 and makes 64 words of 4
+# (v = 1) or 16 (v = 4) streams; K in use: two values of 4 byte limbs (32-bit primes) or 15
+# (GM61), 13 (GM55), 8 (GQ58.4) nibble limbs, and a bias slot each.
+TENSOR_FLOP_PER_WORD = {"GM19": 1280, "GM29": 1280, "GM31": 1280, "GQ58_1": 1280, "GM61": 4096, "GM55": 896,
+                        "GQ58_4": 576}
 # int32 lanes per SM: four schedulers, each issuing one 32-lane warp instruction per
 # cycle (the issue-slot bound of an integer kernel; the SM count and clock are
 # queried at run time)
@@ -355,10 +361,13 @@ def run_gpu(args):
         for dt, ms in (("u32", ms_u[g]), ("f32", ms_f[g])):
             key = f"{g}.{dt}"
             if g in TENSOR_FLOP_PER_WORD:
-                # (bound by the issue of what follows the products: profiles/gm_tc_mt_jump_lfsr.md)
-                rooflines[key] = {"bound": "tensor", "achieved": nS * nP * TENSOR_FLOP_PER_WORD[g] / (ms * 1e-3) / 1e12,
-                                  "peak": _tensor_peak()[0], "unit": "TFLOP/s",
-                                  "ms": ms, "gsamples_per_s": nS * nP / (ms * 1e-3) / 1e9}
+                # instruction issue, in lanes (32 per warp instruction)
+                ops = nS * nP * 32 * WARP_INST_PER_WORD[g][dt == "f32"]
+                tensor = nS * nP * TENSOR_FLOP_PER_WORD[g] / (ms * 1e-3) / 1e12
+                rooflines[key] = {"bound": "alu", "achieved": ops / (ms * 1e-3) / 1e12,
+                                  "peak": int_peak, "unit": "Tops/s",
+                                  "ms": ms, "gsamples_per_s": nS * nP / (ms * 1e-3) / 1e9,
+                                  "tensor_tflops": tensor, "tensor_frac": tensor / _tensor_peak()[0]}
             elif g.startswith("GM") or g.startswith("GQ"):
                 ops = nS * nP * OPS_PER_WORD[g]
                 rooflines[key] = {"bound": "alu", "achieved": ops / (ms * 1e-3) / 1e12,
@@ -380,8 +389,7 @@ def run_gpu(args):
     R = rooflines[dom]
     roofline = {"bound": R["bound"], "achieved": R["achieved"], "peak": R["peak"], "unit": R["unit"],
                 "frac": R["frac"], "traffic": R.get("traffic"), "kernel": dom,
-                "peak_source": int_src if R["bound"] == "alu" else f"{_tensor_peak()[1]} bf16 GEMM TFLOP/s"
-                if R["bound"] == "tensor" else f"{peak_src} HBM copy GB/s"}
+                "peak_source": int_src if R["bound"] == "alu" else f"{peak_src} HBM copy GB/s"}
     per_gen = {g: 2 * nS * nP / ((ms_u[g] + ms_f[g]) * 1e-3) / 1e9 for g in gens}
 
     # ----- end to end: same step through host buffers (device -> pinned host copies inside)
@@ -551,6 +559,9 @@ def run_table(P, torch, sp, args):
             res[dt] = {"ms": ms, "gsamples_per_s": nS * nP / (ms * 1e-3) / 1e9,
                        "hbm_frac": byts / (ms * 1e-3) / 1e9 / hbm_peak}
             if g in TENSOR_FLOP_PER_WORD:
+                tops = nS * nP * 32 * WARP_INST_PER_WORD[g][dt == "f32"] / (ms * 1e-3) / 1e12
+                res[dt]["issue_tops"] = tops
+                res[dt]["issue_frac"] = tops / int_peak
                 res[dt]["tensor_tflops"] = nS * nP * TENSOR_FLOP_PER_WORD[g] / (ms * 1e-3) / 1e12
                 res[dt]["tensor_frac"] = res[dt]["tensor_tflops"] / _tensor_peak()[0]
             if g in OPS_PER_WORD:
