@@ -135,9 +135,9 @@ prand_status_t get_tables(int gen, DevTables **out)
     DevTables &T = g_tables[dev];
     T.device = dev;
     if (!T.ready_basic) {
-        size_t mrg_b = ((size_t)kJumpBits * 18 + (size_t)kJumpBits / 8 * 256 * 20) * sizeof(uint32_t);
+        const size_t mrg_b = kMrgTabWords * sizeof(uint32_t);
         size_t lfsr_b = (size_t)4 * kJumpBits * 32 * sizeof(uint32_t);
-        size_t gm_b = (size_t)(kJumpBits + kJumpBits / 8 * 256) * 2 * sizeof(uint64_t);
+        const size_t gm_b = kGmTabWords * sizeof(uint64_t);
         if (!dev_alloc(&T.mrg, mrg_b)) return PRAND_ERR_NOMEM;
         if (!dev_alloc(&T.lfsr, lfsr_b)) return PRAND_ERR_NOMEM;
         for (int g = 0; g < 8; ++g)

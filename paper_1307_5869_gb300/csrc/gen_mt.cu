@@ -97,8 +97,9 @@ __global__ void __launch_bounds__(32 * kMtWarpsPerBlock) mt_gen_kernel(uint32_t 
 }
 
 // Few streams: a block per stream, which makes each block of words in three rounds
-// (mt_twist_emit_team) where one warp takes twenty steps: 96 streams of 1001 f32 4.1 us
-// (5.7), one of 10^6 u32 415 (1376).  With six streams or more per SM the warps fill it by
+// (mt_twist_emit_team) where one warp takes twenty steps: one stream of 10^6 u32 415 us
+// (1376); short fills are bound by their call (96 x 1001 f32 4.1 us by calls in C, 5.7, but
+// 6.6 and 6.7 from Python).  With six streams or more per SM the warps fill it by
 // themselves (10^4 outputs of 608 streams 12.3 and 18.5 us, of 1216 20.5 and 20.5, of 2432
 // 35.9 and 27.6).
 constexpr int kMtGenTeam = 8;

@@ -290,7 +290,8 @@ __device__ __forceinline__ uint32_t gm_strip_insert(GmZ<GEN> z, uint32_t w)
 }
 
 // ----------------------------------------------------------------- jumps
-// a x + b y (mod p), canonical; every operand <= p.
+// a x + b y (mod p), canonical; a and b at most p, x and y at most p + 2^18 (lazy residues:
+// the sums stay within what reduce_prod folds).
 template <int GEN>
 __device__ __forceinline__ uint64_t gm_lin(uint64_t a, uint64_t x, uint64_t b, uint64_t y)
 {

@@ -19,7 +19,7 @@
 // are the integer sum, and t = 2^20 d0 + 2^8 d1 (mod 2^32) is the fraction, its top v
 // bits the output.
 //
-// t is off by at most a margin of 36 to 314 units of 2^-24 (the rounding of W, bounded
+// t is off by at most a margin of 37 to 314 units of 2^-24 (the rounding of W, bounded
 // on the host when the tables are built); a second bias adds the margin, so a
 // fraction that close to a strip boundary shows as (t mod 1/2^v) < 2 margins.  Every
 // t is checked (one running minimum per point and half block); a point with such a
@@ -363,8 +363,9 @@ __device__ __noinline__ uint4 tc_exact_half(const uint64_t *al_s, const uint64_t
 // A block's words to `to` (this lane's first word): w[half][register], `words` of them
 // in the whole block, `first` the lane's first.  VEC: rows are aligned for stores of
 // two (v = 1) or four (v = 4) elements.  (A block that ends early by vectors too: more
-// registers' worth of code, GM55 65536 x 64 u32 24.9 to 26.9 us.)  Four doubles leave as one store: as two, half a sector each, they took 1.3 to 1.6 times
-// as long into host memory (GQ58.4 4096 x 1000 f64 320 us, as one 209, staged by the other kernel 201).
+// registers' worth of code, GM55 65536 x 64 u32 24.9 to 26.9 us.)  Four doubles leave as one
+// store: as two, half a sector each, they took 1.3 to 1.6 times as long into host memory
+// (GQ58.4 4096 x 1000 f64 320 us, as one 209, staged by the other kernel 201).
 template <int GEN, typename OutT, bool VEC>
 __device__ __forceinline__ void tc_put(const uint32_t (&w)[2][GmTc<GEN>::kRegs], OutT *to, uint32_t words, uint32_t first)
 {

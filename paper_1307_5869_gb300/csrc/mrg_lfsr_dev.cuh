@@ -51,9 +51,6 @@ __device__ __forceinline__ void mrg_apply_bit(const uint32_t *tab, int b, uint32
 
 // The same jumps by bytes of the exponent: entry (i, d) of the table's second part is the
 // pair of matrices of d 2^(8 i) steps, in five 16-byte vectors.
-constexpr int kMrgRow = 20, kMrgBytes = kJumpBits / 8;
-constexpr size_t kMrgTabWords = (size_t)kJumpBits * 18 + (size_t)kMrgBytes * 256 * kMrgRow;
-
 __host__ __device__ __forceinline__ constexpr size_t mrg_byte_row(int i, uint32_t d)
 {
     return (size_t)kJumpBits * 18 + ((size_t)i * 256 + d) * kMrgRow;

@@ -112,6 +112,12 @@ bool variant_params(int gen, int v, Variant *out);
 // ---------------------------------------------------------------------------
 // Per-device jump tables.
 // ---------------------------------------------------------------------------
+// Sizes of the jump tables: MRG32K3A's by bits (18 words) and by bytes (rows of kMrgRow
+// words), a GM/GQ generator's by bits and by bytes (two 64-bit words each).
+constexpr int kMrgRow = 20, kMrgBytes = kJumpBits / 8;
+constexpr size_t kMrgTabWords = (size_t)kJumpBits * 18 + (size_t)kMrgBytes * 256 * kMrgRow;
+constexpr size_t kGmTabWords = (size_t)(kJumpBits + kJumpBits / 8 * 256) * 2;
+
 struct DevTables {
     int device = -1;
     uint32_t *mrg = nullptr;      // [kJumpBits][18]: A^(2^b) mod m1 (9 words), B^(2^b) mod m2 (9 words)
