@@ -127,14 +127,15 @@ __device__ __forceinline__ bool tc_try(uint32_t mbar, uint32_t parity)
     return done != 0;
 }
 // Wait for the phase of `mbar`, with a limit (about a second; a wait that
-// reaches it sets *err, and later ones do not wait).  Every wait of the kernel
+// reaches it sets *err and *late, and later ones do not wait).  Every wait of the kernel
 // inside its loop is one of these, so the kernel always ends.
-__device__ __forceinline__ void tc_wait(uint32_t mbar, uint32_t parity, bool &dead, volatile uint32_t *err)
+__device__ __forceinline__ void tc_wait(uint32_t mbar, uint32_t parity, bool &dead, volatile uint32_t *err, uint32_t *late)
 {
     if (tc_try(mbar, parity) || dead) return;
     for (uint32_t i = 0; i < (1u << 20); ++i)
         if (tc_try(mbar, parity)) return;
     dead = true;
+    *late = 1u;
     *err = 1u;
 }
 
@@ -536,6 +537,7 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
     unsigned char *smA = sm + 2 * C::kImage;      // A: 16-byte columns of 128 rows
     __shared__ __align__(8) uint64_t mbar_s;      // the product is done
     __shared__ uint32_t count_s;                  // warps that have its columns
+    __shared__ uint32_t late_s;                   // a wait was given up
     __shared__ uint32_t tmem_s;
     __shared__ uint64_t al_s[kTcCoefs], be_s[kTcCoefs];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, li = tid % S;
@@ -561,6 +563,7 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         count_s = 0;
+        late_s = 0;
     }
 
     // X0 and X1 of a section from its stream's state (prev, cur) = (zm, zc)
@@ -643,7 +646,7 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
             }
         }
         uint32_t d0[32], d1[32];
-        tc_wait(mbar, parity, dead, err);
+        tc_wait(mbar, parity, dead, err, &late_s);
         parity ^= 1u;
         tc_fence_after();
         tc_ld(d0, cols);
@@ -728,6 +731,11 @@ __device__ __forceinline__ void gm_tc_run(const GmTcTable *__restrict__ tab, con
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
+        // products of waits given up may still be on their way into the tensor memory: a second
+        // more (by a word in shared memory: the threads' own state, kept to the end, cost
+        // doubles 3 % by its registers)
+        if (late_s)
+            for (int i = 0; i < 1024; ++i) __nanosleep(1000000);
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(kTcTmem) : "memory");
     }
 }
