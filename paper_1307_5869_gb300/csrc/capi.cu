@@ -183,6 +183,7 @@ struct prand_handle_s {
     void *d_base = nullptr;
     void *d_state = nullptr;
     void *d_spare = nullptr;
+    void *to_free = nullptr;  // a small buffer whose freeing waits for the device (wait_device)
     uint64_t first = 0, n = 0;
     uint64_t position = 0;
     int variant = 0;       // Table 4 variant of the streams
@@ -238,12 +239,16 @@ void free_states(prand_handle_t h)
 }
 
 // Wait for everything on the device, as freeing a buffer does: cudaFree waits for every
-// stream whatever the size (2 us when there is nothing to wait for), and while another
-// thread captures a graph, where cudaDeviceSynchronize would fail and end that capture.
-bool wait_device()
+// stream whatever the size, and while another thread captures a graph, where
+// cudaDeviceSynchronize would fail and end that capture.  A handle opened again and again
+// has its small buffer for it allocated behind the opening's launches (3 us of an opening of
+// 19 if allocated here, 1 if not).
+bool wait_device(prand_handle_t h)
 {
-    void *p;
-    return dev_alloc(&p, 256) && cudaFree(p) == cudaSuccess;
+    if (!h->to_free && !dev_alloc(&h->to_free, 256)) return false;
+    void *p = h->to_free;
+    h->to_free = nullptr;
+    return cudaFree(p) == cudaSuccess;
 }
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t *r)
@@ -464,7 +469,8 @@ static prand_status_t init_layout(prand_handle_t h, int32_t layout, uint64_t fir
     // as many streams as the handle has: its buffers serve again, after the wait for the
     // device that freeing them would be (2^22 streams of GQ58.3, 1.6 GB: freeing and
     // allocating 1.4 ms of an opening of 1.7)
-    if (h->d_state && h->n == n_streams && wait_device()) h->n = 0;
+    const bool keep = h->d_state && h->n == n_streams && wait_device(h);
+    if (keep) h->n = 0;
     else free_states(h);
     uint64_t bytes;
     if (mul_overflows(n_streams, state_bytes_per_stream(h->gen), &bytes)) return PRAND_ERR_ARG;
@@ -477,6 +483,7 @@ static prand_status_t init_layout(prand_handle_t h, int32_t layout, uint64_t fir
     if (h->gen == PRAND_MT19937) s = mt_init(h->T, h->d_base, h->d_state, first_stream, n_streams, 0, mt_shift);
     else if (is_gm(h->gen)) s = gm_init(h->gen, h->T, h->d_base, h->d_state, first_stream, n_streams, V, 0);
     else s = mrg_lfsr_init(h->gen, h->T, h->d_base, h->d_state, first_stream, n_streams, V, 0);
+    if (keep) dev_alloc(&h->to_free, 256);
     if (s == PRAND_OK && cudaStreamSynchronize(0) != cudaSuccess) s = PRAND_ERR_CUDA;
     if (s != PRAND_OK) { free_states(h); return s; }
     h->first = first_stream;
@@ -684,6 +691,7 @@ prand_status_t prand_destroy(prand_handle_t h)
     cudaStreamSynchronize(h->last_stream);
     free_states(h);
     free_staging(h);
+    if (h->to_free) cudaFree(h->to_free);
     if (h->d_base) cudaFree(h->d_base);
     if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
     delete h;
